@@ -1,9 +1,31 @@
-// Device helpers shared by the packing kernels (bit packing, block scans).
+// Device helpers shared by the kernels (exact conversions, bit packing, block scans).
 #pragma once
 
 #include "dls_internal.cuh"
 
 namespace dls {
+
+// The FP64 pipe issues about two lanes a clock and SM (an FP64 instruction,
+// a conversion from float included, holds a quarter of the SM for 64 clocks),
+// so what integers can do is done with them.
+// (double)x exactly where x is a normal float; infinities and NaNs come out
+// finite: callers screen them.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x);
+  if ((u & 0x7F800000u) == 0u) return (double)x;       // zeros and subnormals
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ bool not_finite(float x) { return (__float_as_uint(x) & 0x7F800000u) == 0x7F800000u; }
+__device__ __forceinline__ bool not_finite(double x) { return (__double2hiint(x) & 0x7FF00000) == 0x7FF00000; }
+// |x| < b for a finite b >= 0, on the bit patterns (false for a NaN x).
+__device__ __forceinline__ bool mag_below(double x, double b) {
+  return (__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) < __double_as_longlong(b);
+}
+// |x| > b for b >= 0, likewise (true for a NaN x).
+__device__ __forceinline__ bool mag_above(double x, double b) {
+  return (__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) > __double_as_longlong(b);
+}
 
 // Word w of a bit stream whose element l (value val(l), width wdt) sits at bit l*wdt.
 template <typename F>

@@ -14,7 +14,8 @@
 //   k_gb_patch    a warp per patch: alpha = Phi^T u, q = rint(alpha / delta),
 //                 the magnitude order, the bisection on the kept count, the
 //                 record into the patch's slot,
-//   scan + copy   the record offsets and the stream.
+//   scan + copy   the record offsets and the stream.  (The FP64 definitions run
+//                 where an FP32 evaluation cannot settle what they decide.)
 // The decoder rebuilds each patch from its kept modes in kept order.
 #include "dls_device.cuh"
 
@@ -26,6 +27,7 @@ constexpr int kGbHdr = 80;
 constexpr uint32_t kGbMagic = 0x47534C44u;   // "DLSG"
 constexpr int kGbWarps = 8;                  // patches in flight per CTA
 constexpr int kGbStatCtas = 512;
+constexpr int kGbTile = 1024;                // records a tile of the size scan
 
 struct GbPlan {
   int64_t dims[4];
@@ -86,7 +88,7 @@ int gb_make_plan(const dls_gb_params* p, GbPlan* g) {
 }
 
 struct GbLayout {
-  size_t Q, G, V, phi, lam, partial, status, sizes, offsets, slots, total;
+  size_t Q, G, V, phi, lam, partial, status, sizes, tiles, slots, total;
 };
 
 GbLayout gb_layout(const GbPlan& g) {
@@ -107,7 +109,7 @@ GbLayout gb_layout(const GbPlan& g) {
   L.partial = take(sizeof(double) * kGbStatCtas);
   L.status = take(sizeof(GbStatus));
   L.sizes = take(sizeof(unsigned long long) * (size_t)(g.nrec + 1));
-  L.offsets = take(sizeof(unsigned long long) * (size_t)(g.nrec + 1));
+  L.tiles = take(sizeof(unsigned long long) * (size_t)cdiv(g.nrec, kGbTile));
   L.slots = take((size_t)g.slot_bytes * (size_t)g.nrec);
   L.total = off;
   return L;
@@ -257,16 +259,32 @@ __global__ void __launch_bounds__(kJacThreads, 1) k_gb_jacobi(GbPlan g, const do
 }
 
 // ---------------------------------------------------------------- step 2: the tolerance
-// CTA c sums u^2 over a fixed contiguous range in a fixed order.
+// CTA c sums u^2 over a fixed contiguous range in a fixed order: a thread's
+// chain of FMAs is the definition, everything else stays off the FP64 pipe and
+// its next values are loaded ahead (33.5 M points: 230 us before).
 __global__ void __launch_bounds__(256) k_gb_norm(GbPlan g, const float* __restrict__ in, double* partial,
                                                  GbStatus* st) {
+  constexpr int kAhead = 16;
   const int64_t per = cdiv(g.K, kGbStatCtas);
   const int64_t i0 = (int64_t)blockIdx.x * per, i1 = (i0 + per) < g.K ? i0 + per : g.K;
   double s = 0.0;
-  int bad = 0;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += 256) {
-    const double x = (double)in[i];
-    if (!isfinite(x)) bad = 1;
+  bool bad = false;
+  int64_t i = i0 + threadIdx.x;
+  for (; i + 256 * (kAhead - 1) < i1; i += 256 * kAhead) {
+    float b[kAhead];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) b[k] = __ldg(in + i + 256 * k);
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) {
+      bad |= not_finite(b[k]);
+      const double x = widen(b[k]);
+      s = __fma_rn(x, x, s);
+    }
+  }
+  for (; i < i1; i += 256) {
+    const float b = __ldg(in + i);
+    bad |= not_finite(b);
+    const double x = widen(b);
     s = __fma_rn(x, x, s);
   }
   __shared__ double sh[256];
@@ -281,28 +299,40 @@ __global__ void __launch_bounds__(256) k_gb_norm(GbPlan g, const float* __restri
 }
 
 // eps = eps_t ||u|| / 100, eps_l^2 = eps^2 M / K, delta = eps / sqrt(K).
-__global__ void k_gb_resolve(GbPlan g, const double* partial, GbStatus* st) {
+__global__ void __launch_bounds__(128) k_gb_resolve(GbPlan g, const double* partial, GbStatus* st) {
+  __shared__ double psum[kGbStatCtas];
+  for (int c = threadIdx.x; c < kGbStatCtas; c += 128) psum[c] = partial[c];
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   double s2 = 0.0;
-  for (int c = 0; c < kGbStatCtas; ++c) s2 = __dadd_rn(s2, partial[c]);
+  for (int c = 0; c < kGbStatCtas; ++c) s2 = __dadd_rn(s2, psum[c]);
   const double eps = __ddiv_rn(__dmul_rn(g.eps_t, __dsqrt_rn(s2)), 100.0);
   st->eps_l2 = __ddiv_rn(__dmul_rn(__dmul_rn(eps, eps), (double)g.M), (double)g.K);
   st->delta = __ddiv_rn(eps, __dsqrt_rn((double)g.K));
 }
 
 // ---------------------------------------------------------------- step 3: the patches
-// Per warp in shared memory (after the basis, M x M doubles, [component][mode]).
-struct GbWarp {
-  double u[kGbMaxM];
-  double al[kGbMaxM];
-  double qd[kGbMaxM];          // q_k delta, by mode
-  long long q[kGbMaxM];
+// Per warp in shared memory, after the CTA's FP32 copy of the basis
+// ([component][mode], rows of odd length so that a warp reads a row or a column
+// of it without bank conflicts, and rows of zeros up to a multiple of 4).
+struct __align__(16) GbWarp {
+  float u[kGbMaxM];            // the patch, zeros up to a multiple of 4
+  float mag[kGbMaxM];          // |alpha| in FP32 of the listed modes
+  float qf[kGbMaxM];           // q delta in FP32, in kept order
+  double al[kGbMaxM];          // alpha by the definition, where it was needed (by list entry)
+  double qd[kGbMaxM];          // q_k delta, by mode (exact evaluations of E)
+  long long q[kGbMaxM];        // by mode
+  int list[kGbMaxM];           // the modes with q != 0, in index order
   int ord[kGbMaxM];            // modes by decreasing |alpha| (index order on ties)
+  unsigned char code[kGbMaxM + 4];      // E(s) <= eps_l^2 for s kept modes: 0 no, 1 yes, 2 open
   uint32_t words[((kGbMaxM * 70 + 31) / 32) + 4];
 };
 
-__host__ __device__ inline size_t gb_patch_smem(int M) {
-  return sizeof(double) * (size_t)M * M + sizeof(GbWarp) * kGbWarps;
+__host__ __device__ inline int gb_ld(int M) { return M | 1; }
+__host__ __device__ inline size_t gb_basis_smem(int M) {
+  return (size_t)align_up((int64_t)sizeof(float) * gb_ld(M) * (int64_t)align_up(M, 4), 16);
 }
+__host__ __device__ inline size_t gb_patch_smem(int M) { return gb_basis_smem(M) + sizeof(GbWarp) * kGbWarps; }
 
 __device__ __forceinline__ uint64_t gb_zz(long long q) { return ((uint64_t)q << 1) ^ (uint64_t)(q >> 63); }
 
@@ -324,79 +354,297 @@ __device__ __forceinline__ double gb_warp_sum(double x) {
   return x;
 }
 
-// A warp per patch, patches in (t, z, y, x) order over the grid's warps.
+// alpha of one mode by the definition: a sequential fma sum over the components.
+__device__ __forceinline__ double gb_alpha(const double* __restrict__ phi, const float* u, int M, int k) {
+  double a = 0.0;
+  for (int j = 0; j < M; ++j) a = __fma_rn(__ldg(phi + j * M + k), widen(u[j]), a);
+  return a;
+}
+__device__ __forceinline__ long long gb_quant(double a, double delta, GbStatus* st) {
+  const double y = rint(__ddiv_rn(a, delta));
+  if (!(fabs(y) < 0x1p62)) {
+    atomicOr(&st->overflow, 1u);
+    return 0;
+  }
+  return (long long)y;
+}
+
+// E of the first `kept` modes by the definition (all lanes): the modes added
+// in kept order, a multiply then an add, the squares of a lane's points in
+// order, the lanes' sums in butterfly order.
+__device__ __noinline__ double gb_error(const GbWarp& W, const double* __restrict__ phi, int M, int kept, int lane) {
+  double part = 0.0;
+  for (int i = lane; i < M; i += 32) {
+    double rec = 0.0;
+    for (int s = 0; s < kept; ++s) {
+      const int k = W.ord[s];
+      rec = __dadd_rn(rec, __dmul_rn(W.qd[k], __ldg(phi + i * M + k)));
+    }
+    const double d = __dsub_rn(widen(W.u[i]), rec);
+    part = __fma_rn(d, d, part);
+  }
+  return gb_warp_sum(part);
+}
+
+// Every mode's alpha and the full order by the definition (all lanes).
+__device__ __noinline__ void gb_order_all(GbWarp& W, const double* __restrict__ phi, int M, int lane) {
+  for (int k = lane; k < M; k += 32) W.al[k] = gb_alpha(phi, W.u, M, k);
+  __syncwarp();
+  for (int k = lane; k < M; k += 32) {
+    const unsigned long long ak = (unsigned long long)__double_as_longlong(W.al[k]) & 0x7FFFFFFFFFFFFFFFull;
+    int rank = 0;
+    for (int j = 0; j < M; ++j) {
+      const unsigned long long aj = (unsigned long long)__double_as_longlong(W.al[j]) & 0x7FFFFFFFFFFFFFFFull;
+      rank += (aj > ak || (aj == ak && j < k)) ? 1 : 0;
+    }
+    W.ord[rank] = k;
+  }
+  __syncwarp();
+}
+
+// A warp per patch, patches in (t, z, y, x) order over the grid's warps; CS =
+// ceil(M / 32) modes (and components) a lane.
+// Every stored value is the FP64 definition's, but FP64 runs only where FP32
+// cannot settle it:
+//  - alpha in FP32 is within ea = (M / 4 + 6) u ||patch|| of the definition's
+//    (four partial sums, the basis rounded once), so a quotient clear of a
+//    half-integer by ea / delta and its own rounding settles q;
+//  - modes with q = 0 change no E and come last in the order, so only the
+//    modes with q != 0 are ordered, by FP32 magnitudes where they lie 2 ea
+//    apart, else by their alphas in FP64;
+//  - E(s) for s kept modes comes from the residual r updated mode by mode.  A
+//    step's error is at most 4.2 u |q delta| ||phi|| (the roundings of q, delta,
+//    their product and phi, the fma's product being exact) plus u ||r||, so the
+//    norm of r is known to B_s = u (4.2 sum |q delta| + 1.1 sum ||r||) and pass(s) follows
+//    unless sqrt(eps_l^2) lies within B_s (and the sum's rounding) of it.
+// Patches whose scale FP32 does not carry, and n = M (no kept count passes),
+// take the definition throughout.  Measured at M = 64, 524 288 patches:
+// @GB@.
+template <int CS>
 __global__ void __launch_bounds__(kGbWarps * 32) k_gb_patch(GbPlan g, const float* __restrict__ in,
-                                                            const double* __restrict__ phi_g, const GbStatus* stc,
+                                                            const double* __restrict__ phi, const GbStatus* stc,
                                                             GbStatus* st, unsigned long long* sizes, uint8_t* slots) {
   extern __shared__ __align__(16) unsigned char gsm[];
-  const int M = g.M;
-  double* phi = reinterpret_cast<double*>(gsm);
-  GbWarp& W = reinterpret_cast<GbWarp*>(gsm + sizeof(double) * (size_t)M * M)[threadIdx.x >> 5];
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr float kU = 5.9604645e-8f;
+  const int M = g.M, ld = gb_ld(M), M4 = (int)align_up(M, 4);
+  float* ph = reinterpret_cast<float*>(gsm);
+  GbWarp& W = reinterpret_cast<GbWarp*>(gsm + gb_basis_smem(M))[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  for (int e = threadIdx.x; e < M * M; e += blockDim.x) phi[e] = phi_g[e];
+  for (int e = threadIdx.x; e < M4 * ld; e += blockDim.x) {
+    const int j = e / ld, k = e - j * ld;
+    ph[e] = j < M && k < M ? __double2float_rn(phi[j * M + k]) : 0.0f;
+  }
   __syncthreads();
   const double eps_l2 = stc->eps_l2, delta = stc->delta;
+  const bool pos = delta > 0.0, scale_ok = delta > 1e-16 && delta < 1e16;
+  const float inv = scale_ok ? __double2float_rn(1.0 / delta) : 0.0f, delta_f = scale_ok ? __double2float_rn(delta) : 0.0f;
+  const float tol = scale_ok ? __double2float_rn(sqrt(eps_l2)) : 0.0f;
   const int ib = g.ib;
+  const uint32_t npx = (uint32_t)g.npx, npxy = (uint32_t)(g.npx * g.npy);
   const int64_t pps = g.npx * g.npy * g.npz;
+  int64_t poff[CS];                          // field offset of this lane's components inside a patch
+#pragma unroll
+  for (int c = 0; c < CS; ++c) {
+    const int i = lane + 32 * c;
+    const int ix = i % g.px, iy = (i / g.px) % g.py, iz = i / (g.px * g.py);
+    poff[c] = ((int64_t)iz * g.dims[1] + iy) * g.dims[0] + ix;
+  }
   for (int64_t p = (int64_t)blockIdx.x * kGbWarps + (threadIdx.x >> 5); p < g.nrec;
        p += (int64_t)gridDim.x * kGbWarps) {
-    const int64_t t = p / pps, rem = p - t * pps;
-    const int64_t bz = rem / (g.npx * g.npy), r2 = rem - bz * g.npx * g.npy;
-    const int64_t by = r2 / g.npx, bx = r2 - by * g.npx;
-    const int64_t x0 = bx * g.px, y0 = by * g.py, z0 = bz * g.pz;
-    for (int i = lane; i < M; i += 32) {
-      const int ix = i % g.px, iy = (i / g.px) % g.py, iz = i / (g.px * g.py);
-      W.u[i] = (double)in[((t * g.dims[2] + z0 + iz) * g.dims[1] + (y0 + iy)) * g.dims[0] + (x0 + ix)];
+    int64_t x0, y0, z0, t;
+    if (g.nrec <= 0x7fffffff) {
+      const uint32_t pp = (uint32_t)p, t32 = pp / (uint32_t)pps, rem = pp - t32 * (uint32_t)pps;
+      const uint32_t bz = rem / npxy, r2 = rem - bz * npxy, by = r2 / npx;
+      t = t32;
+      x0 = (int64_t)(r2 - by * npx) * g.px;
+      y0 = (int64_t)by * g.py;
+      z0 = (int64_t)bz * g.pz;
+    } else {
+      t = p / pps;
+      const int64_t rem = p - t * pps;
+      const int64_t bz = rem / (g.npx * g.npy), r2 = rem - bz * g.npx * g.npy, by = r2 / g.npx;
+      x0 = (r2 - by * g.npx) * g.px;
+      y0 = by * g.py;
+      z0 = bz * g.pz;
+    }
+    const float* src = in + ((t * g.dims[2] + z0) * g.dims[1] + y0) * g.dims[0] + x0;
+    float u[CS], n2 = 0.0f, amax = 0.0f;
+#pragma unroll
+    for (int c = 0; c < CS; ++c) {
+      const int i = lane + 32 * c;
+      u[c] = i < M ? __ldg(src + poff[c]) : 0.0f;
+      n2 = __fmaf_rn(u[c], u[c], n2);
+      amax = fmaxf(amax, fabsf(u[c]));
+      W.u[i] = u[c];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      n2 = __fadd_rn(n2, __shfl_xor_sync(FULL, n2, o));
+      amax = fmaxf(amax, __shfl_xor_sync(FULL, amax, o));
     }
     __syncwarp();
-    // alpha = Phi^T u (each a sequential fma sum over the components), q
-    for (int k = lane; k < M; k += 32) {
-      double a = 0.0;
-      for (int j = 0; j < M; ++j) a = __fma_rn(phi[j * M + k], W.u[j], a);
-      W.al[k] = a;
+    const bool f32 = scale_ok && n2 < 1.0e30f && (n2 > 1.0e-30f || amax == 0.0f);
+    // alpha (FP32), q
+    const float ea = __fmul_rn((float)(M / 4 + 7) * 1.05f * kU, sqrtf(n2));
+    float al[CS];
+    if (f32) {
+      float s0[CS], s1[CS];
+#pragma unroll
+      for (int c = 0; c < CS; ++c) { s0[c] = 0.0f; s1[c] = 0.0f; }
+      int kc[CS];
+#pragma unroll
+      for (int c = 0; c < CS; ++c) kc[c] = lane + 32 * c < M ? lane + 32 * c : 0;
+      float t0[CS], t1[CS];
+#pragma unroll
+      for (int c = 0; c < CS; ++c) { t0[c] = 0.0f; t1[c] = 0.0f; }
+      for (int j = 0; j < M4; j += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(&W.u[j]);
+        const float* r0 = ph + j * ld;
+#pragma unroll
+        for (int c = 0; c < CS; ++c) {
+          s0[c] = __fmaf_rn(r0[kc[c]], v.x, s0[c]);
+          s1[c] = __fmaf_rn(r0[ld + kc[c]], v.y, s1[c]);
+          t0[c] = __fmaf_rn(r0[2 * ld + kc[c]], v.z, t0[c]);
+          t1[c] = __fmaf_rn(r0[3 * ld + kc[c]], v.w, t1[c]);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < CS; ++c) al[c] = __fadd_rn(__fadd_rn(s0[c], s1[c]), __fadd_rn(t0[c], t1[c]));
+    }
+    const float mq = __fmul_rn(ea, __fmul_rn(inv, 1.001f));
+    int nz = 0;
+#pragma unroll
+    for (int c = 0; c < CS; ++c) {
+      const int k = lane + 32 * c;
       long long q = 0;
-      if (delta > 0.0) {
-        const double y = rint(__ddiv_rn(a, delta));
-        if (!(fabs(y) < 0x1p62)) atomicOr(&st->overflow, 1u);
-        else q = (long long)y;
+      float mag = 0.0f;
+      bool open = k < M && pos;
+      if (f32 && open) {
+        const float y = __fmul_rn(al[c], inv), ry = rintf(y);
+        open = !(fabsf(__fsub_rn(y, ry)) < 0.5f - __fadd_rn(mq, __fmaf_rn(fabsf(y), 4.0e-7f, 1.0e-30f)) &&
+                 fabsf(y) < 4.0e6f);
+        q = (long long)(int)ry;
+        mag = fabsf(al[c]);
       }
-      W.q[k] = q;
-      W.qd[k] = __dmul_rn((double)q, delta);
+      if (open) q = gb_quant(gb_alpha(phi, W.u, M, k), delta, st);
+      if (k < M) W.q[k] = q;
+      const unsigned m = __ballot_sync(FULL, q != 0);
+      if (q != 0) {
+        const int at = nz + __popc(m & ((1u << lane) - 1u));
+        W.list[at] = k;
+        W.mag[at] = mag;
+      }
+      nz += __popc(m);
     }
     __syncwarp();
-    // ranks by |alpha| (descending, index order on ties) on the magnitudes'
-    // bit patterns: for non-negative doubles their order is the integers'
-    // order, and the comparisons leave the FP64 pipe to the arithmetic
-    for (int k = lane; k < M; k += 32) {
-      const unsigned long long ak = (unsigned long long)__double_as_longlong(W.al[k]) & 0x7FFFFFFFFFFFFFFFull;
-      int rank = 0;
-      for (int j = 0; j < M; ++j) {
-        const unsigned long long aj = (unsigned long long)__double_as_longlong(W.al[j]) & 0x7FFFFFFFFFFFFFFFull;
-        rank += (aj > ak || (aj == ak && j < k)) ? 1 : 0;
+    // the order of the modes with q != 0
+    if (f32) {
+      const float sep = __fmul_rn(2.0f, ea);
+      unsigned near = 0;                     // entries lane + 32 c with a magnitude within 2 ea of another
+#pragma unroll
+      for (int c = 0; c < CS; ++c) {
+        const int e = lane + 32 * c;
+        int rank = 0;
+        bool amb = false;
+        if (e < nz) {
+          const float a = W.mag[e];
+          for (int j = 0; j < nz; ++j) {
+            const float b = W.mag[j];
+            rank += b > a ? 1 : 0;
+            amb |= j != e && !(fabsf(__fsub_rn(b, a)) > sep);
+          }
+          W.ord[rank] = W.list[e];           // (entries of open pairs are placed again below)
+        }
+        if (amb) near |= 1u << c;
       }
-      W.ord[rank] = k;
+      if (__any_sync(FULL, near != 0)) {
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < CS; ++c)
+          if ((near >> c) & 1u) W.al[lane + 32 * c] = gb_alpha(phi, W.u, M, W.list[lane + 32 * c]);
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < CS; ++c) {
+          const int e = lane + 32 * c;
+          if ((near >> c) & 1u) {
+            const float a = W.mag[e];
+            const unsigned long long ak = (unsigned long long)__double_as_longlong(W.al[e]) & 0x7FFFFFFFFFFFFFFFull;
+            int rank = 0;
+            for (int j = 0; j < nz; ++j) {
+              if (j == e) continue;
+              const float b = W.mag[j];
+              if (fabsf(__fsub_rn(b, a)) > sep) {
+                rank += b > a ? 1 : 0;
+              } else {
+                const unsigned long long aj =
+                    (unsigned long long)__double_as_longlong(W.al[j]) & 0x7FFFFFFFFFFFFFFFull;
+                rank += (aj > ak || (aj == ak && W.list[j] < W.list[e])) ? 1 : 0;
+              }
+            }
+            W.ord[rank] = W.list[e];
+          }
+        }
+      }
+      __syncwarp();
+      for (int s = lane; s < nz; s += 32) W.qf[s] = __fmul_rn(__ll2float_rn(W.q[W.ord[s]]), delta_f);
+    } else {
+      gb_order_all(W, phi, M, lane);
     }
     __syncwarp();
     // the smallest kept count by bisection over [0, M]
     int n = 0;
-    if (delta > 0.0) {
+    if (pos) {
+      const int top = f32 ? nz : M;          // E(s) = E(top) for s > top
+      if (f32) {
+        float r[CS], sum_q = 0.0f, sum_r = 0.0f;
+#pragma unroll
+        for (int c = 0; c < CS; ++c) r[c] = u[c];
+        for (int s = 0; s <= nz; ++s) {
+          if (s > 0) {
+            const int k = W.ord[s - 1];
+            const float qf = W.qf[s - 1];
+            sum_q += fabsf(qf);
+#pragma unroll
+            for (int c = 0; c < CS; ++c) {
+              const int i = lane + 32 * c < M ? lane + 32 * c : 0;
+              r[c] = lane + 32 * c < M ? __fmaf_rn(-qf, ph[i * ld + k], r[c]) : 0.0f;
+            }
+          }
+          float E = 0.0f;
+#pragma unroll
+          for (int c = 0; c < CS; ++c) E = __fmaf_rn(r[c], r[c], E);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) E = __fadd_rn(E, __shfl_xor_sync(FULL, E, o));
+          const float rn = sqrtf(E);
+          if (s > 0) sum_r += rn;
+          const float B = __fmaf_rn(1.05f * kU, __fmaf_rn(4.2f, sum_q, __fmul_rn(1.1f, sum_r)), __fmul_rn(rn, 2.0e-6f));
+          if (lane == 0) W.code[s] = rn + B < tol * 0.999999f ? 1 : (rn - B > tol * 1.000001f ? 0 : 2);
+        }
+      } else {
+        for (int s = lane; s <= M; s += 32) W.code[s] = 2;
+      }
+      __syncwarp();
+      bool have_qd = false;
       int lo = 0, hi = M;
       while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        double part = 0.0;
-        for (int i = lane; i < M; i += 32) {
-          double rec = 0.0;
-          for (int s = 0; s < mid; ++s) {
-            const int k = W.ord[s];
-            rec = __dadd_rn(rec, __dmul_rn(W.qd[k], phi[i * M + k]));
+        const int mid = (lo + hi) >> 1, at = mid < top ? mid : top;
+        int code = W.code[at];
+        if (code == 2) {
+          if (!have_qd) {
+            for (int k = lane; k < M; k += 32) W.qd[k] = __dmul_rn((double)W.q[k], delta);
+            have_qd = true;
           }
-          const double d = __dsub_rn(W.u[i], rec);
-          part = __fma_rn(d, d, part);
+          __syncwarp();
+          code = gb_error(W, phi, M, at, lane) <= eps_l2 ? 1 : 0;
+          if (lane == 0) W.code[at] = (unsigned char)code;
+          __syncwarp();
         }
-        if (gb_warp_sum(part) <= eps_l2) hi = mid;
+        if (code) hi = mid;
         else lo = mid + 1;
       }
       n = lo;
+      if (n > top) gb_order_all(W, phi, M, lane);          // modes with q = 0 are kept too
     }
     // the record: n, wv, n mode indices of ib bits, n zigzag(q) of wv bits
     uint64_t zmax = 0;
@@ -430,19 +678,43 @@ __global__ void __launch_bounds__(kGbWarps * 32) k_gb_patch(GbPlan g, const floa
 }
 
 // ---------------------------------------------------------------- the stream
-// One CTA: the exclusive scan of the record sizes (in place into offsets),
-// the total, and the header, basis and offset table when they fit.
-__global__ void __launch_bounds__(1024) k_gb_scan(GbPlan g, const unsigned long long* sizes,
-                                                  unsigned long long* offsets, const double* phi, GbStatus* st,
-                                                  uint8_t* out, unsigned long long out_cap) {
+// Tiles of kGbTile records: k_gb_tiles sums their sizes, k_gb_scan (one CTA)
+// scans the tiles' sums and writes header and basis, k_gb_copy finishes the
+// scan inside each tile, writing its part of the offset table and its records.
+// (One CTA scanning every record took 586 us for 524 288 of them.)
+__global__ void __launch_bounds__(256) k_gb_tiles(GbPlan g, const unsigned long long* __restrict__ sizes,
+                                                  unsigned long long* tiles) {
+  __shared__ unsigned long long ws[8];
+  const int64_t b = (int64_t)blockIdx.x * kGbTile;
+  unsigned long long s = 0;
+#pragma unroll
+  for (int k = 0; k < kGbTile / 256; ++k) {
+    const int64_t i = b + threadIdx.x + 256 * k;
+    s += i < g.nrec ? sizes[i] : 0ull;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) s += ws[w];
+    tiles[blockIdx.x] = s;
+  }
+}
+
+// The exclusive scan of the tiles' sums (in place), the total, and the header
+// and basis when the stream fits.
+__global__ void __launch_bounds__(1024) k_gb_scan(GbPlan g, unsigned long long* tiles, int64_t ntiles,
+                                                  const double* phi, GbStatus* st, uint8_t* out,
+                                                  unsigned long long out_cap) {
   __shared__ unsigned long long warp_sums[32];
   __shared__ unsigned long long carry;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) carry = 0;
   __syncthreads();
-  for (int64_t base = 0; base < g.nrec; base += 1024) {
+  for (int64_t base = 0; base < ntiles; base += 1024) {
     const int64_t i = base + tid;
-    const unsigned long long v = i < g.nrec ? sizes[i] : 0ull;
+    const unsigned long long v = i < ntiles ? tiles[i] : 0ull;
     unsigned long long x = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -462,17 +734,14 @@ __global__ void __launch_bounds__(1024) k_gb_scan(GbPlan g, const unsigned long 
     }
     __syncthreads();
     const unsigned long long excl = carry + (warp > 0 ? warp_sums[warp - 1] : 0ull) + x - v;
-    if (i < g.nrec) offsets[i] = excl;
+    if (i < ntiles) tiles[i] = excl;
     __syncthreads();
     if (tid == 1023) carry = excl + v;
     __syncthreads();
   }
   const unsigned long long payload = carry;
   const unsigned long long total = (unsigned long long)g.payload_pos + payload;
-  if (tid == 0) {
-    offsets[g.nrec] = payload;
-    st->total = total;
-  }
+  if (tid == 0) st->total = total;
   if (total > out_cap) return;
   const int M = g.M;
   if (tid == 0) {
@@ -489,26 +758,53 @@ __global__ void __launch_bounds__(1024) k_gb_scan(GbPlan g, const unsigned long 
     hd[7] = st->eps_l2;
     hd[8] = st->delta;
     h64[9] = (uint64_t)g.nrec;
+    reinterpret_cast<uint64_t*>(out + g.offsets_pos)[g.nrec] = payload;
   }
   double* basis = reinterpret_cast<double*>(out + kGbHdr);
   for (int e = tid; e < M * M; e += 1024) {
     const int r = e / M, i = e - r * M;          // mode r, component i
     basis[e] = phi[i * M + r];
   }
-  uint64_t* ot = reinterpret_cast<uint64_t*>(out + g.offsets_pos);
-  for (int64_t i = tid; i <= g.nrec; i += 1024) ot[i] = offsets[i];
 }
 
-// The records from their slots to their offsets (8-byte words).
-__global__ void k_gb_copy(GbPlan g, const unsigned long long* sizes, const unsigned long long* offsets,
-                          const uint8_t* slots, const GbStatus* st, uint8_t* out, unsigned long long out_cap) {
+// A tile's offsets, and its records from their slots (8-byte words, eight
+// lanes a record: a record is a few tens of bytes).
+__global__ void __launch_bounds__(256) k_gb_copy(GbPlan g, const unsigned long long* __restrict__ sizes,
+                                                 const unsigned long long* __restrict__ tiles,
+                                                 const uint8_t* __restrict__ slots, const GbStatus* st, uint8_t* out,
+                                                 unsigned long long out_cap) {
+  __shared__ int sh_warp[32];
+  __shared__ unsigned int off[kGbTile + 1];
   if (st->total > out_cap) return;
-  const int64_t p = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (p >= g.nrec) return;
-  const int lane = threadIdx.x & 31;
-  const uint2* src = reinterpret_cast<const uint2*>(slots + p * g.slot_bytes);
-  uint2* dst = reinterpret_cast<uint2*>(out + g.payload_pos + offsets[p]);
-  for (int64_t w = lane; w < (int64_t)(sizes[p] / 8); w += 32) dst[w] = src[w];
+  const int tid = threadIdx.x;
+  const int64_t b = (int64_t)blockIdx.x * kGbTile;
+  const int cnt = (int)((g.nrec - b) < kGbTile ? (g.nrec - b) : kGbTile);
+  const unsigned long long base = tiles[blockIdx.x];
+  int sz[kGbTile / 256], mine = 0;               // four consecutive records a thread
+#pragma unroll
+  for (int k = 0; k < kGbTile / 256; ++k) {
+    const int i = tid * (kGbTile / 256) + k;
+    sz[k] = i < cnt ? (int)sizes[b + i] : 0;
+    mine += sz[k];
+  }
+  int tot;
+  int at = block_excl_scan(mine, sh_warp, &tot);
+#pragma unroll
+  for (int k = 0; k < kGbTile / 256; ++k) {
+    off[tid * (kGbTile / 256) + k] = (unsigned)at;
+    at += sz[k];
+  }
+  if (tid == 0) off[kGbTile] = (unsigned)tot;
+  __syncthreads();
+  uint64_t* ot = reinterpret_cast<uint64_t*>(out + g.offsets_pos);
+  for (int i = tid; i < cnt; i += 256) ot[b + i] = base + off[i];
+  const int sub = tid >> 3, l8 = tid & 7;
+  for (int i = sub; i < cnt; i += 32) {
+    const uint2* src = reinterpret_cast<const uint2*>(slots + (b + i) * g.slot_bytes);
+    uint2* dst = reinterpret_cast<uint2*>(out + g.payload_pos + base + off[i]);
+    const int nw = (int)((off[i + 1] - off[i]) / 8);
+    for (int w = l8; w < nw; w += 8) dst[w] = src[w];
+  }
 }
 
 // ---------------------------------------------------------------- decoder
@@ -536,6 +832,13 @@ __global__ void __launch_bounds__(256) k_gb_decode(GbPlan g, const uint8_t* __re
     if (lane == 0) atomicOr(&st->corrupt, 1u);
     return;
   }
+  // the entries, one a lane: mode and q delta to shared memory, once a record
+  // (each lane unpacking and multiplying every entry for its own points was
+  // half of the decoder's time)
+  __shared__ double sqd[8][kGbMaxM];
+  __shared__ short smode[8][kGbMaxM];
+  double* qd = sqd[threadIdx.x >> 5];
+  short* md = smode[threadIdx.x >> 5];
   const uint32_t* w = r + 2;
   auto get = [&](uint64_t pos, int width) -> uint64_t {
     uint64_t v = 0;
@@ -549,6 +852,20 @@ __global__ void __launch_bounds__(256) k_gb_decode(GbPlan g, const uint8_t* __re
     }
     return v;
   };
+  bool bad = false;
+  for (int s = lane; s < n; s += 32) {
+    const int k = (int)get((uint64_t)s * ib, ib);
+    const uint64_t z = get((uint64_t)n * ib + (uint64_t)s * wv, wv);
+    const long long q = (long long)((z >> 1) ^ (0ull - (z & 1ull)));
+    bad |= k >= M;
+    md[s] = (short)k;
+    qd[s] = __dmul_rn((double)q, delta);
+  }
+  if (__any_sync(0xffffffffu, bad)) {
+    if (lane == 0) atomicOr(&st->corrupt, 1u);
+    return;
+  }
+  __syncwarp();
   const int64_t pps = g.npx * g.npy * g.npz;
   const int64_t t = p / pps, rem = p - t * pps;
   const int64_t bz = rem / (g.npx * g.npy), r2 = rem - bz * g.npx * g.npy;
@@ -556,16 +873,7 @@ __global__ void __launch_bounds__(256) k_gb_decode(GbPlan g, const uint8_t* __re
   const int64_t x0 = bx * g.px, y0 = by * g.py, z0 = bz * g.pz;
   for (int i = lane; i < M; i += 32) {
     double rec = 0.0;
-    for (int s = 0; s < n; ++s) {
-      const int k = (int)get((uint64_t)s * ib, ib);
-      const uint64_t z = get((uint64_t)n * ib + (uint64_t)s * wv, wv);
-      const long long q = (long long)((z >> 1) ^ (0ull - (z & 1ull)));
-      if (k >= M) {
-        if (lane == 0) atomicOr(&st->corrupt, 1u);
-        return;
-      }
-      rec = __dadd_rn(rec, __dmul_rn(__dmul_rn((double)q, delta), basis[(int64_t)k * M + i]));
-    }
+    for (int s = 0; s < n; ++s) rec = __dadd_rn(rec, __dmul_rn(qd[s], __ldg(basis + (int64_t)md[s] * M + i)));
     const int ix = i % g.px, iy = (i / g.px) % g.py, iz = i / (g.px * g.py);
     out[((t * g.dims[2] + z0 + iz) * g.dims[1] + (y0 + iy)) * g.dims[0] + (x0 + ix)] = rec;
   }
@@ -608,7 +916,7 @@ int dls_gb_compress(const dls_gb_params* p, const float* d_in, const int64_t* d_
   double* partial = (double*)(w + L.partial);
   GbStatus* gs = (GbStatus*)(w + L.status);
   unsigned long long* sizes = (unsigned long long*)(w + L.sizes);
-  unsigned long long* offsets = (unsigned long long*)(w + L.offsets);
+  unsigned long long* tiles = (unsigned long long*)(w + L.tiles);
   uint8_t* slots = w + L.slots;
   if (cudaMemsetAsync(gs, 0, sizeof(GbStatus), s) != cudaSuccess) return DLS_ERR_CUDA;
   k_gb_sample<<<(unsigned)g.S, 128, 0, s>>>(g, d_in, d_origins, Q, gs);
@@ -621,21 +929,28 @@ int dls_gb_compress(const dls_gb_params* p, const float* d_in, const int64_t* d_
     return DLS_ERR_CUDA;
   k_gb_jacobi<<<1, kJacThreads, jsm, s>>>(g, G, V, phi, lam, v_shared);
   k_gb_norm<<<kGbStatCtas, 256, 0, s>>>(g, d_in, partial, gs);
-  k_gb_resolve<<<1, 1, 0, s>>>(g, partial, gs);
+  k_gb_resolve<<<1, 128, 0, s>>>(g, partial, gs);
   const size_t psm = gb_patch_smem(g.M);
-  if (cudaFuncSetAttribute(k_gb_patch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm) != cudaSuccess)
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return DLS_ERR_CUDA;
-  int per = 0, dev = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_gb_patch, kGbWarps * 32, psm) != cudaSuccess ||
-      cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+  auto patches = [&](auto kern) -> bool {
+    int per = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kGbWarps * 32, psm) != cudaSuccess || per < 1)
+      return false;
+    const int64_t need = cdiv(g.nrec, kGbWarps);
+    const unsigned grid = (unsigned)((int64_t)per * sms < need ? (int64_t)per * sms : need);
+    kern<<<grid, kGbWarps * 32, psm, s>>>(g, d_in, phi, gs, gs, sizes, slots);
+    return true;
+  };
+  if (!(g.M <= 32 ? patches(k_gb_patch<1>) : g.M <= 64 ? patches(k_gb_patch<2>) : g.M <= 96 ? patches(k_gb_patch<3>)
+                                                                                            : patches(k_gb_patch<4>)))
     return DLS_ERR_CUDA;
-  if (per < 1) return DLS_ERR_CUDA;
-  const int64_t need = cdiv(g.nrec, kGbWarps);
-  const unsigned grid = (unsigned)((int64_t)per * sms < need ? (int64_t)per * sms : need);
-  k_gb_patch<<<grid, kGbWarps * 32, psm, s>>>(g, d_in, phi, gs, gs, sizes, slots);
-  k_gb_scan<<<1, 1024, 0, s>>>(g, sizes, offsets, phi, gs, (uint8_t*)d_out, (unsigned long long)out_cap);
-  k_gb_copy<<<(unsigned)cdiv(g.nrec, 8), 256, 0, s>>>(g, sizes, offsets, slots, gs, (uint8_t*)d_out,
-                                                     (unsigned long long)out_cap);
+  const int64_t ntiles = cdiv(g.nrec, kGbTile);
+  k_gb_tiles<<<(unsigned)ntiles, 256, 0, s>>>(g, sizes, tiles);
+  k_gb_scan<<<1, 1024, 0, s>>>(g, tiles, ntiles, phi, gs, (uint8_t*)d_out, (unsigned long long)out_cap);
+  k_gb_copy<<<(unsigned)ntiles, 256, 0, s>>>(g, sizes, tiles, slots, gs, (uint8_t*)d_out, (unsigned long long)out_cap);
   if (cudaGetLastError() != cudaSuccess) return DLS_ERR_CUDA;
   GbStatus hs;
   if (cudaMemcpyAsync(&hs, gs, sizeof(hs), cudaMemcpyDeviceToHost, s) != cudaSuccess ||

@@ -205,21 +205,6 @@ __global__ void __launch_bounds__(kPackThreads) k_pack(Plan P, const T* __restri
 constexpr int kStatCtas = 512;
 constexpr int kRangeCtas = 152 * 8;      // k_range: all that are resident at 256 threads
 
-// (double)x exactly by integer operations where x is normal: the conversion
-// instruction issues on the FP64 pipe (about two lanes a clock and SM), which
-// the sums below already keep busy.  Infinities and NaNs come out finite: the
-// caller screens them by their exponent.
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t u = __float_as_uint(x);
-  if ((u & 0x7F800000u) == 0u) return (double)x;       // zeros and subnormals
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
-}
-__device__ __forceinline__ double widen(double x) { return x; }
-__device__ __forceinline__ bool not_finite(float x) { return (__float_as_uint(x) & 0x7F800000u) == 0x7F800000u; }
-__device__ __forceinline__ bool not_finite(double x) {
-  return (__double2hiint(x) & 0x7FF00000) == 0x7FF00000;
-}
-
 // A thread's running minimum, maximum and non-finite flag.  float64 values are
 // compared as integers (order-preserving for finite values): FP64 comparisons
 // would issue on the FP64 pipe.

@@ -22,7 +22,7 @@
 // finite tests and magnitude comparisons are integer operations.
 // 512 blocks of 16^3 x 16 float32: 14.48 -> 2.10 ms; 64 blocks of 8 x 8 x 32
 // float64: 15.04 -> 1.73 ms (before: all of it in FP64, the eigensolve in one warp).
-#include "dls_internal.cuh"
+#include "dls_device.cuh"
 
 namespace dls {
 namespace {
@@ -47,26 +47,6 @@ template <> __device__ __forceinline__ double dequant<double>(int32_t q, double 
 template <typename T> __device__ __forceinline__ T tfma(T a, T b, T c);
 template <> __device__ __forceinline__ float tfma<float>(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 template <> __device__ __forceinline__ double tfma<double>(double a, double b, double c) { return __fma_rn(a, b, c); }
-
-// (double)x by integer operations where x is a normal float: the conversion
-// instruction issues on the FP64 pipe.  Callers screen infinities and NaNs.
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t u = __float_as_uint(x);
-  if ((u & 0x7F800000u) == 0u) return (double)x;       // zeros and subnormals
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
-}
-__device__ __forceinline__ double widen(double x) { return x; }
-__device__ __forceinline__ bool not_finite(float x) { return (__float_as_uint(x) & 0x7F800000u) == 0x7F800000u; }
-__device__ __forceinline__ bool not_finite(double x) { return (__double2hiint(x) & 0x7FF00000) == 0x7FF00000; }
-// |x| < b for a finite b >= 0, on the bit patterns (false for a NaN x).
-__device__ __forceinline__ bool mag_below(double x, double b) {
-  return (__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) < __double_as_longlong(b);
-}
-
-// |x| > b for b >= 0, likewise (true for a NaN x).
-__device__ __forceinline__ bool mag_above(double x, double b) {
-  return (__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) > __double_as_longlong(b);
-}
 
 // Rotation parameters of one round.
 template <int NM>
