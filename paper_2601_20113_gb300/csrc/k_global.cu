@@ -419,7 +419,7 @@ __device__ __noinline__ void gb_order_all(GbWarp& W, const double* __restrict__ 
 //    unless sqrt(eps_l^2) lies within B_s (and the sum's rounding) of it.
 // Patches whose scale FP32 does not carry, and n = M (no kept count passes),
 // take the definition throughout.  Measured at M = 64, 524 288 patches:
-// @GB@.
+// 15.57 -> 1.58 ms; the whole compression and read-back 25.7 -> 10.3 ms.
 template <int CS>
 __global__ void __launch_bounds__(kGbWarps * 32) k_gb_patch(GbPlan g, const float* __restrict__ in,
                                                             const double* __restrict__ phi, const GbStatus* stc,
