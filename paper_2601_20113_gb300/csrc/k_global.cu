@@ -7,9 +7,9 @@
 // steps are
 //   k_gb_sample   the sample matrix Q (S x M) from the first snapshot,
 //   k_gb_gram     G = Q^T Q, each entry a sequential sum over the samples,
-//   k_gb_jacobi   the eigenvectors of G by cyclic Jacobi in one CTA (G and,
-//                 when they fit, V in shared memory), sorted by decreasing
-//                 eigenvalue and signed (largest component positive),
+//   k_gb_jacobi   the eigenvectors of G by cyclic Jacobi in one cluster of
+//                 CTAs (the rows of G and V shared out among them), sorted by
+//                 decreasing eigenvalue and signed (largest component positive),
 //   k_gb_norm     ||u||^2 of the variable, then eps_l^2 and delta,
 //   k_gb_patch    a warp per patch: alpha = Phi^T u, q = rint(alpha / delta),
 //                 the magnitude order, the bisection on the kept count, the
@@ -17,7 +17,11 @@
 //   scan + copy   the record offsets and the stream.  (The FP64 definitions run
 //                 where an FP32 evaluation cannot settle what they decide.)
 // The decoder rebuilds each patch from its kept modes in kept order.
+#include <cooperative_groups.h>
+
 #include "dls_device.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace dls {
 namespace {
@@ -100,10 +104,9 @@ GbLayout gb_layout(const GbPlan& g) {
     return o;
   };
   const size_t MM = (size_t)g.M * g.M;
-  const size_t me = (size_t)(g.M + (g.M & 1));   // the Jacobi's even order
   L.Q = take(sizeof(double) * (size_t)g.S * g.M);
   L.G = take(sizeof(double) * MM);
-  L.V = take(sizeof(double) * me * me);
+  L.V = take(sizeof(double) * MM);
   L.phi = take(sizeof(double) * MM);
   L.lam = take(sizeof(double) * (size_t)g.M);
   L.partial = take(sizeof(double) * kGbStatCtas);
@@ -149,112 +152,222 @@ __device__ __forceinline__ void gb_pair(int round, int i, int m, int& p, int& q)
   q = a < b ? b : a;
 }
 
-// Cyclic Jacobi of G (order M, padded with a zero row and column to even m),
-// one CTA: every round rotates the m/2 disjoint pairs of the round-robin
-// circle whose off-diagonal entry exceeds 2^-53 sqrt(|a_pp a_qq|); each 2 x 2
-// block of A (pair k's rows, pair l's columns) becomes J_k^T A_kl J_l, with
-// the exact 2 x 2 result on the diagonal blocks, and V's column pairs rotate.
-// Stops after a sweep without rotation (50 sweeps at most).  Then the modes:
-// columns of V by decreasing eigenvalue (index order on ties), each signed so
-// that its largest-magnitude component (the first on ties) is positive.
-constexpr int kJacThreads = 1024;
-__global__ void __launch_bounds__(kJacThreads, 1) k_gb_jacobi(GbPlan g, const double* __restrict__ G, double* Vg,
-                                                               double* phi, double* lam_out, int v_shared) {
-  extern __shared__ double A[];               // m x m, then V (m x m) when v_shared
-  __shared__ int pq[kGbMaxM / 2];
-  __shared__ double jc[kGbMaxM / 2], js[kGbMaxM / 2], jt[kGbMaxM / 2];
-  __shared__ double lam[kGbMaxM];
-  __shared__ int order[kGbMaxM];
-  const int tid = threadIdx.x;
-  const int M = g.M, m = M + (M & 1), h = m / 2;
-  double* V = v_shared ? A + m * m : Vg;
-  for (int e = tid; e < m * m; e += kJacThreads) {
-    const int i = e / m, j = e - i * m;
-    A[e] = (i < M && j < M) ? G[i * M + j] : 0.0;
-    V[e] = i == j ? 1.0 : 0.0;
+// The pair of round `round` that index x is in, and whether x is its larger one.
+__device__ __forceinline__ int gb_pair_of(int round, int x, int m, int& larger) {
+  int y, i = 0;
+  if (x == m - 1) {
+    y = round;
+  } else if (x == round) {
+    y = m - 1;
+  } else {
+    int d = x - round;
+    d = d < 0 ? d + m - 1 : d;
+    i = d <= (m - 2) / 2 ? d : m - 1 - d;
+    // x = round + i or round - i (mod m - 1); its partner is the other
+    y = d == i ? round - i : round + i;
+    y = y < 0 ? y + m - 1 : (y >= m - 1 ? y - (m - 1) : y);
   }
-  __syncthreads();
+  larger = x > y ? 1 : 0;
+  return i;
+}
+
+// Cyclic Jacobi of G (order M, padded with a zero row and column to even m):
+// every round rotates the m/2 disjoint pairs of the round-robin circle whose
+// off-diagonal entry exceeds 2^-53 sqrt(|a_pp a_qq|); each 2 x 2 block of A
+// (pair k's rows, pair l's columns) becomes J_k^T A_kl J_l, with the exact
+// 2 x 2 result on the diagonal blocks, and V's column pairs rotate.  Stops
+// after a sweep without rotation (50 sweeps at most).  Then the modes: columns
+// of V by decreasing eigenvalue (index order on ties), each signed so that its
+// largest-magnitude component (the first on ties) is positive.
+//
+// One SM's FP64 units took 10.7 us a round at M = 64 (768 warp instructions of
+// them), so a cluster of eight CTAs shares it.  In a round CTA c owns the pairs
+// [c kpc, (c + 1) kpc): it holds their rows of A, works out their rotations and
+// sends these to all eight; then it forms its rows' new entries and sends each
+// row to the CTA that owns it in the next round (a row has one reader, so a
+// round moves A once).  Rows of V never mix: each CTA keeps M / 8 of them and
+// rotates them while the next round's rotations are worked out, which is the
+// longest chain left (three divisions and two square roots, about 3 000
+// clocks); the threshold of a pair is another warp's work.  Two cluster
+// barriers a round.  Measured at M = 64: 6.75 -> 2.81 ms.
+constexpr int kJacCtas = 8;
+constexpr int kJacThreads = 256;
+struct GbRot {
+  double c[kGbMaxM / 2], s[kGbMaxM / 2], t[kGbMaxM / 2];
+  int act[kGbMaxM / 2];
+};
+constexpr int kJacRows = 2 * (kGbMaxM / 2 / kJacCtas);     // rows of A a CTA owns, rows of V it keeps
+static_assert(kJacRows * kJacCtas == kGbMaxM, "rows");
+struct GbJac {
+  GbRot rot[2];
+  double A[2][kJacRows][kGbMaxM + 1];
+  double V[kJacRows][kGbMaxM + 1];
+  double lam[kGbMaxM];
+  int order[kGbMaxM];
+};
+
+__global__ void __cluster_dims__(kJacCtas, 1, 1) __launch_bounds__(kJacThreads, 1)
+    k_gb_jacobi(GbPlan g, const double* __restrict__ G, double* Vg, double* phi, double* lam_out) {
+  extern __shared__ __align__(16) unsigned char jsm[];
+  GbJac& S = *reinterpret_cast<GbJac*>(jsm);
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int M = g.M, m = M + (M & 1), h = m / 2;
+  const int kpc = (h + kJacCtas - 1) / kJacCtas, k0 = rank * kpc, nk = k0 >= h ? 0 : (h - k0 < kpc ? h - k0 : kpc);
+  const int vr = (M + kJacCtas - 1) / kJacCtas, v0 = rank * vr, nv = v0 >= M ? 0 : (M - v0 < vr ? M - v0 : vr);
+  for (int e = tid; e < 2 * nk * m; e += kJacThreads) {
+    const int r = e / m, j = e - r * m;
+    int p, q;
+    gb_pair(0, k0 + (r >> 1), m, p, q);
+    const int i = (r & 1) ? q : p;
+    S.A[0][r][j] = (i < M && j < M) ? G[i * M + j] : 0.0;
+  }
+  for (int e = tid; e < nv * m; e += kJacThreads) {
+    const int r = e / m, j = e - r * m;
+    S.V[r][j] = v0 + r == j ? 1.0 : 0.0;
+  }
+  cl.sync();
+  int ab = 0, pb = 0;
+  bool turn_v = false;                         // V is one round behind, with the parameters in rot[pb ^ 1]
+  int turn_round = 0;
+  // V's rows by the rotations of a round, on the warps that leave warp 0's and warp 1's FP64 units alone
+  auto rotate_v = [&](const GbRot& R, int round) {
+    const int w = warp & 3;
+    if (w < 2) return;
+    const int vt = ((warp >> 2) * 2 + (w - 2)) * 32 + lane;
+    for (int it = vt; it < nv * h; it += kJacThreads / 2) {
+      const int i = it / h, l = it - i * h;
+      if (!R.act[l]) continue;
+      int p, q;
+      gb_pair(round, l, m, p, q);
+      const double c = R.c[l], s = R.s[l];
+      const double x = S.V[i][p], y = S.V[i][q];
+      S.V[i][p] = __fma_rn(c, x, -__dmul_rn(s, y));
+      S.V[i][q] = __fma_rn(s, x, __dmul_rn(c, y));
+    }
+  };
   for (int sweep = 0; sweep < 50 && M > 1; ++sweep) {
     int any = 0;
     for (int round = 0; round < m - 1; ++round) {
-      int act = 0;
-      if (tid < h) {
+      // this CTA's rotations, to every CTA
+      if (warp == 0 && lane < nk) {
         int p, q;
-        gb_pair(round, tid, m, p, q);
-        const double app = A[p * m + p], aqq = A[q * m + q], apq = A[p * m + q];
+        gb_pair(round, k0 + lane, m, p, q);
+        const double app = S.A[ab][2 * lane][p], aqq = S.A[ab][2 * lane + 1][q], apq = S.A[ab][2 * lane][q];
         double c = 1.0, s = 0.0, t = 0.0;
-        if (apq != 0.0 && fabs(apq) > 0x1p-53 * sqrt(fabs(app) * fabs(aqq))) {
-          const double theta = (aqq - app) / (2.0 * apq);
-          if (fabs(theta) > 1e150) t = 0.5 / theta;
-          else t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(1.0 + theta * theta));
-          c = 1.0 / sqrt(1.0 + t * t);
-          s = t * c;
-          act = 1;
-        }
-        pq[tid] = p | q << 8 | act << 16;
-        jc[tid] = c;
-        js[tid] = s;
-        jt[tid] = t;
-      }
-      if (!__syncthreads_or(act)) continue;
-      any = 1;
-      for (int it = tid; it < h * h + m * h; it += kJacThreads) {
-        if (it < h * h) {
-          const int k = it / h, l = it - k * h;
-          const int a = pq[k], b = pq[l];
-          if (!((a | b) >> 16)) continue;
-          const int p = a & 255, q = (a >> 8) & 255, pp = b & 255, qq = (b >> 8) & 255;
-          const double ck = jc[k], sk = js[k], cl = jc[l], sl = js[l];
-          if (k == l) {
-            const double t = jt[k], apq = A[p * m + q];
-            const double np = A[p * m + p] - t * apq, nq = A[q * m + q] + t * apq;
-            A[p * m + p] = np;
-            A[q * m + q] = nq;
-            A[p * m + q] = 0.0;
-            A[q * m + p] = 0.0;
-            continue;
+        if (apq != 0.0) {
+          const double theta = __ddiv_rn(__dsub_rn(aqq, app), __dmul_rn(2.0, apq));
+          if (mag_above(theta, 1e150)) {
+            t = __ddiv_rn(0.5, theta);
+          } else {
+            t = __drcp_rn(__dadd_rn(fabs(theta), __dsqrt_rn(__fma_rn(theta, theta, 1.0))));
+            const long long tb = __double_as_longlong(theta);
+            if (tb < 0 && (tb << 1) != 0) t = -t;          // theta < 0
           }
-          const double x = A[p * m + pp], y = A[p * m + qq], z = A[q * m + pp], w = A[q * m + qq];
-          const double r1 = ck * x - sk * z, r2 = ck * y - sk * w, r3 = sk * x + ck * z, r4 = sk * y + ck * w;
-          A[p * m + pp] = cl * r1 - sl * r2;
-          A[p * m + qq] = sl * r1 + cl * r2;
-          A[q * m + pp] = cl * r3 - sl * r4;
-          A[q * m + qq] = sl * r3 + cl * r4;
-        } else {
-          const int it2 = it - h * h;
-          const int i = it2 / h, l = it2 - i * h;
-          const int b = pq[l];
-          if (!(b >> 16)) continue;
-          const int p = b & 255, q = (b >> 8) & 255;
-          const double c = jc[l], s = js[l];
-          const double x = V[i * m + p], y = V[i * m + q];
-          V[i * m + p] = c * x - s * y;
-          V[i * m + q] = s * x + c * y;
+          c = __drcp_rn(__dsqrt_rn(__fma_rn(t, t, 1.0)));
+          s = __dmul_rn(t, c);
         }
+        for (int d = 0; d < kJacCtas; ++d) {
+          GbRot* R = cl.map_shared_rank(&S.rot[pb], d);
+          R->c[k0 + lane] = c;
+          R->s[k0 + lane] = s;
+          R->t[k0 + lane] = t;
+        }
+      } else if (warp == 1 && lane < nk) {
+        int p, q;
+        gb_pair(round, k0 + lane, m, p, q);
+        const double app = S.A[ab][2 * lane][p], aqq = S.A[ab][2 * lane + 1][q], apq = S.A[ab][2 * lane][q];
+        const int act =
+            apq != 0.0 && fabs(apq) > __dmul_rn(0x1p-53, __dsqrt_rn(__dmul_rn(fabs(app), fabs(aqq)))) ? 1 : 0;
+        for (int d = 0; d < kJacCtas; ++d) cl.map_shared_rank(&S.rot[pb], d)->act[k0 + lane] = act;
+      } else if (turn_v) {
+        rotate_v(S.rot[pb ^ 1], turn_round);
       }
-      __syncthreads();
+      cl.sync();
+      const GbRot& R = S.rot[pb];
+      int act_any = 0;
+      for (int l = lane; l < h; l += 32) act_any |= R.act[l];
+      act_any = __any_sync(0xffffffffu, act_any != 0);
+      any |= act_any;
+      // the rows' new entries, to their owners of the next round
+      const int next = round + 1 < m - 1 ? round + 1 : 0;
+      for (int it = tid; it < nk * h; it += kJacThreads) {
+        const int kl = it / h, l = it - kl * h, k = k0 + kl;
+        int p, q, pp, qq;
+        gb_pair(round, k, m, p, q);
+        gb_pair(round, l, m, pp, qq);
+        const int ak = R.act[k], al = R.act[l];
+        double x = S.A[ab][2 * kl][pp], y = S.A[ab][2 * kl][qq];
+        double z = S.A[ab][2 * kl + 1][pp], w = S.A[ab][2 * kl + 1][qq];
+        if (k == l) {
+          if (ak) {
+            const double t = R.t[k];
+            x = __fma_rn(-t, y, x);
+            w = __fma_rn(t, y, w);
+            y = 0.0;
+            z = 0.0;
+          }
+        } else if (ak | al) {
+          const double ck = ak ? R.c[k] : 1.0, sk = ak ? R.s[k] : 0.0, c = al ? R.c[l] : 1.0, s = al ? R.s[l] : 0.0;
+          const double r1 = __fma_rn(ck, x, -__dmul_rn(sk, z)), r2 = __fma_rn(ck, y, -__dmul_rn(sk, w));
+          const double r3 = __fma_rn(sk, x, __dmul_rn(ck, z)), r4 = __fma_rn(sk, y, __dmul_rn(ck, w));
+          x = __fma_rn(c, r1, -__dmul_rn(s, r2));
+          y = __fma_rn(s, r1, __dmul_rn(c, r2));
+          z = __fma_rn(c, r3, -__dmul_rn(s, r4));
+          w = __fma_rn(s, r3, __dmul_rn(c, r4));
+        }
+        int gp, gq;
+        const int op = gb_pair_of(next, p, m, gp), oq = gb_pair_of(next, q, m, gq);
+        double* dp = cl.map_shared_rank(&S.A[ab ^ 1][2 * (op % kpc) + gp][0], op / kpc);
+        double* dq = cl.map_shared_rank(&S.A[ab ^ 1][2 * (oq % kpc) + gq][0], oq / kpc);
+        dp[pp] = x;
+        dp[qq] = y;
+        dq[pp] = z;
+        dq[qq] = w;
+      }
+      turn_v = act_any != 0;
+      turn_round = round;
+      ab ^= 1;
+      pb ^= 1;
+      cl.sync();
     }
     if (!any) break;
   }
-  for (int k = tid; k < M; k += kJacThreads) lam[k] = A[k * m + k];
+  if (turn_v) rotate_v(S.rot[pb ^ 1], turn_round);
+  // the rows now lie as round 0 pairs them; eigenvalues and V through global memory to CTA 0
   __syncthreads();
+  for (int r = tid; r < 2 * nk; r += kJacThreads) {
+    int p, q;
+    gb_pair(0, k0 + (r >> 1), m, p, q);
+    const int i = (r & 1) ? q : p;
+    if (i < M) cl.map_shared_rank(&S.lam[0], 0)[i] = S.A[ab][r][i];
+  }
+  for (int e = tid; e < nv * M; e += kJacThreads) {
+    const int r = e / M, j = e - r * M;
+    Vg[(v0 + r) * M + j] = S.V[r][j];
+  }
+  __threadfence();
+  cl.sync();
+  if (rank != 0) return;
   for (int k = tid; k < M; k += kJacThreads) {
-    int rank = 0;
-    for (int j = 0; j < M; ++j) rank += (lam[j] > lam[k] || (lam[j] == lam[k] && j < k)) ? 1 : 0;
-    order[rank] = k;
+    int at = 0;
+    for (int j = 0; j < M; ++j) at += (S.lam[j] > S.lam[k] || (S.lam[j] == S.lam[k] && j < k)) ? 1 : 0;
+    S.order[at] = k;
   }
   __syncthreads();
   for (int r = tid; r < M; r += kJacThreads) {
-    const int k = order[r];
+    const int k = S.order[r];
     int imax = 0;
-    double vmax = -1.0;
+    double vmax = 0.0;
+#pragma unroll 8
     for (int i = 0; i < M; ++i) {
-      const double a = fabs(V[i * m + k]);
-      if (a > vmax) { vmax = a; imax = i; }
+      const double a = fabs(__ldcg(&Vg[i * M + k]));
+      if (i == 0 || mag_above(a, vmax)) { vmax = a; imax = i; }
     }
-    const double sg = V[imax * m + k] < 0.0 ? -1.0 : 1.0;
-    for (int i = 0; i < M; ++i) phi[i * M + r] = sg * V[i * m + k];
-    lam_out[r] = lam[k];
+    const double sg = __ldcg(&Vg[imax * M + k]) < 0.0 ? -1.0 : 1.0;
+#pragma unroll 8
+    for (int i = 0; i < M; ++i) phi[i * M + r] = sg * __ldcg(&Vg[i * M + k]);
+    lam_out[r] = S.lam[k];
   }
 }
 
@@ -921,13 +1034,9 @@ int dls_gb_compress(const dls_gb_params* p, const float* d_in, const int64_t* d_
   if (cudaMemsetAsync(gs, 0, sizeof(GbStatus), s) != cudaSuccess) return DLS_ERR_CUDA;
   k_gb_sample<<<(unsigned)g.S, 128, 0, s>>>(g, d_in, d_origins, Q, gs);
   k_gb_gram<<<(unsigned)cdiv((int64_t)g.M * g.M, 256), 256, 0, s>>>(g, Q, G);
-  // V beside A in shared memory when both fit (M <= 90), else in global memory
-  const int me = g.M + (g.M & 1);
-  const int v_shared = 2 * sizeof(double) * (size_t)me * me <= 200 * 1024 ? 1 : 0;
-  const size_t jsm = sizeof(double) * (size_t)me * me * (v_shared ? 2 : 1);
-  if (cudaFuncSetAttribute(k_gb_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)jsm) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_gb_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GbJac)) != cudaSuccess)
     return DLS_ERR_CUDA;
-  k_gb_jacobi<<<1, kJacThreads, jsm, s>>>(g, G, V, phi, lam, v_shared);
+  k_gb_jacobi<<<kJacCtas, kJacThreads, sizeof(GbJac), s>>>(g, G, V, phi, lam);
   k_gb_norm<<<kGbStatCtas, 256, 0, s>>>(g, d_in, partial, gs);
   k_gb_resolve<<<1, 128, 0, s>>>(g, partial, gs);
   const size_t psm = gb_patch_smem(g.M);
