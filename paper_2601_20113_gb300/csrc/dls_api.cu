@@ -672,6 +672,7 @@ int dls_decompress(const void* d_comp, size_t comp_bytes, void* d_out, size_t ou
   cudaFreeAsync(dst, s);
   CK(cudaStreamSynchronize(s));
   if (st != DLS_OK) return st;
+  if (hs.timeout) return DLS_ERR_TIMEOUT;
   return hs.corrupt ? DLS_ERR_CORRUPT : DLS_OK;
 }
 

@@ -16,10 +16,6 @@ constexpr int kDecThreads = 256;
 // Shared-memory words for a record's coefficient and correction sections
 // (72 KB: three CTAs per SM, as the launch bounds ask of the registers).
 constexpr int kDecStageWords = 18432;
-// Resident CTAs asked of the registers: 3 (80 registers) or 2 (128, no
-// spills; faster where records are small, the unrolled rows dominating).
-constexpr int kDecMinBlocks = 3;
-constexpr int kDecSmallRecord = 32768;     // mean record bytes up to which the 2-CTA form runs
 
 template <typename T> __device__ __forceinline__ T dq(int32_t q, T d);
 template <> __device__ __forceinline__ float dq<float>(int32_t q, float d) { return __fmul_rn(__int2float_rn(q), d); }
@@ -68,16 +64,15 @@ __device__ __forceinline__ int64_t elem_off(const Plan& p, const Geom& g, int64_
   return spatial_off(p, g, (int)(e - lt * g.M)) + (g.t0 + lt) * p.P;
 }
 
-template <typename T, int NM, int MINB>
-__global__ void __launch_bounds__(kDecThreads, MINB) k_decode(Plan P, const uint8_t* __restrict__ comp,
-                                                        unsigned long long comp_bytes, T* __restrict__ out,
-                                                        Status* st) {
-  extern __shared__ __align__(16) uint32_t stage_sm[];   // kDecStageWords
+// One block of any shape, rank and correction width, by all NT threads of a
+// CTA; stage_sm holds stage_words words.
+template <typename T, int NM, int NT>
+__device__ __forceinline__ void decode_block(const Plan& P, const uint8_t* __restrict__ comp, unsigned long long comp_bytes,
+                             T* __restrict__ out, Status* st, int64_t bi, uint32_t* stage_sm, int stage_words) {
   __shared__ T vst[NM * NM];
   __shared__ int64_t wbase[NM + 1];
   __shared__ int64_t soff_col[NM];   // spatial-side blocks: field offset of column j (time 0)
   __shared__ int bad;
-  const int64_t bi = blockIdx.x;
   const int tid = threadIdx.x;
   const Geom g = block_geom(P, P.b0 + bi);
   const int64_t N = g.N, L = g.L;
@@ -105,7 +100,7 @@ __global__ void __launch_bounds__(kDecThreads, MINB) k_decode(Plan P, const uint
       return;
     }
     const T* vals = reinterpret_cast<const T*>(rec + 16);
-    for (int64_t e = tid; e < N; e += kDecThreads) out[elem_off(P, g, e)] = vals[e];
+    for (int64_t e = tid; e < N; e += NT) out[elem_off(P, g, e)] = vals[e];
     return;
   }
   const int rcap = P.rank_cap < n ? P.rank_cap : n;
@@ -155,7 +150,7 @@ __global__ void __launch_bounds__(kDecThreads, MINB) k_decode(Plan P, const uint
   const double step = reinterpret_cast<const double*>(comp + kHdr + kVarRec * v)[3];
   const T delta_t = from_d<T>(delta), step_t = from_d<T>(step);
   const T* vin = reinterpret_cast<const T*>(rec + lay.off_v);
-  for (int i = tid; i < n * r; i += kDecThreads) {
+  for (int i = tid; i < n * r; i += NT) {
     const int c = i / n, j = i - c * n;
     vst[j * NM + c] = vin[i];
   }
@@ -165,10 +160,10 @@ __global__ void __launch_bounds__(kDecThreads, MINB) k_decode(Plan P, const uint
   // the row loop then reads them at shared-memory latency
   const int64_t cw_at = (lay.off_c - lay.off_q) / 4;
   const int64_t nstage = cw_at + lay.corr_words;
-  const bool staged = nstage <= kDecStageWords;
+  const bool staged = nstage <= stage_words;
   const uint32_t* qw = reinterpret_cast<const uint32_t*>(rec + lay.off_q);
   if (staged)
-    for (int64_t i = tid; i < nstage; i += kDecThreads) stage_sm[i] = qw[i];
+    for (int64_t i = tid; i < nstage; i += NT) stage_sm[i] = qw[i];
   __syncthreads();
   if (staged) qw = stage_sm;
   const uint32_t* cw = qw + cw_at;
@@ -182,7 +177,7 @@ __global__ void __launch_bounds__(kDecThreads, MINB) k_decode(Plan P, const uint
     const uint32_t* qc[R];
 #pragma unroll
     for (int c = 0; c < R; ++c) { wqc[c] = wq[c]; qc[c] = qw + wbase[c]; }
-    for (int64_t l = tid; l < L; l += kDecThreads) {
+    for (int64_t l = tid; l < L; l += NT) {
       const int64_t row_off = g.side == 0 ? spatial_off(P, g, (int)l) + g.t0 * P.P : (g.t0 + l) * P.P;
       T ch[R];
 #pragma unroll
@@ -206,51 +201,7 @@ __global__ void __launch_bounds__(kDecThreads, MINB) k_decode(Plan P, const uint
       }
     }
   };
-  // Time-side blocks of order 16 (the full 16^3 x 16 blocks) at ranks 1-4: the
-  // 16 outputs of a row unrolled, dense corrections read with 32-bit bit
-  // positions one time plane (M wk bits) apart (N wk < 2^32 here), blocks
-  // without dense corrections compiled without their test.
-  auto rows_t16 = [&](auto RK, auto DK) {
-    constexpr int R = decltype(RK)::value;
-    constexpr bool D = decltype(DK)::value;
-    int wqc[R];
-    const uint32_t* qc[R];
-#pragma unroll
-    for (int c = 0; c < R; ++c) { wqc[c] = wq[c]; qc[c] = qw + wbase[c]; }
-    const uint32_t pstep = (uint32_t)g.M * (uint32_t)wk;
-    for (int l = tid; l < (int)L; l += kDecThreads) {
-      T ch[R];
-#pragma unroll
-      for (int c = 0; c < R; ++c) ch[c] = dq<T>(unzigzag(get_bits32(qc[c], (uint32_t)l * (uint32_t)wqc[c], wqc[c])), delta_t);
-      T* o = out + spatial_off(P, g, l) + g.t0 * P.P;
-      uint32_t pos = (uint32_t)l * (uint32_t)wk;
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        T acc = T(0);
-#pragma unroll
-        for (int c = 0; c < R; ++c) acc = tf<T>(ch[c], vst[j * NM + c], acc);
-        if (D) {
-          const int32_t kv = unzigzag(get_bits32(cw, pos, wk));
-          pos += pstep;
-          if (kv != 0) acc = tf<T>((T)kv, step_t, acc);
-        }
-        *o = acc;
-        o += P.P;
-      }
-    }
-  };
-  auto rows_t16_d = [&](auto RK) {
-    if (dense) rows_t16(RK, BoolC<true>());
-    else rows_t16(RK, BoolC<false>());
-  };
-  if (NM == 16 && g.side == 0 && n == 16 && r >= 1 && r <= 4) {
-    switch (r) {
-      case 1: rows_t16_d(RankC<1>()); break;
-      case 2: rows_t16_d(RankC<2>()); break;
-      case 3: rows_t16_d(RankC<3>()); break;
-      default: rows_t16_d(RankC<4>()); break;
-    }
-  } else switch (r) {
+  switch (r) {
     case 1: rows_fixed(RankC<1>()); break;
     case 2: rows_fixed(RankC<2>()); break;
     case 3: rows_fixed(RankC<3>()); break;
@@ -260,7 +211,7 @@ __global__ void __launch_bounds__(kDecThreads, MINB) k_decode(Plan P, const uint
     case 7: rows_fixed(RankC<7>()); break;
     case 8: rows_fixed(RankC<8>()); break;
     default:
-      for (int64_t l = tid; l < L; l += kDecThreads) {
+      for (int64_t l = tid; l < L; l += NT) {
         // row l's field offset: a spatial point (time side) or a time step (spatial side)
         const int64_t row_off = g.side == 0 ? spatial_off(P, g, (int)l) + g.t0 * P.P : (g.t0 + l) * P.P;
         T ch[NM];
@@ -301,7 +252,7 @@ __global__ void __launch_bounds__(kDecThreads, MINB) k_decode(Plan P, const uint
     const int64_t nch = cdiv(N, kRiceChunk);
     const uint32_t* rw = cw + 2 + nch;
     const uint64_t nbits = (uint64_t)cw[0] * 32;
-    for (int64_t ch = tid; ch < nch; ch += kDecThreads) {
+    for (int64_t ch = tid; ch < nch; ch += NT) {
       const int64_t c1 = (ch + 1) * kRiceChunk < N ? (ch + 1) * kRiceChunk : N;
       int64_t e = ch * kRiceChunk;
       uint64_t pos = cw[2 + ch];
@@ -359,13 +310,13 @@ __global__ void __launch_bounds__(kDecThreads, MINB) k_decode(Plan P, const uint
     // thread at a time, all eight loads issued before the first store, so that
     // the read-backs overlap (entries name distinct elements)
     constexpr int kB = 8;
-    for (int64_t i0 = tid; i0 < ncorr; i0 += (int64_t)kB * kDecThreads) {
+    for (int64_t i0 = tid; i0 < ncorr; i0 += (int64_t)kB * NT) {
       int64_t gi[kB];
       int32_t kv[kB];
       T val[kB];
 #pragma unroll
       for (int b = 0; b < kB; ++b) {
-        const int64_t i = i0 + (int64_t)b * kDecThreads;
+        const int64_t i = i0 + (int64_t)b * NT;
         gi[b] = -1;
         kv[b] = 0;
         if (i < ncorr) {
@@ -387,13 +338,425 @@ __global__ void __launch_bounds__(kDecThreads, MINB) k_decode(Plan P, const uint
   if (nesc > 0) {
     const uint32_t* ei = reinterpret_cast<const uint32_t*>(rec + lay.off_ei);
     const T* ev = reinterpret_cast<const T*>(rec + lay.off_ev);
-    for (int64_t i = tid; i < nesc; i += kDecThreads) {
+    for (int64_t i = tid; i < nesc; i += NT) {
       const int64_t e = ei[i];
       if (e >= N) { atomicOr(&st->corrupt, 1u); continue; }
       out[elem_off(P, g, e)] = ev[i];
     }
   }
 }
+
+template <typename T, int NM>
+__global__ void __launch_bounds__(kDecThreads, 3) k_decode(Plan P, const uint8_t* __restrict__ comp,
+                                                           unsigned long long comp_bytes, T* __restrict__ out,
+                                                           Status* st) {
+  extern __shared__ __align__(16) uint32_t stage_sm[];   // kDecStageWords
+  decode_block<T, NM, kDecThreads>(P, comp, comp_bytes, out, st, blockIdx.x, stage_sm, kDecStageWords);
+}
+
+// ---------------------------------------------------------------- float32, Gram order <= 16
+// Persistent decoder of float32 plans with Gram order <= 16 and blocks of at
+// most 65 536 points: CTAs take blocks from a counter and bring each record in
+// whole by one bulk copy.  Time-side blocks of rank <= 8 take the path below
+// when their corrections are dense (up to 8 bits) or listed or Rice coded (up
+// to 4 bits, |k| <= 8), any other block decode_block.
+//  - Listed and Rice-coded corrections go to a nibble a point in shared memory
+//    first (entries by all threads, a Rice chunk a thread), so that the rows
+//    add them as they write each output: no output is read back.
+//  - A thread takes four neighbouring rows where lines are whole multiples of
+//    16 bytes: 16-byte stores, four corrections a load, the basis read once for
+//    four outputs (about 10 instructions an output; a row a thread with
+//    read-backs took 34, which bound it).
+//  - Three CTAs an SM (32 KB of nibbles, 41 KB of record, 80 registers) cover
+//    each other's copies, scatter and Rice chains.  A byte a point with two
+//    staged records (one CTA of 512 threads, or two with records up to 23 KB)
+//    left the SM waiting at barriers: 1.07 and 1.71 to 2.96 ms on the two below.
+// Measured: 4 GiB at 1e-3 x range (23 KB records) 1.50 -> 1.05 ms; five ragged
+// variables with Rice-coded corrections (193 M points) 2.61 -> 0.99 ms.
+// (out of line: the registers of the common path stay its own)
+__device__ __noinline__ void decode_block_f32(const Plan& P, const uint8_t* comp, unsigned long long comp_bytes,
+                                              float* out, Status* st, int64_t bi, uint32_t* stage_sm, int words) {
+  decode_block<float, 16, kDecThreads>(P, comp, comp_bytes, out, st, bi, stage_sm, words);
+}
+constexpr int kPlaneBytes = 32768;
+constexpr int kRecPad = 64;                 // readable bytes past a staged record
+constexpr int kRecCap = 41920;              // bytes of a record staged beside the plane
+constexpr int kRecCapAll = kPlaneBytes + kRecCap;   // ... over it (records that need no plane)
+constexpr uint32_t kNoCorr = 0x88888888u;   // eight nibbles k + 8 = 8
+struct DecRec {                             // one staged record, parsed by warp 0
+  int r, wk, wv, kr, n, M, ncorr, nesc, mode, dense, rice, bad;
+  uint32_t off_v, off_c, rice_words;
+  uint32_t qbase[8];                        // word offset of column c in the record
+  int wq[8];
+  int64_t off_ei, off_ev;
+};
+enum : int { kDecSkip = 0, kDecFast = 1, kDecRaw = 2, kDecGeneric = 3 };
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// Waits at most about a second of SM clock.
+__device__ __forceinline__ bool bar_wait(unsigned long long* b, unsigned parity) {
+  const long long t0 = clock64();
+  for (;;) {
+    for (int i = 0; i < 256; ++i) {
+      uint32_t ok;
+      asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                   : "=r"(ok) : "r"(smem_addr(b)), "r"(parity) : "memory");
+      if (ok) return true;
+    }
+    if (clock64() - t0 > (1ll << 31)) return false;
+  }
+}
+
+// Field `i` of width w (<= 32; mask (1 << w) - 1) of a column of words; reads
+// one word past the field's own.
+__device__ __forceinline__ uint32_t field(const uint32_t* w, uint32_t i, int width, uint32_t mask) {
+  const uint32_t pos = i * (uint32_t)width;
+  const uint32_t* p = w + (pos >> 5);
+  return __funnelshift_r(p[0], p[1], pos & 31u) & mask;
+}
+
+// The rows of a block: R modes, V neighbouring rows a thread, corrections from
+// nowhere (CM = 0), the nibble plane (1) or the dense section (2).
+template <int R, int V, int CM, int NT>
+__device__ __forceinline__ void dec_rows(const Plan& P, const Geom& g, const DecRec& D, const uint32_t* rec,
+                                         const float* vst, const uint8_t* plane, float delta, float step,
+                                         float* __restrict__ out) {
+  const int M = D.M, n = D.n, wk = D.wk;
+  const int64_t tstep = P.P;
+  uint32_t kmask = 0;
+  const uint32_t* cw = rec;
+  if (CM == 2) {
+    kmask = (1u << wk) - 1u;
+    cw = rec + D.off_c / 4;
+  }
+  for (int l = threadIdx.x * V; l < M; l += NT * V) {
+    float ch[R > 0 ? R : 1][V];
+#pragma unroll
+    for (int c = 0; c < R; ++c) {
+      const int w = D.wq[c];
+      const uint32_t mask = w >= 32 ? 0xFFFFFFFFu : (1u << w) - 1u;
+      const uint32_t* col = rec + D.qbase[c];
+#pragma unroll
+      for (int v = 0; v < V; ++v) ch[c][v] = dq<float>(unzigzag(field(col, (uint32_t)(l + v), w, mask)), delta);
+    }
+    float* o = out + spatial_off(P, g, l) + g.t0 * P.P;
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+      float acc[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) acc[v] = 0.0f;
+      if (R > 0) {
+        float b[R > 4 ? 8 : 4];
+        *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(vst + j * 8);
+        if (R > 4) *reinterpret_cast<float4*>(b + 4) = *reinterpret_cast<const float4*>(vst + j * 8 + 4);
+#pragma unroll
+        for (int c = 0; c < R; ++c)
+#pragma unroll
+          for (int v = 0; v < V; ++v) acc[v] = __fmaf_rn(ch[c][v], b[c], acc[v]);
+      }
+      // a correction of zero adds zero
+      if (CM == 1) {
+        // (float)k as (2^23 + k + 8) - (2^23 + 8): exact, and off the conversion pipe
+        const int e = j * M + l;
+        const uint32_t k4 = V == 4 ? (uint32_t)reinterpret_cast<const uint16_t*>(plane)[e >> 2]
+                                   : (uint32_t)plane[e >> 1] >> ((e & 1) * 4);
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+          acc[v] = __fmaf_rn(__fsub_rn(__uint_as_float(((k4 >> (4 * v)) & 15u) | 0x4B000000u), 8388616.0f), step, acc[v]);
+      }
+      if (CM == 2) {
+        // V wk <= 32 bits from one unaligned word
+        const uint32_t pos = (uint32_t)(j * M + l) * (uint32_t)wk;
+        const uint32_t* p = cw + (pos >> 5);
+        const uint32_t f = __funnelshift_r(p[0], p[1], pos & 31u);
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+          acc[v] = __fmaf_rn((float)unzigzag((f >> (v * wk)) & kmask), step, acc[v]);
+      }
+      if (V == 4) *reinterpret_cast<float4*>(o) = make_float4(acc[0], acc[V > 1 ? 1 : 0], acc[V > 2 ? 2 : 0], acc[V > 3 ? 3 : 0]);
+      else *o = acc[0];
+      o += tstep;
+    }
+  }
+}
+template <int V, int CM, int NT>
+__device__ __forceinline__ void dec_rows_rank(const Plan& P, const Geom& g, const DecRec& D, const uint32_t* rec,
+                                              const float* vst, const uint8_t* plane, float delta, float step,
+                                              float* __restrict__ out) {
+  switch (D.r) {
+    case 0: dec_rows<0, V, CM, NT>(P, g, D, rec, vst, plane, delta, step, out); break;
+    case 1: dec_rows<1, V, CM, NT>(P, g, D, rec, vst, plane, delta, step, out); break;
+    case 2: dec_rows<2, V, CM, NT>(P, g, D, rec, vst, plane, delta, step, out); break;
+    case 3: dec_rows<3, V, CM, NT>(P, g, D, rec, vst, plane, delta, step, out); break;
+    case 4: dec_rows<4, V, CM, NT>(P, g, D, rec, vst, plane, delta, step, out); break;
+    case 5: dec_rows<5, V, CM, NT>(P, g, D, rec, vst, plane, delta, step, out); break;
+    case 6: dec_rows<6, V, CM, NT>(P, g, D, rec, vst, plane, delta, step, out); break;
+    case 7: dec_rows<7, V, CM, NT>(P, g, D, rec, vst, plane, delta, step, out); break;
+    default: dec_rows<8, V, CM, NT>(P, g, D, rec, vst, plane, delta, step, out); break;
+  }
+}
+
+// Correction k (|k| <= 8, below 8) of element e into the nibble plane (once an element).
+__device__ __forceinline__ void plane_put(uint32_t* plane, uint32_t e, int32_t k) {
+  atomicXor(&plane[e >> 3], (((uint32_t)(k + 8) ^ 8u) & 15u) << ((e & 7u) * 4));
+}
+
+// One Rice chunk [e, c1) into the plane by one thread; false when the coded
+// words do not hold it.  A code is read from one 64-bit window at its first bit
+// (31 ones, a zero, kr <= 20 and wv <= 4 bits at most), so that the chain from
+// one code to the next is a load, a count and a few shifts; longer runs of ones
+// take the loop.
+__device__ bool dec_rice_chunk(const uint32_t* __restrict__ rw, uint32_t words, uint32_t pos, int kr, int wv, int e,
+                               int c1, uint32_t* plane) {
+  const uint32_t nbits = words * 32u, kmask = (1u << kr) - 1u, vmask = (1u << wv) - 1u;
+  if (pos >= nbits) return false;
+  for (;;) {
+    const uint32_t* p = rw + (pos >> 5);
+    const uint32_t w0 = p[0], w1 = p[1], w2 = p[2], sh = pos & 31u;
+    const uint64_t win = (uint64_t)__funnelshift_r(w0, w1, sh) | ((uint64_t)__funnelshift_r(w1, w2, sh) << 32);
+    const uint32_t ones = ~(uint32_t)win;
+    uint32_t q, rest;
+    if (ones != 0u) {
+      q = (uint32_t)__ffs(ones) - 1u;
+      rest = (uint32_t)(win >> (q + 1u));
+    } else {
+      // 32 ones or more
+      q = 32;
+      for (;;) {
+        const uint32_t at = pos + q;
+        if (at >= nbits || q > (uint32_t)kRiceChunk) return false;
+        const uint32_t* r = rw + (at >> 5);
+        const uint32_t z = ~__funnelshift_r(r[0], r[1], at & 31u);
+        if (z != 0u) { q += (uint32_t)__ffs(z) - 1u; break; }
+        q += 32;
+      }
+      const uint32_t at = pos + q + 1u;
+      if (at >= nbits + 32u) return false;
+      const uint32_t* r = rw + (at >> 5);
+      rest = __funnelshift_r(r[0], r[1], at & 31u);
+    }
+    const uint32_t run = (q << kr) | (rest & kmask);
+    pos += q + 1u + (uint32_t)kr;
+    if (pos > nbits || run > (uint32_t)(c1 - e)) return false;
+    e += (int)run;
+    if (e == c1) return true;
+    pos += (uint32_t)wv;
+    if (pos > nbits) return false;
+    plane_put(plane, (uint32_t)e, unzigzag(((rest >> kr) & vmask) + 1u));
+    ++e;
+  }
+}
+
+// Parses and checks a staged record (warp 0).
+__device__ void dec_parse(const Plan& P, const Geom& g, const uint8_t* rec, int nbytes, DecRec& D) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t* rec32 = reinterpret_cast<const uint32_t*>(rec);
+  const int r = rec[0], flags = rec[1], wk = rec[2], ib = rec[3], n = g.n;
+  const uint32_t ncorr = rec32[1], nesc = rec32[2];
+  const int N = (int)g.N, L = (int)g.L;
+  int mode = kDecFast;
+  if ((int)rec32[3] != nbytes || (flags & ~(int)(kFlagRaw | kFlagSpatial | kFlagDense | kFlagRice)) != 0) mode = kDecGeneric;
+  else if (flags & kFlagRaw) mode = kDecRaw;
+  else if (g.side != 0 || (flags & kFlagSpatial) || r > 8 || wk > 8 || 24 > nbytes || r > (P.rank_cap < n ? P.rank_cap : n) ||
+           ib != bit_width((uint32_t)(N - 1)) || ncorr > (uint32_t)N || nesc > (uint32_t)N)
+    mode = kDecGeneric;                     // refused there where it is damaged
+  if (mode == kDecRaw && 16 + N * 4 > nbytes) mode = kDecGeneric;
+  int w = 0, words = 0;
+  if (mode == kDecFast && lane < r) {
+    w = rec[16 + lane];
+    words = (int)(((int64_t)L * w + 31) >> 5);
+  }
+  if (__any_sync(0xffffffffu, w > 32)) mode = kDecGeneric;
+  int incl = words;
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  const int qwords = __shfl_sync(0xffffffffu, incl, 7);
+  const uint32_t off_v = 16u + (r > 0 ? 8u : 0u), off_q = off_v + (((uint32_t)(n * r) * 4u + 7u) & ~7u);
+  if (lane < 8) {
+    D.wq[lane] = w;
+    D.qbase[lane] = off_q / 4 + (uint32_t)(incl - words);
+  }
+  if (lane != 0) return;
+  D.mode = mode;
+  if (mode != kDecFast) return;
+  const int64_t dense_w = ((int64_t)N * wk + 31) >> 5, sparse_w = ((int64_t)ncorr * (ib + wk) + 31) >> 5;
+  const bool dense = wk > 0 && dense_w < sparse_w, rice = (flags & kFlagRice) != 0;
+  int64_t cwords = wk == 0 ? 0 : (dense ? dense_w : sparse_w);
+  const int64_t off_c = (int64_t)off_q + (((int64_t)qwords * 4 + 7) & ~7ll);
+  D.rice_words = 0;
+  D.kr = D.wv = 0;
+  if (rice) {
+    if (wk == 0 || (flags & kFlagDense) || off_c + 8 > nbytes) { D.mode = kDecGeneric; return; }
+    const uint32_t* cw = reinterpret_cast<const uint32_t*>(rec + off_c);
+    D.rice_words = cw[0];
+    D.kr = (int)(cw[1] & 0xFFu);
+    D.wv = (int)((cw[1] >> 8) & 0xFFu);
+    if ((cw[1] >> 16) != 0u || D.kr > kRiceMaxKr || D.wv > 3 || cw[0] > (uint32_t)nbytes) { D.mode = kDecGeneric; return; }
+    cwords = 2 + (N + kRiceChunk - 1) / kRiceChunk + (int64_t)cw[0];
+  } else if (dense != ((flags & kFlagDense) != 0)) {
+    D.mode = kDecGeneric;
+    return;
+  }
+  if (!dense || rice) {
+    // the nibbles hold -8 .. 7, and the plane must lie beside the record
+    if (wk > 4 || nbytes > kRecCap) { D.mode = kDecGeneric; return; }
+  }
+  D.off_ei = off_c + ((cwords * 4 + 7) & ~7ll);
+  D.off_ev = D.off_ei + (((int64_t)nesc * 4 + 7) & ~7ll);
+  const int64_t size = (D.off_ev + (((int64_t)nesc * 4 + 7) & ~7ll) + 15) & ~15ll;
+  if (size != nbytes) { D.mode = kDecGeneric; return; }
+  D.r = r;
+  D.wk = wk;
+  D.n = n;
+  D.M = (int)g.M;
+  D.ncorr = (int)ncorr;
+  D.nesc = (int)nesc;
+  D.dense = dense ? 1 : 0;
+  D.rice = rice ? 1 : 0;
+  D.off_v = off_v;
+  D.off_c = (uint32_t)off_c;
+}
+
+__global__ void __launch_bounds__(kDecThreads, 3) k_decode_f32(Plan P, const uint8_t* __restrict__ comp,
+                                                               unsigned long long comp_bytes, float* __restrict__ out,
+                                                               Status* st, int vec) {
+  extern __shared__ __align__(128) unsigned char dsm[];       // the record, then the plane
+  constexpr int NT = kDecThreads;
+  uint32_t* plane = reinterpret_cast<uint32_t*>(dsm + kRecCap + kRecPad);
+  const uint8_t* rec = dsm;
+  __shared__ __align__(16) float vst[16 * 8];
+  __shared__ DecRec D;
+  __shared__ unsigned long long full;
+  __shared__ int64_t blk;
+  __shared__ int bytes;                      // of the staged record (0: not staged)
+  __shared__ int stop;
+  const int tid = threadIdx.x;
+  const uint64_t* offs = reinterpret_cast<const uint64_t*>(comp + P.offsets_pos);
+  // the next block (thread 0)
+  auto fetch = [&]() {
+    const int64_t b = (int64_t)atomicAdd(&st->pad[0], 1ull);
+    blk = b;
+    bytes = 0;
+    if (b >= P.nb) return;
+    const uint64_t o0 = offs[b], o1 = offs[b + 1];
+    if (o1 < o0 + 16 || (uint64_t)P.payload_pos + o1 > comp_bytes || ((o0 | o1) & 15) != 0 || o1 - o0 > (uint64_t)kRecCapAll)
+      return;
+    const uint32_t nb = (uint32_t)(o1 - o0);
+    bytes = (int)nb;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&full)), "r"(nb) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_addr(dsm)),
+                 "l"(comp + P.payload_pos + o0), "r"(nb), "r"(smem_addr(&full))
+                 : "memory");
+  };
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&full)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    stop = 0;
+    fetch();
+  }
+  __syncthreads();
+  unsigned phase = 0u;
+  for (;;) {
+    const int64_t bi = blk;
+    if (bi >= P.nb) break;
+    const Geom g = block_geom(P, P.b0 + bi);
+    const int nbytes = bytes;
+    if (nbytes > 0) {
+      if (bar_wait(&full, phase)) phase ^= 1u;
+      else stop = 1;
+      if (tid < 32) {
+        dec_parse(P, g, rec, nbytes, D);
+      } else if (nbytes <= kRecCap && rec[2] != 0 && !(rec[1] & kFlagDense)) {
+        // (the plane of a record whose corrections are not dense)
+        for (int i = tid - 32; i < ((int)g.N + 31) / 32; i += NT - 32)
+          reinterpret_cast<uint4*>(plane)[i] = make_uint4(kNoCorr, kNoCorr, kNoCorr, kNoCorr);
+      }
+      {
+        // basis by component, modes padded to 8 (records' own order: mode by mode)
+        const int r = rec[0] < 8 ? rec[0] : 8;
+        const float* vin = reinterpret_cast<const float*>(rec + 24);
+        for (int i = tid; i < g.n * r; i += NT) {
+          const int c = i / g.n, j = i - c * g.n;
+          vst[j * 8 + c] = vin[i];
+        }
+      }
+    } else if (tid == 0) {
+      D.mode = kDecGeneric;
+    }
+    __syncthreads();
+    if (stop) break;
+    const int mode = D.mode;
+    if (mode == kDecFast) {
+      const double* vt = reinterpret_cast<const double*>(comp + kHdr + kVarRec * g.v);
+      const float delta = __double2float_rn(vt[2]), step = __double2float_rn(vt[3]);
+      const uint32_t* rec32 = reinterpret_cast<const uint32_t*>(rec);
+      const uint32_t* cw = rec32 + D.off_c / 4;
+      const int N = (int)g.N;
+      const bool use_plane = D.wk > 0 && !(D.dense && !D.rice);
+      if (use_plane) {
+        if (D.rice) {
+          const int nch = (N + kRiceChunk - 1) / kRiceChunk;
+          for (int c = tid; c < nch; c += NT) {
+            const int c1 = (c + 1) * kRiceChunk < N ? (c + 1) * kRiceChunk : N;
+            if (!dec_rice_chunk(cw + 2 + nch, D.rice_words, cw[2 + c], D.kr, D.wv, c * kRiceChunk, c1, plane))
+              atomicOr(&st->corrupt, 1u);
+          }
+        } else {
+          const int ib = bit_width((uint32_t)(N - 1)), wk = D.wk, W = ib + wk;      // W <= 20
+          const uint32_t em = (1u << ib) - 1u, km = (1u << wk) - 1u;
+          for (int i = tid; i < D.ncorr; i += NT) {
+            const uint32_t f = field(cw, (uint32_t)i, W, 0xFFFFFFFFu);
+            const uint32_t e = f & em;
+            if (e >= (uint32_t)N) atomicOr(&st->corrupt, 1u);
+            else plane_put(plane, e, unzigzag((f >> ib) & km));
+          }
+        }
+        __syncthreads();
+      }
+      const bool v4 = vec && (g.sx & 3) == 0;
+      const uint8_t* pl = reinterpret_cast<const uint8_t*>(plane);
+      if (use_plane) {
+        if (v4) dec_rows_rank<4, 1, NT>(P, g, D, rec32, vst, pl, delta, step, out);
+        else dec_rows_rank<1, 1, NT>(P, g, D, rec32, vst, pl, delta, step, out);
+      } else if (D.wk > 0) {
+        if (v4) dec_rows_rank<4, 2, NT>(P, g, D, rec32, vst, pl, delta, step, out);
+        else dec_rows_rank<1, 2, NT>(P, g, D, rec32, vst, pl, delta, step, out);
+      } else {
+        if (v4) dec_rows_rank<4, 0, NT>(P, g, D, rec32, vst, pl, delta, step, out);
+        else dec_rows_rank<1, 0, NT>(P, g, D, rec32, vst, pl, delta, step, out);
+      }
+      if (D.nesc > 0) {
+        __syncthreads();
+        const uint32_t* ei = reinterpret_cast<const uint32_t*>(rec + D.off_ei);
+        const float* ev = reinterpret_cast<const float*>(rec + D.off_ev);
+        for (int i = tid; i < D.nesc; i += NT) {
+          const uint32_t e = ei[i];
+          if (e >= (uint32_t)N) { atomicOr(&st->corrupt, 1u); continue; }
+          out[elem_off(P, g, e)] = ev[i];
+        }
+      }
+    } else if (mode == kDecRaw) {
+      const float* vals = reinterpret_cast<const float*>(rec + 16);
+      for (int64_t e = tid; e < g.N; e += NT) out[elem_off(P, g, e)] = vals[e];
+    } else {
+      decode_block_f32(P, comp, comp_bytes, out, st, bi, reinterpret_cast<uint32_t*>(dsm), kRecCapAll / 4);
+    }
+    __syncthreads();
+    if (tid == 0) fetch();
+    __syncthreads();
+  }
+  // a copy did not arrive: report it, and wait for it once more before leaving
+  if (stop && tid == 0) {
+    atomicOr(&st->timeout, 1u);
+    bar_wait(&full, phase);
+  }
+}
+
 
 // ---------------------------------------------------------------- verification
 // acc layout (doubles): per variable v (16 doubles): [0] max_abs_err key (as
@@ -574,8 +937,21 @@ __global__ void k_verify_stream(Plan P, const uint8_t* comp, unsigned long long 
 int launch_decode(const Plan& p, const void* d_comp, unsigned long long comp_bytes, void* d_out,
                         Status* st, cudaStream_t s) {
   if (p.nb == 0) return DLS_OK;
-  const unsigned grid = (unsigned)p.nb;
   const uint8_t* c = (const uint8_t*)d_comp;
+  const int64_t nblk = (int64_t)p.block[0] * p.block[1] * p.block[2] * p.block[3];
+  if (p.dtype == DLS_F32 && p.nmax <= 16 && nblk <= 2 * kPlaneBytes) {
+    int dev = 0, sms = 152;
+    const int smem = kRecCapAll + kRecPad;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(k_decode_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+      return DLS_ERR_CUDA;
+    // 16-byte stores need whole x lines and planes of 16-byte multiples
+    const int vec = p.dims[0] % 4 == 0 && p.block[0] % 4 == 0 && ((uintptr_t)d_out & 15) == 0 ? 1 : 0;
+    const int64_t most = (int64_t)sms * 3;
+    k_decode_f32<<<(unsigned)(p.nb < most ? p.nb : most), kDecThreads, smem, s>>>(p, c, comp_bytes, (float*)d_out, st, vec);
+    return cudaGetLastError() == cudaSuccess ? DLS_OK : DLS_ERR_CUDA;
+  }
+  const unsigned grid = (unsigned)p.nb;
   const int sm = kDecStageWords * 4;
   // the stage buffer is above the 48 KB default: opt in before each launch
   auto go = [&](auto kern, auto* outp) -> bool {
@@ -584,18 +960,10 @@ int launch_decode(const Plan& p, const void* d_comp, unsigned long long comp_byt
     return true;
   };
   bool ok;
-  // measured on 16^3 x 16 float32 blocks: 2 CTAs per SM 1.78 ms against 2.13 at
-  // 1e-3 (21 KB records), 3 CTAs 3.52 against 3.79 at 1e-4 (52 KB records)
-  const bool small = comp_bytes / (unsigned long long)p.nb <= (unsigned long long)kDecSmallRecord;
-  if (p.dtype == DLS_F32) {
-    if (p.nmax <= 16)
-      ok = small ? go(k_decode<float, 16, 2>, (float*)d_out) : go(k_decode<float, 16, kDecMinBlocks>, (float*)d_out);
-    else
-      ok = go(k_decode<float, 32, kDecMinBlocks>, (float*)d_out);
-  } else {
-    ok = p.nmax <= 16 ? go(k_decode<double, 16, kDecMinBlocks>, (double*)d_out)
-                      : go(k_decode<double, 32, kDecMinBlocks>, (double*)d_out);
-  }
+  if (p.dtype == DLS_F32)
+    ok = p.nmax <= 16 ? go(k_decode<float, 16>, (float*)d_out) : go(k_decode<float, 32>, (float*)d_out);
+  else
+    ok = p.nmax <= 16 ? go(k_decode<double, 16>, (double*)d_out) : go(k_decode<double, 32>, (double*)d_out);
   return ok && cudaGetLastError() == cudaSuccess ? DLS_OK : DLS_ERR_CUDA;
 }
 
