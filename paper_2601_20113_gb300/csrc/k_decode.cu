@@ -763,29 +763,90 @@ __global__ void __launch_bounds__(kDecThreads, 3) k_decode_f32(Plan P, const uin
 // u64), [1] n_over (u64), [2] sum_sq_err, [3] sum_sq; then stream totals at
 // 16*nvars: [0] n_raw, [1] sum rank, [2] n_corr, [3] n_esc, [4] basis bytes,
 // [5] coeff bytes, [6] corr bytes, [7] esc bytes, [8] raw bytes, [9] header bytes.
+
+// The stream's composition, by the CTAs of the grid's last row (they run
+// beside the points' CTAs): whole numbers, summed over a warp before the
+// atomics.
+__device__ void verify_stream(const Plan& P, const uint8_t* __restrict__ comp, unsigned long long comp_bytes, int es,
+                              double* acc) {
+  double* t = acc + 16 * P.nvars;
+  const uint64_t* offs = reinterpret_cast<const uint64_t*>(comp + P.offsets_pos);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t first = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+  for (int64_t b0 = first; b0 < P.nb; b0 += stride) {
+    const int64_t bi = b0 + (threadIdx.x & 31);
+    unsigned long long n[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    if (bi < P.nb) {
+      const uint64_t o0 = offs[bi], o1 = offs[bi + 1];
+      if (!(o1 < o0 + 16 || (uint64_t)P.payload_pos + o1 > comp_bytes || (o0 & 15) != 0)) {
+        const uint8_t* rec = comp + P.payload_pos + o0;
+        const uint32_t* rec32 = reinterpret_cast<const uint32_t*>(rec);
+        const int r = rec[0], flags = rec[1];
+        if (flags & kFlagRaw) {
+          n[0] = 1;
+          n[8] = rec32[3];
+        } else if (r <= kMaxN && 16 + align_up(r, 8) <= (int64_t)(o1 - o0)) {
+          const Geom g = block_geom(P, P.b0 + bi);
+          RecLayout lay = rec_layout(r, g.n, g.L, g.N, es, rec + 16, rec[2], rec[3], rec32[1], rec32[2]);
+          if ((flags & kFlagRice) && lay.off_c + 4 <= (int64_t)(o1 - o0))
+            lay = rice_layout(lay, g.N, reinterpret_cast<const uint32_t*>(rec + lay.off_c)[0], rec32[2], es);
+          n[1] = (unsigned long long)r;
+          n[2] = rec32[1];
+          n[3] = rec32[2];
+          n[4] = (unsigned long long)(lay.off_q - lay.off_v);
+          n[5] = (unsigned long long)(lay.off_c - lay.off_q);
+          n[6] = (unsigned long long)(lay.off_ei - lay.off_c);
+          n[7] = (unsigned long long)(lay.size - lay.off_ei);
+          n[9] = (unsigned long long)lay.off_v;
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) n[k] += __shfl_xor_sync(0xffffffffu, n[k], o);
+      if ((threadIdx.x & 31) == 0 && n[k]) atomicAdd(&t[k], (double)n[k]);
+    }
+  }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_verify_points(Plan P, const T* __restrict__ a, const T* __restrict__ b,
-                                                       const uint8_t* comp, double* acc) {
+                                                       const uint8_t* comp, unsigned long long comp_bytes, double* acc) {
   const int v = blockIdx.y;
+  if (v == P.nvars) {
+    verify_stream(P, comp, comp_bytes, (int)sizeof(T), acc);
+    return;
+  }
   const double eb = reinterpret_cast<const double*>(comp + kHdr + kVarRec * v)[1];
   const bool pointwise = P.eb_type != DLS_EB_NRMSE;
-  double mx = 0.0, se = 0.0, sx = 0.0;
+  // three FP64 operations a point; the comparisons are integer ones (a NaN
+  // difference counts nowhere, as in a floating comparison)
+  const long long inf = 0x7FF0000000000000ll, ebb = pointwise ? __double_as_longlong(eb) : inf;
+  long long mxb = 0;
+  double se = 0.0, sx = 0.0;
   unsigned long long over = 0;
   const int64_t base = (int64_t)v * P.K;
+#pragma unroll 4
   for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < P.K; i += (int64_t)gridDim.x * 256) {
     const double x = (double)a[base + i], y = (double)b[base + i];
     const double d = fabs(x - y);
-    mx = fmax(mx, d);
-    if (pointwise && d > eb) ++over;
+    const long long db = __double_as_longlong(d);
+    if (db <= inf) {
+      mxb = db > mxb ? db : mxb;
+      over += db > ebb ? 1ull : 0ull;
+    }
     se = fma(d, d, se);
     sx = fma(x, x, sx);
   }
   for (int o = 16; o > 0; o >>= 1) {
-    mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const long long m2 = __shfl_xor_sync(0xffffffffu, mxb, o);
+    mxb = m2 > mxb ? m2 : mxb;
     se += __shfl_xor_sync(0xffffffffu, se, o);
     sx += __shfl_xor_sync(0xffffffffu, sx, o);
     over += __shfl_xor_sync(0xffffffffu, over, o);
   }
+  const double mx = __longlong_as_double(mxb);
   if ((threadIdx.x & 31) == 0) {
     unsigned long long* u = reinterpret_cast<unsigned long long*>(acc + 16 * v);
     atomicMax(&u[0], dkey(mx));
@@ -797,96 +858,172 @@ __global__ void __launch_bounds__(256) k_verify_points(Plan P, const T* __restri
 
 // float32 fields: the same report with the FP64 pipe kept for what needs it.
 // A point's difference is s = fl32(x - y) and its rounding error e (TwoSum,
-// s + e = x - y exactly); the bound test decides in FP32 outside a relative
-// 2^-20 band around eb and in FP64 inside it; the maximum is taken in FP64 on
-// the points whose |s| reaches the thread's running maximum (rounding is
-// monotone, so the point of the largest |x - y| is among them); the sums of
-// squares run as unevaluated float pairs (x^2 = p + fma(x, x, -p) exactly,
-// d^2 = s^2 + 2 s e to within e^2 <= 2^-48 s^2) per batch of 1024 points of a
-// thread, each batch then added in FP64.  Values beyond 2^60 take the FP64
-// path.  Loads are float4 when the field allows (4 | K, 16-byte pointers).
-__device__ __forceinline__ void ff_add(float& hi, float& lo, float a, float ae) {
-  const float s = __fadd_rn(hi, a);
-  const float bb = __fsub_rn(s, hi);
-  const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(a, bb));
-  hi = s;
-  lo = __fadd_rn(lo, __fadd_rn(err, ae));
+// s + e = x - y exactly).  A point is looked at one by one, in FP64, only when
+// |s| reaches the thread's running maximum (rounding is monotone, so the point
+// of the largest |x - y| is among them) or the bound less a relative 2^-20, or
+// is not finite: one test for four points.  The sums of squares run as
+// unevaluated float pairs (x^2 = p + fma(x, x, -p) exactly, d^2 = s^2 + 2 s e
+// to within e^2 <= 2^-48 s^2), two points an instruction (packed FP32), per
+// batch of 1024 points of a thread; each batch is added in FP64, and one whose
+// pairs overflowed is summed again in FP64.  Loads are float4 when the field
+// allows (4 | K, 16-byte pointers).  Bound by the issue slots (about 20
+// instructions a point; scalar FP32 with a branch a point took twice that):
+// two fields of 1 GiB 0.74 -> 0.49 ms, the records' pass included.
+struct FF2 {
+  float2 hi, lo;
+};
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+__device__ __forceinline__ void ff2_add(FF2& f, float2 a, float2 ae) {
+  const float2 s = __fadd2_rn(f.hi, a);
+  const float2 bb = sub2(s, f.hi);
+  const float2 err = __fadd2_rn(sub2(f.hi, sub2(s, bb)), sub2(a, bb));
+  f.hi = s;
+  f.lo = __fadd2_rn(f.lo, __fadd2_rn(err, ae));
+}
+// a^2 + 2 a e into f
+__device__ __forceinline__ void ff2_square(FF2& f, float2 a, float2 two_a, float2 e) {
+  const float2 p = __fmul2_rn(a, a);
+  const float2 np = __fmul2_rn(p, make_float2(-1.0f, -1.0f));
+  ff2_add(f, p, __ffma2_rn(two_a, e, __ffma2_rn(a, a, np)));
+}
+__device__ __forceinline__ void ff2_square(FF2& f, float2 a) {
+  const float2 p = __fmul2_rn(a, a);
+  const float2 np = __fmul2_rn(p, make_float2(-1.0f, -1.0f));
+  ff2_add(f, p, __ffma2_rn(a, a, np));
+}
+__device__ __forceinline__ float max_nan(float a, float b) {     // a NaN when either is one
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
 }
 
-// The FP64 work of a point, out of line so that it runs only when taken
-// (inlined, it would be predicated and issued for every point).
-__device__ __noinline__ double fp64_diff(float x, float y) { return fabs((double)x - (double)y); }
+// A thread's state that rarely changes, and its (out of line) look at one point.
+struct VerRare {
+  double mx, eb;
+  unsigned long long over;
+  float mx32, eb_lo, eb_hi;
+  bool pointwise;
+};
+__device__ __noinline__ void verify_point(VerRare& V, float x, float y) {
+  const float ad = fabsf(__fsub_rn(x, y));
+  const bool plain = ad < 0x1p60f, top = !plain || ad >= V.mx32;
+  const bool edge = V.pointwise && (!plain || (ad >= V.eb_lo && !(ad > V.eb_hi)));
+  if (V.pointwise && plain && ad > V.eb_hi) ++V.over;
+  if (!(top || edge)) return;
+  const double d = fabs((double)x - (double)y);
+  if (top) V.mx = fmax(V.mx, d);
+  if (ad > V.mx32) V.mx32 = ad;
+  if (edge && d > V.eb) ++V.over;
+}
+__device__ __noinline__ void verify_sums_fp64(const float* __restrict__ a, const float* __restrict__ b, int64_t i, int64_t n,
+                                              int64_t stride, int width, double* se, double* sx) {
+  for (int64_t k = 0; k < n; ++k, i += stride)
+    for (int c = 0; c < width; ++c) {
+      const double x = (double)a[i * width + c], y = (double)b[i * width + c], d = fabs(x - y);
+      *se = fma(d, d, *se);
+      *sx = fma(x, x, *sx);
+    }
+}
 
 __global__ void __launch_bounds__(256) k_verify_points_f32(Plan P, const float* __restrict__ a,
                                                            const float* __restrict__ b, const uint8_t* comp,
-                                                           double* acc, int vec4) {
+                                                           unsigned long long comp_bytes, double* acc, int vec4) {
   const int v = blockIdx.y;
-  const double eb = reinterpret_cast<const double*>(comp + kHdr + kVarRec * v)[1];
-  const bool pointwise = P.eb_type != DLS_EB_NRMSE;
-  const float eb_lo = __double2float_rd(eb * (1.0 - 0x1p-20)), eb_hi = __double2float_ru(eb * (1.0 + 0x1p-20));
-  const float big = 0x1p60f;
-  double mx = 0.0, se = 0.0, sx = 0.0;
-  float mx32 = 0.0f;
-  unsigned long long over = 0;
-  float eh = 0.0f, el = 0.0f, xh = 0.0f, xl = 0.0f;
-  auto point = [&](float x, float y) {
-    const float sd = __fsub_rn(x, y);
-    const float bb = __fsub_rn(sd, x);
-    const float e = __fadd_rn(__fsub_rn(x, __fsub_rn(sd, bb)), __fsub_rn(-y, bb));
-    const float ad = fabsf(sd);
-    if (!(fabsf(x) < big) || !(fabsf(y) < big) || !(ad < big)) {
-      // far out of range (or not finite): this point in FP64
-      const double d = fp64_diff(x, y);
-      mx = fmax(mx, d);
-      if (pointwise && d > eb) ++over;
-      se = fma(d, d, se);
-      sx = fma((double)x, (double)x, sx);
-      return;
-    }
-    if (ad >= mx32 && ad > 0.0f) {
-      mx32 = ad;
-      mx = fmax(mx, fp64_diff(x, y));
-    }
-    if (pointwise) {
-      if (ad > eb_hi) ++over;
-      else if (ad >= eb_lo && fp64_diff(x, y) > eb) ++over;
-    }
-    const float p = __fmul_rn(sd, sd);
-    ff_add(eh, el, p, __fmaf_rn(__fmul_rn(2.0f, sd), e, __fmaf_rn(sd, sd, -p)));
-    const float q = __fmul_rn(x, x);
-    ff_add(xh, xl, q, __fmaf_rn(x, x, -q));
+  if (v == P.nvars) {
+    verify_stream(P, comp, comp_bytes, 4, acc);
+    return;
+  }
+  VerRare V;
+  V.eb = reinterpret_cast<const double*>(comp + kHdr + kVarRec * v)[1];
+  V.pointwise = P.eb_type != DLS_EB_NRMSE;
+  V.mx = 0.0;
+  V.over = 0;
+  V.mx32 = 0.0f;
+  // |s| below this needs no look: below the bound with room for the roundings, and below the maximum so far
+  const float eb_lo = V.pointwise ? __double2float_rd(V.eb * (1.0 - 0x1p-20)) : INFINITY;
+  V.eb_lo = eb_lo;
+  V.eb_hi = __double2float_ru(V.eb * (1.0 + 0x1p-20));
+  float thr = 0.0f;
+  double se = 0.0, sx = 0.0;
+  const float2 zero = make_float2(0.0f, 0.0f);
+  FF2 fe{zero, zero}, fx{zero, zero};
+  auto pair = [&](float2 x, float2 y) -> float2 {
+    const float2 s = sub2(x, y);
+    const float2 bb = sub2(s, x);
+    const float2 e = sub2(sub2(x, sub2(s, bb)), __fadd2_rn(y, bb));
+    ff2_square(fe, s, __fadd2_rn(s, s), e);
+    ff2_square(fx, x);
+    return s;
   };
-  auto flush = [&]() {
-    se += (double)eh + (double)el;
-    sx += (double)xh + (double)xl;
-    eh = el = xh = xl = 0.0f;
+  auto flush = [&](const float* a0, const float* b0, int64_t i, int64_t n, int64_t stride, int width) {
+    const float h = (fe.hi.x + fe.hi.y) + (fx.hi.x + fx.hi.y) + (fe.lo.x + fe.lo.y) + (fx.lo.x + fx.lo.y);
+    if (fabsf(h) < 3.0e38f) {
+      se += ((double)fe.hi.x + (double)fe.lo.x) + ((double)fe.hi.y + (double)fe.lo.y);
+      sx += ((double)fx.hi.x + (double)fx.lo.x) + ((double)fx.hi.y + (double)fx.lo.y);
+    } else {
+      verify_sums_fp64(a0, b0, i, n, stride, width, &se, &sx);
+    }
+    fe = FF2{zero, zero};
+    fx = FF2{zero, zero};
   };
   const int64_t base = (int64_t)v * P.K;
   const int64_t stride = (int64_t)gridDim.x * 256;
   if (vec4) {
-    // four points a load; batches of 256 loads (1024 points) per float pair
+    // four points a load; batches of 256 loads (1024 points)
     const float4* a4 = reinterpret_cast<const float4*>(a + base);
     const float4* b4 = reinterpret_cast<const float4*>(b + base);
     const int64_t K4 = P.K / 4;
     int64_t i = blockIdx.x * 256ll + threadIdx.x;
-    while (i < K4) {
-#pragma unroll 4
-      for (int n = 0; n < 256 && i < K4; ++n, i += stride) {
-        const float4 x = a4[i], y = b4[i];
-        point(x.x, y.x);
-        point(x.y, y.y);
-        point(x.z, y.z);
-        point(x.w, y.w);
+    auto four = [&](const float4& x, const float4& y) {
+      const float2 s0 = pair(make_float2(x.x, x.y), make_float2(y.x, y.y));
+      const float2 s1 = pair(make_float2(x.z, x.w), make_float2(y.z, y.w));
+      const float m = max_nan(max_nan(fabsf(s0.x), fabsf(s0.y)), max_nan(fabsf(s1.x), fabsf(s1.y)));
+      if (!(m < thr) && m != 0.0f) {
+        verify_point(V, x.x, y.x);
+        verify_point(V, x.y, y.y);
+        verify_point(V, x.z, y.z);
+        verify_point(V, x.w, y.w);
+        thr = fminf(V.mx32, eb_lo);
       }
-      flush();
+    };
+    while (i < K4) {
+      const int64_t i0 = i;
+      int n = 0;
+      for (; n < 256 && i + 3 * stride < K4; n += 4, i += 4 * stride) {
+        float4 x[4], y[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { x[k] = __ldcs(a4 + i + k * stride); y[k] = __ldcs(b4 + i + k * stride); }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) four(x[k], y[k]);
+      }
+      if (n < 256)
+        for (; i < K4; ++n, i += stride) four(a4[i], b4[i]);
+      flush(a + base, b + base, i0, n, stride, 4);
     }
   } else {
     int64_t i = blockIdx.x * 256ll + threadIdx.x;
     while (i < P.K) {
-      for (int n = 0; n < 1024 && i < P.K; ++n, i += stride) point(a[base + i], b[base + i]);
-      flush();
+      const int64_t i0 = i;
+      int n = 0;
+      for (; n < 1024 && i < P.K; n += 2, i += 2 * stride) {
+        // (a missing second point is a pair of zeros)
+        const bool two = i + stride < P.K;
+        const float2 x = make_float2(a[base + i], two ? a[base + i + stride] : 0.0f);
+        const float2 y = make_float2(b[base + i], two ? b[base + i + stride] : 0.0f);
+        const float2 s = pair(x, y);
+        const float m = max_nan(fabsf(s.x), fabsf(s.y));
+        if (!(m < thr) && m != 0.0f) {
+          verify_point(V, x.x, y.x);
+          if (two) verify_point(V, x.y, y.y);
+          thr = fminf(V.mx32, eb_lo);
+        }
+      }
+      const int64_t left = (P.K - i0 + stride - 1) / stride;
+      flush(a + base, b + base, i0, n < left ? n : left, stride, 1);
     }
   }
+  double mx = V.mx;
+  unsigned long long over = V.over;
   for (int o = 16; o > 0; o >>= 1) {
     mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     se += __shfl_xor_sync(0xffffffffu, se, o);
@@ -900,36 +1037,6 @@ __global__ void __launch_bounds__(256) k_verify_points_f32(Plan P, const float* 
     atomicAdd(&acc[16 * v + 2], se);
     atomicAdd(&acc[16 * v + 3], sx);
   }
-}
-
-__global__ void k_verify_stream(Plan P, const uint8_t* comp, unsigned long long comp_bytes, int es, double* acc) {
-  const int64_t bi = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (bi >= P.nb) return;
-  const Geom g = block_geom(P, P.b0 + bi);
-  const uint64_t* offs = reinterpret_cast<const uint64_t*>(comp + P.offsets_pos);
-  const uint64_t o0 = offs[bi], o1 = offs[bi + 1];
-  if (o1 < o0 + 16 || (uint64_t)P.payload_pos + o1 > comp_bytes || (o0 & 15) != 0) return;
-  const uint8_t* rec = comp + P.payload_pos + o0;
-  const uint32_t* rec32 = reinterpret_cast<const uint32_t*>(rec);
-  double* t = acc + 16 * P.nvars;
-  const int r = rec[0], flags = rec[1];
-  if (!(flags & kFlagRaw) && (r > kMaxN || 16 + align_up(r, 8) > (int64_t)(o1 - o0))) return;
-  if (flags & kFlagRaw) {
-    atomicAdd(&t[0], 1.0);
-    atomicAdd(&t[8], (double)rec32[3]);
-    return;
-  }
-  RecLayout lay = rec_layout(r, g.n, g.L, g.N, es, rec + 16, rec[2], rec[3], rec32[1], rec32[2]);
-  if ((flags & kFlagRice) && lay.off_c + 4 <= (int64_t)(o1 - o0))
-    lay = rice_layout(lay, g.N, reinterpret_cast<const uint32_t*>(rec + lay.off_c)[0], rec32[2], es);
-  atomicAdd(&t[1], (double)r);
-  atomicAdd(&t[2], (double)rec32[1]);
-  atomicAdd(&t[3], (double)rec32[2]);
-  atomicAdd(&t[4], (double)(lay.off_q - lay.off_v));
-  atomicAdd(&t[5], (double)(lay.off_c - lay.off_q));
-  atomicAdd(&t[6], (double)(lay.off_ei - lay.off_c));
-  atomicAdd(&t[7], (double)(lay.size - lay.off_ei));
-  atomicAdd(&t[9], (double)lay.off_v);
 }
 
 }  // namespace
@@ -969,15 +1076,20 @@ int launch_decode(const Plan& p, const void* d_comp, unsigned long long comp_byt
 
 int launch_verify(const Plan& p, const void* d_orig, const void* d_recon, const void* d_comp,
                   unsigned long long comp_bytes, double* acc, cudaStream_t s) {
-  dim3 grid(1024, p.nvars);
+  // the points' CTAs, all resident at once (each a few batches), and a row for the stream's records
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return DLS_ERR_CUDA;
+  const int64_t want = cdiv(p.K, 4096), most = (int64_t)sms * 8;
+  const dim3 grid((unsigned)(want < 1 ? 1 : want < most ? want : most), (unsigned)p.nvars + 1);
   if (p.dtype == DLS_F32)
-    k_verify_points_f32<<<grid, 256, 0, s>>>(p, (const float*)d_orig, (const float*)d_recon, (const uint8_t*)d_comp, acc,
+    k_verify_points_f32<<<grid, 256, 0, s>>>(p, (const float*)d_orig, (const float*)d_recon, (const uint8_t*)d_comp,
+                                             comp_bytes, acc,
                                              (p.K % 4 == 0 && ((uintptr_t)d_orig & 15) == 0 &&
                                               ((uintptr_t)d_recon & 15) == 0) ? 1 : 0);
   else
-    k_verify_points<double><<<grid, 256, 0, s>>>(p, (const double*)d_orig, (const double*)d_recon, (const uint8_t*)d_comp, acc);
-  if (p.nb > 0)
-    k_verify_stream<<<(unsigned)cdiv(p.nb, 256), 256, 0, s>>>(p, (const uint8_t*)d_comp, comp_bytes, p.dtype == DLS_F32 ? 4 : 8, acc);
+    k_verify_points<double><<<grid, 256, 0, s>>>(p, (const double*)d_orig, (const double*)d_recon, (const uint8_t*)d_comp,
+                                                 comp_bytes, acc);
   return cudaGetLastError() == cudaSuccess ? DLS_OK : DLS_ERR_CUDA;
 }
 
