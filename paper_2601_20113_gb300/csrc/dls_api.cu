@@ -1,6 +1,7 @@
 // Host side of the C ABI: parameter validation, block plan, workspace layout,
 // launch sequence and status readback.  See include/dls.h for the contract.
 #include <atomic>
+#include <mutex>
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -263,7 +264,20 @@ static int upload_basis(const dls_params* p, const Plan& P, const Layout& L, voi
 static int64_t bound_bytes(const Plan& P) {
   int64_t tot = P.payload_pos;
   const int es = esize(P.dtype);
-  // records of blocks sharing a shape have equal bounds: sum per block
+  if (P.b0 == 0 && P.nb == P.nb_total) {
+    // the whole field: on each axis whole blocks and at most one edge, so at
+    // most 16 shapes (a sum over 34 560 blocks took longer than some launches)
+    for (int c = 0; c < 16; ++c) {
+      int64_t cnt = P.nvars, N = 1;
+      for (int a = 0; a < 4; ++a) {
+        const int64_t edge = P.dims[a] % P.block[a];
+        cnt *= (c >> a & 1) ? (edge ? 1 : 0) : P.dims[a] / P.block[a];
+        N *= (c >> a & 1) ? edge : P.block[a];
+      }
+      if (cnt > 0) tot += cnt * raw_record_bytes(N, es);
+    }
+    return tot;
+  }
   for (int64_t b = 0; b < P.nb; ++b) tot += raw_record_bytes(block_geom(P, P.b0 + b).N, es);
   return tot;
 }
@@ -272,6 +286,41 @@ static int64_t bound_bytes(const Plan& P) {
   do {                                         \
     if ((x) != cudaSuccess) return DLS_ERR_CUDA; \
   } while (0)
+
+// Small stream-ordered device scratch (a status block, report sums).  The
+// default pool hands its pages back at every synchronisation, so that each
+// call paid for mapping and unmapping them (90 and 75 us of a decompression or
+// a verification); a pool of the library's own, one a device, keeps what it
+// has mapped up to 64 MiB (in practice one chunk: the requests are a few KB).
+// Safe from any thread and stream, as the allocator is.
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+  constexpr int kMaxDev = 64;
+  static std::once_flag once[kMaxDev];
+  static cudaMemPool_t pool[kMaxDev];
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 0 && dev < kMaxDev) {
+    std::call_once(once[dev], [dev] {
+      cudaMemPoolProps props;
+      memset(&props, 0, sizeof(props));
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      cudaMemPool_t m = nullptr;
+      uint64_t keep = 64u << 20;
+      if (cudaMemPoolCreate(&m, &props) == cudaSuccess &&
+          cudaMemPoolSetAttribute(m, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+        pool[dev] = m;
+      cudaGetLastError();
+    });
+    if (pool[dev]) {
+      if (cudaMallocFromPoolAsync(p, bytes, pool[dev], s) == cudaSuccess) return cudaSuccess;
+      cudaGetLastError();
+    }
+  }
+  return cudaMallocAsync(p, bytes, s);
+}
 
 struct HostHeader {
   dls_params p;
@@ -283,8 +332,10 @@ struct HostHeader {
 // Reads and validates a stream header from device memory.
 static int read_header(const void* d_comp, size_t comp_bytes, cudaStream_t s, HostHeader* h, Plan* P) {
   if (!d_comp || comp_bytes < (size_t)kHdr || ((uintptr_t)d_comp & 15)) return DLS_ERR_INVALID_ARG;
-  uint8_t hdr[kHdr];
-  CK(cudaMemcpyAsync(hdr, d_comp, kHdr, cudaMemcpyDeviceToHost, s));
+  // header and variable table in one copy (as much of a full table as the stream holds)
+  alignas(16) uint8_t hdr[kHdr + kVarRec * kMaxVars];
+  const size_t got = comp_bytes < sizeof(hdr) ? comp_bytes : sizeof(hdr);
+  CK(cudaMemcpyAsync(hdr, d_comp, got, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   uint32_t u32[32];
   uint64_t u64[16];
@@ -294,9 +345,8 @@ static int read_header(const void* d_comp, size_t comp_bytes, cudaStream_t s, Ho
   const int nvars = (int)u32[3];
   if (nvars < 1 || nvars > kMaxVars) return DLS_ERR_CORRUPT;
   if ((size_t)(kHdr + kVarRec * nvars) > comp_bytes) return DLS_ERR_CORRUPT;
-  std::vector<double> vt(4 * (size_t)nvars);
-  CK(cudaMemcpyAsync(vt.data(), (const uint8_t*)d_comp + kHdr, kVarRec * (size_t)nvars, cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+  double vt[4 * kMaxVars];
+  memcpy(vt, hdr + kHdr, kVarRec * (size_t)nvars);
   memset(h, 0, sizeof(*h));
   for (int v = 0; v < nvars; ++v) {
     h->eb_user[v] = vt[4 * v + 0];
@@ -663,7 +713,7 @@ int dls_decompress(const void* d_comp, size_t comp_bytes, void* d_out, size_t ou
   if (!d_out || ((uintptr_t)d_out & (esize(P.dtype) - 1))) return DLS_ERR_INVALID_ARG;
   if (out_cap < (size_t)(P.K * P.nvars * esize(P.dtype))) return DLS_ERR_CAPACITY;
   Status* dst = nullptr;
-  CK(cudaMallocAsync((void**)&dst, sizeof(Status), s));
+  CK(scratch_alloc((void**)&dst, sizeof(Status), s));
   CK(cudaMemsetAsync(dst, 0, sizeof(Status), s));
   st = launch_decode(P, d_comp, (unsigned long long)comp_bytes, d_out, dst, s);
   Status hs;
@@ -1022,7 +1072,7 @@ int dls_verify(const void* d_orig, const void* d_recon, const void* d_comp, size
   if (st != DLS_OK) return st;
   const size_t nacc = 16 * (size_t)P.nvars + 16;
   double* acc = nullptr;
-  CK(cudaMallocAsync((void**)&acc, nacc * sizeof(double), s));
+  CK(scratch_alloc((void**)&acc, nacc * sizeof(double), s));
   CK(cudaMemsetAsync(acc, 0, nacc * sizeof(double), s));
   st = launch_verify(P, d_orig, d_recon, d_comp, (unsigned long long)comp_bytes, acc, s);
   std::vector<double> ha(nacc);

@@ -289,6 +289,9 @@ int make_plan(const dls_params* p, Plan* out);
 // first staged chunk the per-block kernel never copies; -1 for none.
 int64_t fault_withheld_block();
 
+// Small stream-ordered device allocation (freed with cudaFreeAsync): dls_api.cu.
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+
 // ---------------------------------------------------------------- launchers (defined in .cu files)
 int launch_mixed_compress(const Plan& p, const void* d_in, const MixedWork& w, int learned, int variant,
                           int spatial_only, cudaStream_t s);

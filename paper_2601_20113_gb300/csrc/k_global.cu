@@ -1111,7 +1111,7 @@ int dls_gb_decompress(const void* d_comp, size_t comp_bytes, double* d_out, size
     return DLS_ERR_CUDA;
   if (first != 0 || (uint64_t)g.payload_pos + last != (uint64_t)comp_bytes) return DLS_ERR_CORRUPT;
   GbStatus* gs = nullptr;
-  if (cudaMallocAsync((void**)&gs, sizeof(GbStatus), s) != cudaSuccess) return DLS_ERR_CUDA;
+  if (scratch_alloc((void**)&gs, sizeof(GbStatus), s) != cudaSuccess) return DLS_ERR_CUDA;
   if (cudaMemsetAsync(gs, 0, sizeof(GbStatus), s) != cudaSuccess) {
     cudaFreeAsync(gs, s);
     return DLS_ERR_CUDA;

@@ -2824,6 +2824,29 @@ size_t tile_smem_bytes(bool tc) {
 // Dynamic shared memory of k_eig: the shared struct up to the staging ring.
 size_t eig_smem_bytes() { return 1024 + (size_t)offsetof(TileSmem, ring); }
 
+// The device's per-SM limits, read once a device (cudaGetDeviceProperties
+// fills in far more and took tens of microseconds at every launch).
+struct SmLimits {
+  int regs, smem, reserved, threads, blocks;
+  bool ok;
+};
+static const SmLimits* sm_limits() {
+  constexpr int kMaxDev = 64;
+  static std::once_flag once[kMaxDev];
+  static SmLimits lim[kMaxDev];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return nullptr;
+  std::call_once(once[dev], [dev] {
+    SmLimits& l = lim[dev];
+    l.ok = cudaDeviceGetAttribute(&l.regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&l.smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&l.reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&l.threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&l.blocks, cudaDevAttrMaxBlocksPerMultiprocessor, dev) == cudaSuccess;
+  });
+  return lim[dev].ok ? &lim[dev] : nullptr;
+}
+
 // Resident CTAs per SM from the kernel's registers and shared memory and the
 // device's per-SM limits (and, with the tensor-core Gram, the TMEM columns).
 // Computed here because the occupancy query treats a kernel that contains
@@ -2832,20 +2855,16 @@ template <class K>
 int ctas_per_sm_of(K kernel, size_t smem, bool tc) {
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   cudaFuncAttributes fa;
-  int dev = 0;
-  cudaDeviceProp prop;
-  if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
-      cudaGetDeviceProperties(&prop, dev) != cudaSuccess)
-    return 0;
+  const SmLimits* lim = sm_limits();
+  if (!lim || cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return 0;
   // registers are allocated per warp in units of 256
   const int regs_warp = (int)align_up((int64_t)fa.numRegs * 32, 256);
-  const int by_regs = prop.regsPerMultiprocessor / (regs_warp * (kTT / 32));
-  const int by_smem = (int)(prop.sharedMemPerMultiprocessor /
-                            (smem + (size_t)fa.sharedSizeBytes + prop.reservedSharedMemPerBlock));
-  const int by_threads = prop.maxThreadsPerMultiProcessor / kTT;
+  const int by_regs = lim->regs / (regs_warp * (kTT / 32));
+  const int by_smem = (int)(lim->smem / (smem + (size_t)fa.sharedSizeBytes + lim->reserved));
+  const int by_threads = lim->threads / kTT;
   int n = by_regs < by_smem ? by_regs : by_smem;
   n = n < by_threads ? n : by_threads;
-  n = n < prop.maxBlocksPerMultiProcessor ? n : prop.maxBlocksPerMultiProcessor;
+  n = n < lim->blocks ? n : lim->blocks;
   if (tc) n = n < (int)(512 / kTmemCols) ? n : (int)(512 / kTmemCols);
   return n;
 }
