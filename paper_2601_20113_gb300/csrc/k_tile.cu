@@ -1246,6 +1246,277 @@ __device__ __noinline__ bool pass_encode(const TileArgs& a, const Maps& tm, Tile
   return true;
 }
 
+// ---------------------------------------------------------------- k_enc's row pass
+// Rows of a chunk in block order: row i of the chunk is block row lbase + i
+// (x fastest; a chunk is whole planes, or lines of one plane).
+struct ChunkRows {
+  int lbase, count, ys;
+};
+__device__ __forceinline__ ChunkRows chunk_rows(const TileArgs& a, const Geom& g, const Chunks& ch, int c) {
+  ChunkRows r;
+  const int cz = c / ch.ncy, z0 = cz * a.zc, y0 = (c - cz * ch.ncy) * a.yc;
+  r.ys = g.sy - y0 < a.yc ? g.sy - y0 : a.yc;
+  const int zs = g.sz - z0 < a.zc ? g.sz - z0 : a.zc;
+  r.lbase = (z0 * g.sy + y0) * g.sx;
+  r.count = g.sx * r.ys * zs;
+  return r;
+}
+
+// Projection, quantization and decode at rank r with FP32 estimates of E(r-1)
+// and E(r) (S.Ered[0], [1]) and, POINT, the corrections: q and k8 into the
+// block's slot, the nonzero-correction bitmap into S.bitsm; blocks of at most
+// 32 kBitsSmem points with 1 to NP time steps.  One row a thread.
+// Every correction of a row is worked out, two a packed instruction, without a
+// branch: y = R / 2eb, k = rint(y) by adding 1.5 x 2^23 (k is then the low
+// byte of that sum, ready to store), xt = k 2eb + xhat.  A row is settled when
+// every |y - k| is clear of 1/2, every |x - xt| of the bound, by more than
+// their roundings (|k| <= 59 bounds the first), else its elements go one by one
+// through corr_decide.  A ballot a column is one word of the bitmap, and each
+// warp writes whole 32-byte sectors of k8.
+// MC = 4096: the 16 x 16 x 16 x 16 block (chunks of 256 rows, every row and
+// offset known); 0: any shape, by row arithmetic and, where a column's rows do
+// not start on a word of the bitmap, by OR-ing shifted words.
+// Bound by its instructions and their latencies at 16 warps an SM: 700 warp
+// instructions a 32 rows at rank 3, 30.4 of 32 lanes active (1001 and 22.4 with
+// a per-lane loop over the corrections' candidates, a select chain each).
+// 128 blocks of 16^3 x 16: 100 -> 70 us; 16 384: 2.65 -> 2.51 ms; 4096 at rank
+// 7: 1.19 -> 0.96 ms.
+constexpr float kMagicF = 12582912.0f;              // 1.5 x 2^23
+constexpr int kMagicI = 0x4B400000;                 // its bits
+constexpr int kFastK = 59;
+template <int NP, bool POINT, int MC>
+__device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
+                                       const Geom& g, int r, const RowConst& rcst, const CorrConst& cc,
+                                       int32_t* __restrict__ qs, int8_t* __restrict__ k8, int32_t* __restrict__ k32) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = MC ? NP : g.n, M = MC ? MC : (int)g.M, rc = MC ? 256 : a.rc;
+  const RowConst rq = rcst;
+  const CorrConst cq = cc;
+  const int Lq = MC ? MC : (int)align_up(g.L, 4);
+  const Chunks ch0 = chunks_of(a, g);
+  // every chunk starts on a multiple of 32 rows, in every column
+  const bool words = MC || ((M & 31) == 0 && (chunk_rows(a, g, ch0, 0).count & 31) == 0 &&
+                            (ch0.ncy == 1 || (g.sx * g.sy & 31) == 0));
+  if (tid == 0) { S.kmax = 0; S.ncorr = 0; S.nesc = 0; S.nesc_slot = 0; }
+  if (POINT && !words)
+    for (int i = tid; i < (n * M + 31) / 32; i += kTT) S.bitsm[i] = 0u;
+  __syncthreads();
+  const float2 m1 = make_float2(-1.0f, -1.0f), mg = make_float2(kMagicF, kMagicF), nmg = make_float2(-kMagicF, -kMagicF);
+  const float2 inv2 = make_float2(cq.inv_step_f, cq.inv_step_f), step2 = make_float2(cq.step_f, cq.step_f);
+  float2 e1 = make_float2(0.0f, 0.0f), e2 = make_float2(0.0f, 0.0f);
+  uint32_t qor_lane = 0, kmx = 0;
+  int nc = 0, ne = 0, ovf = 0, zmx = kMagicI, zmn = kMagicI;
+  const uint32_t msx = MC ? 0u : (g.sx > 1 ? 0xFFFFFFFFu / (uint32_t)g.sx + 1u : 0u);
+  const bool ok = stream_block(a, tm, S, cu, bi, g, kLayoutRow, [&](int c, const Chunks& ch, const float* tile) {
+    ChunkRows cr;
+    uint32_t mys = 0;
+    if (MC) {
+      cr.lbase = c * 256;
+      cr.count = 256;
+      cr.ys = 16;
+    } else {
+      cr = chunk_rows(a, g, ch, c);
+      mys = cr.ys > 1 ? 0xFFFFFFFFu / (uint32_t)cr.ys + 1u : 0u;
+    }
+#pragma unroll 1
+    for (int rb = 0; rb < cr.count; rb += kTT) {        // same trip count in every lane
+      const int i = rb + tid, l = cr.lbase + i;
+      const bool valid = MC ? true : i < cr.count;
+      int rr = i;
+      if (!MC) {
+        // (x, y, z) in the chunk, and the row of its tile; invalid lanes take zeros and store nothing
+        const int t = fdiv(i, msx), x = i - t * g.sx, zl = fdiv(t, mys), yl = t - zl * cr.ys;
+        rr = valid ? (zl * a.yc + yl) * a.bxb + x : 0;
+      }
+      float x[NP], d[NP], acc[NP];
+#pragma unroll
+      for (int j = 0; j < NP; ++j) {
+        x[j] = (MC || (valid && j < n)) ? tile[j * rc + rr] : 0.0f;
+        acc[j] = 0.0f;
+      }
+      const float a0 = x[0];
+#pragma unroll
+      for (int j = 0; j < NP; j += 2) {
+        // (time steps past the block's stay zero: their modes are)
+        const float2 t = __ffma2_rn(make_float2(a0, a0), m1, make_float2(x[j], x[j + 1]));
+        d[j] = t.x;
+        d[j + 1] = t.y;
+      }
+#pragma unroll 1
+      for (int k = 0; k < r; ++k) {
+        float v[NP];
+        const float4* vp = reinterpret_cast<const float4*>(&S.VstT[k * NM]);
+#pragma unroll
+        for (int j4 = 0; j4 < NP / 4; ++j4) {
+          const float4 t = vp[j4];
+          v[4 * j4 + 0] = t.x; v[4 * j4 + 1] = t.y; v[4 * j4 + 2] = t.z; v[4 * j4 + 3] = t.w;
+        }
+        // the coefficient as every pass forms it (project): partial sums j mod 4
+        float2 s01 = make_float2(0.0f, 0.0f), s23 = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int j4 = 0; j4 < NP / 4; ++j4) {
+          s01 = __ffma2_rn(make_float2(d[4 * j4 + 0], d[4 * j4 + 1]), make_float2(v[4 * j4 + 0], v[4 * j4 + 1]), s01);
+          s23 = __ffma2_rn(make_float2(d[4 * j4 + 2], d[4 * j4 + 3]), make_float2(v[4 * j4 + 2], v[4 * j4 + 3]), s23);
+        }
+        const float cf = __fmaf_rn(a0, S.vsum[k], __fadd_rn(__fadd_rn(s01.x, s01.y), __fadd_rn(s23.x, s23.y)));
+        // quant_exact with the rounding by kMagicF (|y| below 2^22)
+        const float y = __fmul_rn(cf, rq.inv_delta);
+        const float z = __fadd_rn(y, kMagicF);
+        float rq_f = __fsub_rn(z, kMagicF);
+        int32_t q = __float_as_int(z) - kMagicI;
+        if (!(fabsf(__fsub_rn(y, rq_f)) < 0.5f - __fmaf_rn(fabsf(y), 4.0e-7f, 1.0e-30f) && fabsf(y) < 4.0e6f)) {
+          q = quant_fp64(cf, rq.delta, &ovf);
+          rq_f = __int2float_rn(q);
+        }
+        if (valid) qs[k * Lq + l] = q;
+        const uint32_t wor = __reduce_or_sync(FULL, valid ? zigzag(q) : 0u);
+        if (lane == k) qor_lane |= wor;
+        const float chk = __fmul_rn(rq_f, rq.delta_f);
+        if (k == r - 1) {
+#pragma unroll
+          for (int j = 0; j < NP; j += 2) {
+            const float2 t = __ffma2_rn(make_float2(acc[j], acc[j + 1]), m1, make_float2(x[j], x[j + 1]));
+            e1 = __ffma2_rn(t, t, e1);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < NP; j += 2) {
+          const float2 t = __ffma2_rn(make_float2(chk, chk), make_float2(v[j], v[j + 1]), make_float2(acc[j], acc[j + 1]));
+          acc[j] = t.x;
+          acc[j + 1] = t.y;
+        }
+      }
+      if (!POINT) {
+#pragma unroll
+        for (int j = 0; j < NP; j += 2) {
+          const float2 t = __ffma2_rn(make_float2(acc[j], acc[j + 1]), m1, make_float2(x[j], x[j + 1]));
+          e2 = __ffma2_rn(t, t, e2);
+        }
+        continue;
+      }
+      // corrections
+      int zi[NP];
+      bool settled = true;
+#pragma unroll
+      for (int j = 0; j < NP; j += 2) {
+        const float2 x2 = make_float2(x[j], x[j + 1]), h2 = make_float2(acc[j], acc[j + 1]);
+        const float2 R = __ffma2_rn(h2, m1, x2);
+        e2 = __ffma2_rn(R, R, e2);
+        const float2 y = __fmul2_rn(R, inv2);
+        const float2 z = __fadd2_rn(y, mg);
+        const float2 k = __fadd2_rn(z, nmg);
+        const float2 fr = __ffma2_rn(k, m1, y);
+        const float2 xt = __ffma2_rn(k, step2, h2);
+        const float2 dd = __ffma2_rn(xt, m1, x2);
+        zi[j] = __float_as_int(z.x);
+        zi[j + 1] = __float_as_int(z.y);
+        settled = settled && fabsf(fr.x) < 0.49997f && fabsf(fr.y) < 0.49997f && fabsf(dd.x) <= cq.eb_lo_f &&
+                  fabsf(dd.y) <= cq.eb_lo_f;
+      }
+      int hi = zi[0], lo = zi[0];
+#pragma unroll
+      for (int j = 1; j < NP; ++j) {
+        hi = max(hi, zi[j]);
+        lo = min(lo, zi[j]);
+      }
+      uint32_t escm = 0;
+      if (settled && hi <= kMagicI + kFastK && lo >= kMagicI - kFastK) {
+        zmx = max(zmx, hi);
+        zmn = min(zmn, lo);
+      } else {
+        // one by one, by the definition where FP32 leaves it open
+#pragma unroll 1
+        for (int jj = 0; jj < n; ++jj) {
+          float aj = acc[0], xj = x[0];
+#pragma unroll
+          for (int j = 1; j < NP; ++j) {
+            aj = j == jj ? acc[j] : aj;
+            xj = j == jj ? x[j] : xj;
+          }
+          const int32_t k = corr_decide(xj, aj, cq);
+          const bool big = k < -127 || k > 127;            // includes escapes
+          const int zb = kMagicI + (big ? -128 : k);
+          if (big && valid) k32[jj * M + l] = k;
+          if (k == kEscape) escm |= 1u << jj;
+          else kmx |= zigzag(k);
+#pragma unroll
+          for (int j = 0; j < NP; ++j) zi[j] = j == jj ? zb : zi[j];
+        }
+      }
+      uint32_t w = 0;
+      int8_t* kp = k8 + l;
+#pragma unroll
+      for (int j = 0; j < NP; ++j) {
+        if (MC || j < n) {
+          const unsigned bal = __ballot_sync(FULL, zi[j] != kMagicI);
+          w = lane == j ? bal : w;
+          if (valid) kp[j * M] = (int8_t)zi[j];
+        }
+      }
+      if (__any_sync(FULL, escm != 0u)) {
+        // rare: escapes are no corrections; listed for the deferred packer (in no particular order)
+#pragma unroll 1
+        for (int j = 0; j < n; ++j) {
+          const unsigned eb = __ballot_sync(FULL, (escm >> j) & 1u);
+          w = lane == j ? w & ~eb : w;
+        }
+        ne += __popc(escm);
+        uint32_t* const el = S.esc_list;
+        for (uint32_t em = escm; em; em &= em - 1) {
+          const int at = atomicAdd(&S.nesc_slot, 1);
+          if (el && at < S.esc_cap) el[at] = (uint32_t)((__ffs(em) - 1) * M + l);
+        }
+      }
+      nc += __popc(w);
+      if (lane < n && (w != 0u || (words && (MC || i - lane < cr.count)))) {
+        const uint32_t e0 = (uint32_t)(lane * M + (l - lane));
+        if (words) {
+          S.bitsm[e0 >> 5] = w;
+        } else {
+          const uint32_t sh = e0 & 31u;
+          atomicOr(&S.bitsm[e0 >> 5], w << sh);
+          const uint32_t up = sh ? w >> (32u - sh) : 0u;
+          if (up) atomicOr(&S.bitsm[(e0 >> 5) + 1], up);
+        }
+      }
+    }
+  });
+  if (!ok) return false;
+  kmx |= max(zigzag(zmx - kMagicI), zigzag(zmn - kMagicI));
+  nc = __reduce_add_sync(FULL, nc);
+  ne = __reduce_add_sync(FULL, ne);
+  kmx = __reduce_or_sync(FULL, kmx);
+  const unsigned ov = __ballot_sync(FULL, ovf != 0);
+  if (lane == 0) {
+    if (nc) atomicAdd(&S.ncorr, nc);
+    if (ne) atomicAdd(&S.nesc, ne);
+    if (kmx) atomicOr(reinterpret_cast<unsigned int*>(&S.kmax), kmx);
+    if (ov) S.ovf = 1;
+  }
+  if (lane < NM) S.qor[warp][lane] = qor_lane;
+  __syncthreads();
+  if (tid < NM) {
+    uint32_t o = 0;
+    for (int w = 0; w < kWarps; ++w) o |= S.qor[w][tid];
+    S.wq[tid] = tid < r ? bit_width(o) : 0;
+  }
+  const float ev[2] = {__fadd_rn(e1.x, e1.y), __fadd_rn(e2.x, e2.y)};
+  cta_reduce(S, ev, 2);
+  return true;
+}
+
+// The row pass in the form that fits the block.
+template <bool POINT>
+__device__ __forceinline__ bool encode_rows(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
+                                            const Geom& g, int r, const RowConst& rcst, const CorrConst& cc, int32_t* qs,
+                                            int8_t* k8, int32_t* k32) {
+  if (g.n == NM && g.M == 4096 && a.rc == 256 && g.sx == a.bxb && bitmap_rows(a, g))
+    return pass_rows<NM, POINT, 4096>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32);
+  if (g.n <= 4) return pass_rows<4, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32);
+  if (g.n <= 8) return pass_rows<8, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32);
+  return pass_rows<NM, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32);
+}
+
 // E(r) for every r in [0, rcap] (FP32 estimates into S.Ered).
 template <int NF>
 __device__ __noinline__ bool pass_all_errors(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
@@ -1612,7 +1883,7 @@ __device__ __forceinline__ void pack_dense(uint32_t* cw, const int8_t* k8, const
 __device__ __forceinline__ void bitmap_list(uint32_t* list, const uint32_t* bits, int64_t N, int64_t ncorr,
                                             int* warp_cnt) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nw = (int)(N / 32);
+  const int nw = (int)cdiv(N, 32);
   const int per_w = (int)cdiv(nw, kWarps * 32) * 32;
   const int wb = warp * per_w, we = (wb + per_w) < nw ? (wb + per_w) : nw;
   int cnt = 0;
@@ -1715,25 +1986,25 @@ __device__ __forceinline__ void zero_padding(uint8_t* rec, const RecLayout& lay,
 // until k_pack_tile writes it at its stream offset.  The slot holds a raw
 // record (16 + 4 N bytes), which leaves room for all three when the rank is
 // small next to n, and for the sparse entry list after them (list_cap
-// entries).
+// entries).  Without pointwise corrections the q columns are all there is.
 struct SlotScratch {
   int64_t off_q, off_bits, off_k8, end, off_esc, esc_cap, off_list, list_cap;
   bool fits;
 };
 constexpr int kMaxSlotEsc = 1024;             // escapes a deferred record can carry
-__host__ __device__ inline SlotScratch slot_scratch(int r, int n, int64_t L, int64_t N) {
+__host__ __device__ inline SlotScratch slot_scratch(int r, int n, int64_t L, int64_t N, bool pointwise = true) {
   SlotScratch o;
   const int64_t off_pre = 16 + align_up(r, 8) + align_up((int64_t)n * r * 4, 8);   // the record's q offset
   o.off_q = align_up(off_pre, 16);
   o.off_bits = o.off_q + (int64_t)r * align_up(L, 4) * 4;
-  o.off_k8 = o.off_bits + align_up(N / 8, 16);
-  o.end = o.off_k8 + align_up(N, 16);
+  o.off_k8 = o.off_bits + (pointwise ? align_up(cdiv(N, 32) * 4, 16) : 0);
+  o.end = o.off_k8 + (pointwise ? align_up(N, 16) : 0);
   const int64_t room = o.end <= raw_record_bytes(N, 4) ? (raw_record_bytes(N, 4) - o.end) / 4 : 0;
   o.off_esc = o.end;
   o.esc_cap = room < kMaxSlotEsc ? room / 4 * 4 : kMaxSlotEsc;
   o.off_list = o.off_esc + o.esc_cap * 4;
   o.list_cap = room - o.esc_cap;
-  o.fits = r > 0 && N % 32 == 0 && N <= (int64_t)kBitsSmem * 32 && o.end <= raw_record_bytes(N, 4);
+  o.fits = r > 0 && N <= (int64_t)kBitsSmem * 32 && o.end <= raw_record_bytes(N, 4);
   return o;
 }
 constexpr int kDeferMaxWk = 7;                // deferred records have |k| < 64: no k32 values
@@ -1893,10 +2164,13 @@ __device__ __noinline__ void defer_record(const TileArgs& a, TileSmem& S, const 
     record_raw(a, S, g, slot);
     return;
   }
-  const SlotScratch sc = slot_scratch(r, g.n, g.L, g.N);
+  const bool pointwise = a.P.eb_type != DLS_EB_NRMSE;
+  const SlotScratch sc = slot_scratch(r, g.n, g.L, g.N, pointwise);
   record_prefix(S, g, slot, sc.off_q);
-  uint32_t* dst = reinterpret_cast<uint32_t*>(slot + sc.off_bits);
-  for (int64_t i = threadIdx.x; i < g.N / 32; i += kTT) dst[i] = bits[i];
+  if (pointwise) {
+    uint32_t* dst = reinterpret_cast<uint32_t*>(slot + sc.off_bits);
+    for (int i = threadIdx.x; i < (int)cdiv(g.N, 32); i += kTT) dst[i] = bits[i];
+  }
   __syncthreads();
 }
 
@@ -2374,13 +2648,13 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
   PhaseClock pc;
   Cursor cu;
   cu.iss = 0; cu.con = 0; cu.pf_blk = -1; cu.pf_cnt = 0; cu.pf_layout = kLayoutRow;
+  const bool pointwise = P.eb_type != DLS_EB_NRMSE;
   auto eligible = [&](int64_t b, int* rp_out) -> bool {
     const Geom gb = block_geom(P, P.b0 + b);
     const FastBlock& fb = a.fb[b];
     const int rp = fb.rpred;
     *rp_out = rp;
-    return !(fb.flags & (kFbNonfinite | kFbRR | kFbOverflow)) && gb.n == NM && bitmap_rows(a, gb) &&
-           gb.N <= (int64_t)kBitsSmem * 32 && slot_scratch(rp, gb.n, gb.L, gb.N).fits;
+    return !(fb.flags & (kFbNonfinite | kFbRR | kFbOverflow)) && slot_scratch(rp, gb.n, gb.L, gb.N, pointwise).fits;
   };
   auto to_list = [&](int64_t b) {
     if (threadIdx.x == 0) {
@@ -2388,7 +2662,6 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
       a.list[i] = (int32_t)b;
     }
   };
-  const bool pointwise = P.eb_type != DLS_EB_NRMSE;
   if (threadIdx.x == 0) S.bnext = grab_range(a, &a.ctl->next_enc);
   __syncthreads();
   for (;;) {
@@ -2398,7 +2671,7 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
     if (threadIdx.x == 0) S.bnext = grab_range(a, &a.ctl->next_enc);
     const Geom g = block_geom(P, P.b0 + bi);
     int rp = 0;
-    if (!pointwise || !eligible(bi, &rp)) {
+    if (!eligible(bi, &rp)) {
       if (!(a.fb[bi].flags & kFbNonfinite)) to_list(bi);
       __syncthreads();          // thread 0 has taken the next block
       continue;
@@ -2411,14 +2684,15 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
     pc.start();
     load_basis(S, a.fb[bi]);
     uint8_t* const slot = a.staging + align_up((g.pt_off - P.pt_base) * 4, 16) + 48 * bi;
-    const SlotScratch sc = slot_scratch(rp, g.n, g.L, g.N);
+    const SlotScratch sc = slot_scratch(rp, g.n, g.L, g.N, pointwise);
     if (threadIdx.x == 0) {
       S.esc_list = reinterpret_cast<uint32_t*>(slot + sc.off_esc);
       S.esc_cap = (int)sc.esc_cap;
     }
-    if (!pass_encode<NM, true>(a, tm, S, cu, bi, g, rp, true, rcst, cc, true,
-                               reinterpret_cast<int32_t*>(slot + sc.off_q), reinterpret_cast<int8_t*>(slot + sc.off_k8),
-                               k32, S.bitsm))
+    int32_t* const qs = reinterpret_cast<int32_t*>(slot + sc.off_q);
+    int8_t* const k8 = reinterpret_cast<int8_t*>(slot + sc.off_k8);
+    if (!(pointwise ? encode_rows<true>(a, tm, S, cu, bi, g, rp, rcst, cc, qs, k8, k32)
+                    : encode_rows<false>(a, tm, S, cu, bi, g, rp, rcst, cc, qs, k8, k32)))
       break;
     pc.mark(S, kPhEncode);
     bool accepted = false;
@@ -2451,7 +2725,7 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
     {
       int rn = 0;
       const int64_t bn = S.bnext;
-      if (bn < a.bhi && pointwise && eligible(bn, &rn)) prefetch(a, tm, S, cu, bn, block_geom(P, P.b0 + bn), kLayoutRow);
+      if (bn < a.bhi && eligible(bn, &rn)) prefetch(a, tm, S, cu, bn, block_geom(P, P.b0 + bn), kLayoutRow);
     }
     defer_record(a, S, g, bi, rp, S.bitsm);
     pc.mark(S, kPhPack);
@@ -2684,7 +2958,7 @@ __global__ void __launch_bounds__(kTT, 6) k_pack_tile(Plan P, const BlockMeta* m
       int sk = !(m.flags & kFlagDeferred);
       if (!sk) {
         lay = rec_layout(m.r, g.n, g.L, g.N, 4, m.wq, m.wk, m.ib, m.ncorr, m.nesc);
-        const SlotScratch sc = slot_scratch(m.r, g.n, g.L, g.N);
+        const SlotScratch sc = slot_scratch(m.r, g.n, g.L, g.N, P.eb_type != DLS_EB_NRMSE);
         // a deferred record is one the tile kernel could defer: check before use
         if (!sc.fits || lay.size != m.nbytes || m.nesc > sc.esc_cap || m.wk > kDeferMaxWk || m.r > g.n ||
             (!lay.dense && m.ncorr > sc.list_cap)) {
@@ -2702,7 +2976,7 @@ __global__ void __launch_bounds__(kTT, 6) k_pack_tile(Plan P, const BlockMeta* m
       __syncthreads();
       continue;
     }
-    const SlotScratch sc = slot_scratch(m.r, g.n, g.L, g.N);
+    const SlotScratch sc = slot_scratch(m.r, g.n, g.L, g.N, P.eb_type != DLS_EB_NRMSE);
     uint8_t* slot = staging + align_up((g.pt_off - P.pt_base) * 4, 16) + 48 * bi;
     uint8_t* rec = out + P.payload_pos + offsets[bi];
     if (tid == 0) zero_padding(rec, lay, m, g.n, colbase[m.r], m.nbytes);
@@ -2710,8 +2984,8 @@ __global__ void __launch_bounds__(kTT, 6) k_pack_tile(Plan P, const BlockMeta* m
     // the prefix (header, widths, basis; its padding zeroed) as it is
     for (int64_t i = tid; i < lay.off_q / 8; i += kTT)
       reinterpret_cast<uint2*>(rec)[i] = reinterpret_cast<const uint2*>(slot)[i];
-    const int64_t nw = g.N / 32;
-    for (int64_t i = tid; i < nw; i += kTT) bitsm[i] = reinterpret_cast<const uint32_t*>(slot + sc.off_bits)[i];
+    const int nw = m.wk > 0 ? (int)cdiv(g.N, 32) : 0;
+    for (int i = tid; i < nw; i += kTT) bitsm[i] = reinterpret_cast<const uint32_t*>(slot + sc.off_bits)[i];
     const int32_t* qs = reinterpret_cast<const int32_t*>(slot + sc.off_q);
     const int8_t* k8 = reinterpret_cast<const int8_t*>(slot + sc.off_k8);
     pack_q<true>(reinterpret_cast<uint32_t*>(rec + lay.off_q), qs, m.wq, colbase, m.r, g.L);
