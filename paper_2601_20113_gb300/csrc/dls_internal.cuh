@@ -66,11 +66,25 @@ struct Geom {
 
 __host__ __device__ inline Geom block_geom(const Plan& p, int64_t b) {
   Geom g;
-  int64_t ix = b % p.nbk[0]; b /= p.nbk[0];
-  int64_t iy = b % p.nbk[1]; b /= p.nbk[1];
-  int64_t iz = b % p.nbk[2]; b /= p.nbk[2];
-  int64_t it = b % p.nbk[3]; b /= p.nbk[3];
-  g.v = (int32_t)b;
+  int64_t ix, iy, iz, it;
+  if (p.nb_total <= 0x7FFFFFFF) {
+    // 32-bit divisions (64-bit ones are some seventy instructions each, and
+    // every thread of a kernel works its blocks' geometry out)
+    uint32_t r = (uint32_t)b;
+    const uint32_t n0 = (uint32_t)p.nbk[0], n1 = (uint32_t)p.nbk[1], n2 = (uint32_t)p.nbk[2], n3 = (uint32_t)p.nbk[3];
+    uint32_t q = r / n0;
+    ix = r - q * n0; r = q; q = r / n1;
+    iy = r - q * n1; r = q; q = r / n2;
+    iz = r - q * n2; r = q; q = r / n3;
+    it = r - q * n3;
+    g.v = (int32_t)q;
+  } else {
+    ix = b % p.nbk[0]; b /= p.nbk[0];
+    iy = b % p.nbk[1]; b /= p.nbk[1];
+    iz = b % p.nbk[2]; b /= p.nbk[2];
+    it = b % p.nbk[3]; b /= p.nbk[3];
+    g.v = (int32_t)b;
+  }
   g.x0 = ix * p.block[0]; g.y0 = iy * p.block[1]; g.z0 = iz * p.block[2]; g.t0 = it * p.block[3];
   int64_t rx = p.dims[0] - g.x0, ry = p.dims[1] - g.y0, rz = p.dims[2] - g.z0, rt = p.dims[3] - g.t0;
   g.sx = (int32_t)(rx < p.block[0] ? rx : p.block[0]);

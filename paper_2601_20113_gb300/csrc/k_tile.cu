@@ -381,8 +381,11 @@ __device__ void drain(TileSmem& S, Cursor& cu) {
 }
 
 // Streams every chunk of block bi through the ring, calling body(c, tile) for
-// each; all threads call.  Returns false if a wait timed out.
-template <class F>
+// each; all threads call.  Returns false if a wait timed out.  Every thread
+// waits for the chunk itself, so the barrier that frees its stage also carries
+// the word of a wait that ran out (a warp whose wait did skips the body).
+// SYNC: a body that holds CTA barriers, entered by all warps or none.
+template <bool SYNC = false, class F>
 __device__ bool stream_block(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
                              const Geom& g, int layout, F&& body) {
   const Chunks ch = chunks_of(a, g);
@@ -394,11 +397,15 @@ __device__ bool stream_block(const TileArgs& a, const Maps& tm, TileSmem& S, Cur
   cu.pf_cnt = 0;
   cu.pf_blk = -1;
   for (int c = 0; c < ch.n; ++c) {
-    wait_chunk(S, cu.con);
-    __syncthreads();
-    if (S.abort_flag) return false;
-    body(c, ch, &S.ring[cu.con % kStages][0]);
-    __syncthreads();
+    const bool in = __all_sync(FULL, wait_chunk(S, cu.con));
+    if (SYNC) {
+      if (__syncthreads_or(!in)) return false;
+      body(c, ch, &S.ring[cu.con % kStages][0]);
+      __syncthreads();
+    } else {
+      if (in) body(c, ch, &S.ring[cu.con % kStages][0]);
+      if (__syncthreads_or(!in)) return false;
+    }
     ++cu.con;
     if (c + kStages < ch.n) issue_chunk(a, tm, S, bi, g, ch, c + kStages, cu.iss, layout);
   }
@@ -651,7 +658,7 @@ __device__ __noinline__ bool pass_gram_tc(const TileArgs& a, const Maps& tm, Til
   const uint32_t fmt = bf ? 1u : 2u;
   const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
   uint32_t accum = 0;
-  const bool ok = stream_block(a, tm, S, cu, bi, g, kLayoutGram, [&](int c, const Chunks& ch, const float* tile_c) {
+  const bool ok = stream_block<true>(a, tm, S, cu, bi, g, kLayoutGram, [&](int c, const Chunks& ch, const float* tile_c) {
     float* tile = const_cast<float*>(tile_c);
     // statistics of the valid elements (read-only pass: neighbours are read)
     for (int gi = tid; gi < 1024; gi += kTT) {
@@ -1000,253 +1007,7 @@ __device__ __forceinline__ void row_decode_step(const TileSmem& S, int k, float 
 }
 
 
-// Bit-matrix transpose across a warp (lane i's bit j becomes lane j's bit i):
-// five butterfly stages, each swapping the off-diagonal halves of the blocks.
-__device__ __forceinline__ uint32_t warp_transpose_bits(uint32_t v, int lane) {
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
-    const uint32_t lo = s == 16 ? 0x0000FFFFu : s == 8 ? 0x00FF00FFu : s == 4 ? 0x0F0F0F0Fu : s == 2 ? 0x33333333u : 0x55555555u;
-    const uint32_t t = __shfl_xor_sync(FULL, v, s);
-    v = (lane & s) ? ((v & ~lo) | ((t >> s) & lo)) : ((v & lo) | ((t << s) & ~lo));
-  }
-  return v;
-}
-
-// ---------------------------------------------------------------- encode pass
-// Projection, quantization and decode at rank r, q into the CTA scratch,
-// corrections into k8/k32; with `check`, FP32 estimates of E(r-1), E(r) land
-// in S.Ered[0], S.Ered[1].  One row per thread; the column loop is not
-// unrolled (r is small), and each basis row is read once per column for both
-// the projection and the decode step.  Column widths: OR of zigzag(q) over
-// the warp (same bit width as the maximum), kept by lane k for column k, into S.qor.
-// SPARSE (pointwise bound, bitmap rows): k8 is written only for the elements
-// whose correction may be nonzero, and the record reads k8 through the
-// nonzero-correction bitmap; escapes cannot be listed from such a k8, so a
-// block that has any is encoded again without SPARSE.
-template <int NF, bool SPARSE>
-__device__ __noinline__ bool pass_encode(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
-                            const Geom& g, int r, bool check, const RowConst& rcst, const CorrConst& cc, bool pointwise,
-                            int32_t* qs, int8_t* k8, int32_t* k32, uint32_t* bits) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = NF ? NF : g.n;
-  // full blocks whose chunk rows are the block rows in order: each warp step
-  // covers 32 consecutive rows starting at a multiple of 32, so a ballot per
-  // column is one word of the nonzero-correction bitmap (element e -> bit e)
-  const bool use_bits = bitmap_rows(a, g);
-  // the constants by value: the loop's stores cannot be assumed not to alias them
-  const RowConst rq = rcst;
-  const CorrConst cq = cc;
-  uint32_t qor_lane = 0;   // lane k: OR of zigzag(q) of column k over this warp's rows
-  if (tid == 0) { S.kmax = 0; S.ncorr = 0; S.nesc = 0; S.nesc_slot = 0; }
-  __syncthreads();
-  float e1 = 0.0f, e2 = 0.0f;
-  float2 e1v = make_float2(0.0f, 0.0f), e2v = make_float2(0.0f, 0.0f);   // order 16: even / odd elements
-  int nc = 0, ne = 0, ovf = 0;
-  uint32_t kmx = 0;
-  const int M = (int)g.M, Lq = (int)align_up(g.L, 4), rc = a.rc;
-  const bool ok = stream_block(a, tm, S, cu, bi, g, kLayoutRow, [&](int c, const Chunks& ch, const float* tile) {
-    for (int rb = 0; rb < rc; rb += kTT) {          // same trip count in every lane
-      const int rr = rb + tid;
-      int xx = 0;
-      const int l = rr < rc ? (use_bits ? c * rc + rr : row_index(a, g, ch, c, rr, &xx)) : -1;
-      const bool valid = l >= 0;
-      const float* xr = tile + (valid ? rr : 0);
-      const float a0 = valid ? xr[0] : 0.0f;
-      float d[NM], acc[NM];
-      // order 16: element pairs as packed FMAs; fma(a, -1, x) rounds as x - a
-      const float2 m1 = make_float2(-1.0f, -1.0f);
-      auto x2 = [&](int j2) { return make_float2(xr[2 * j2 * rc], xr[(2 * j2 + 1) * rc]); };
-      if (NF == NM && valid) {
-#pragma unroll
-        for (int j2 = 0; j2 < NM / 2; ++j2) {
-          const float2 t = __ffma2_rn(make_float2(a0, a0), m1, x2(j2));
-          d[2 * j2] = t.x;
-          d[2 * j2 + 1] = t.y;
-          acc[2 * j2] = 0.0f;
-          acc[2 * j2 + 1] = 0.0f;
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < NM; ++j) {
-          d[j] = (valid && j < n) ? __fsub_rn(xr[j * rc], a0) : 0.0f;
-          acc[j] = 0.0f;
-        }
-      }
-#pragma unroll 1
-      for (int k = 0; k < r; ++k) {
-        float v[NM];
-        const float4* vp = reinterpret_cast<const float4*>(&S.VstT[k * NM]);
-#pragma unroll
-        for (int j4 = 0; j4 < NM / 4; ++j4) {
-          const float4 t = vp[j4];
-          v[4 * j4 + 0] = t.x; v[4 * j4 + 1] = t.y; v[4 * j4 + 2] = t.z; v[4 * j4 + 3] = t.w;
-        }
-        const float cf = project<NF>(d, v, a0, S.vsum[k], n);
-        const int32_t q = quant_exact(cf, rq.delta, rq.inv_delta, ovf);
-        if (valid) qs[k * Lq + l] = q;
-        const uint32_t wor = __reduce_or_sync(FULL, valid ? zigzag(q) : 0u);
-        if (lane == k) qor_lane |= wor;
-        const float chk = __fmul_rn(__int2float_rn(q), rq.delta_f);
-        if (check && k == r - 1 && valid) {
-          if (NF == NM) {
-#pragma unroll
-            for (int j2 = 0; j2 < NM / 2; ++j2) {
-              const float2 dd = __ffma2_rn(make_float2(acc[2 * j2], acc[2 * j2 + 1]), m1, x2(j2));
-              e1v = __ffma2_rn(dd, dd, e1v);
-            }
-          } else {
-#pragma unroll
-            for (int j = 0; j < NM; ++j)
-              if (j < n) { const float dd = __fsub_rn(xr[j * rc], acc[j]); e1 = __fmaf_rn(dd, dd, e1); }
-          }
-        }
-#pragma unroll
-        for (int j2 = 0; j2 < NM / 2; ++j2) {
-          // decode step, two elements per packed FMA (each as __fmaf_rn)
-          const float2 t = __ffma2_rn(make_float2(chk, chk), make_float2(v[2 * j2], v[2 * j2 + 1]),
-                                      make_float2(acc[2 * j2], acc[2 * j2 + 1]));
-          acc[2 * j2] = t.x;
-          acc[2 * j2 + 1] = t.y;
-        }
-      }
-      if (SPARSE && valid) {
-        // elements with |fl(x - xhat)| < eb (rounded down) need no correction
-        // (the first test of the decision); the others are decided one by one
-        uint32_t cand = 0;
-        if (NF == NM) {
-#pragma unroll
-          for (int j2 = 0; j2 < NM / 2; ++j2) {
-            const float2 R = __ffma2_rn(make_float2(acc[2 * j2], acc[2 * j2 + 1]), m1, x2(j2));
-            if (check) e2v = __ffma2_rn(R, R, e2v);
-            cand |= (corr_candidate(R.x, cq) ? 1u : 0u) << (2 * j2);
-            cand |= (corr_candidate(R.y, cq) ? 1u : 0u) << (2 * j2 + 1);
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < NM; ++j) {
-            if (j < n) {
-              const float R = __fsub_rn(xr[j * rc], acc[j]);
-              if (check) e2 = __fmaf_rn(R, R, e2);
-              cand |= (corr_candidate(R, cq) ? 1u : 0u) << j;
-            }
-          }
-        }
-        uint32_t nzb = 0, escm = 0;
-        while (cand) {
-          const int jj = __ffs(cand) - 1;
-          cand &= cand - 1;
-          float aj = acc[0];
-#pragma unroll
-          for (int j = 1; j < NM; ++j) aj = (j == jj) ? acc[j] : aj;
-          const int32_t k = corr_decide(xr[jj * rc], aj, cq);
-          const int e = jj * M + l;
-          const bool big = k < -127 || k > 127;            // includes escapes
-          k8[e] = big ? (int8_t)-128 : (int8_t)k;
-          if (big) k32[e] = k;
-          escm |= (k == kEscape ? 1u : 0u) << jj;
-          nc += k != 0 ? 1 : 0;
-          kmx |= k == kEscape ? 0u : zigzag(k);
-          nzb |= (k != 0 && k != kEscape ? 1u : 0u) << jj;
-        }
-        if (escm) {
-          // rare: the row's escapes, listed for the deferred packer (in no
-          // particular order)
-          ne += __popc(escm);
-          uint32_t* const el = S.esc_list;
-          if (el) {
-            for (uint32_t em = escm; em; em &= em - 1) {
-              const int i = atomicAdd(&S.nesc_slot, 1);
-              if (i < S.esc_cap) el[i] = (uint32_t)((__ffs(em) - 1) * M + l);
-            }
-          }
-        }
-        // lane j gets column j's word of the bitmap (this warp's 32 rows)
-        const uint32_t mk = warp_transpose_bits(nzb, lane);
-        if (lane < n) bits[(lane * M + (l - lane)) >> 5] = mk;
-      } else if (valid) {
-        // corrections: every element decided first without branches (so they
-        // interleave); the few the FP32 evaluation leaves open take the FP64 path
-        int32_t kv[NM];
-        uint32_t unsure = 0;
-#pragma unroll
-        for (int j = 0; j < NM; ++j) {
-          kv[j] = 0;
-          if (j < n) {
-            const float xj = xr[j * rc];
-            if (check) { const float dd = __fsub_rn(xj, acc[j]); e2 = __fmaf_rn(dd, dd, e2); }
-            if (pointwise) {
-              bool u;
-              kv[j] = corr_fast(xj, acc[j], cq, &u);
-              unsure |= (u ? 1u : 0u) << j;
-            }
-          }
-        }
-        while (unsure) {
-          const int jj = __ffs(unsure) - 1;
-          unsure &= unsure - 1;
-          float aj = acc[0];
-#pragma unroll
-          for (int j = 1; j < NM; ++j) aj = (j == jj) ? acc[j] : aj;
-          const int32_t v = corr_slow(xr[jj * rc], aj, cq);
-#pragma unroll
-          for (int j = 0; j < NM; ++j) kv[j] = (j == jj) ? v : kv[j];
-        }
-#pragma unroll
-        for (int j = 0; j < NM; ++j) {
-          if (j < n) {
-            const int e = j * M + l;
-            const int32_t k = kv[j];
-            const bool big = k < -127 || k > 127;            // includes escapes
-            k8[e] = big ? (int8_t)-128 : (int8_t)k;
-            if (big) k32[e] = k;
-            ne += k == kEscape ? 1 : 0;
-            nc += k != 0 ? 1 : 0;                             // escapes taken out below
-            kmx |= k == kEscape ? 0u : zigzag(k);             // OR: same bit width as the maximum
-          }
-        }
-        if (use_bits) {
-#pragma unroll
-          for (int j = 0; j < NM; ++j) {
-            if (j < n) {
-              const unsigned mk = __ballot_sync(FULL, kv[j] != 0 && kv[j] != kEscape);
-              if (lane == 0) bits[(j * M + l) >> 5] = mk;
-            }
-          }
-        }
-      }
-    }
-  });
-  if (!ok) return false;
-  nc -= ne;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    nc += __shfl_xor_sync(FULL, nc, o);
-    ne += __shfl_xor_sync(FULL, ne, o);
-    kmx |= __shfl_xor_sync(FULL, kmx, o);
-    ovf |= __shfl_xor_sync(FULL, ovf, o);
-  }
-  if (lane == 0) {
-    if (nc) atomicAdd(&S.ncorr, nc);
-    if (ne) atomicAdd(&S.nesc, ne);
-    if (kmx) atomicOr(reinterpret_cast<unsigned int*>(&S.kmax), kmx);
-    if (ovf) S.ovf = 1;
-  }
-  if (lane < NM) S.qor[warp][lane] = qor_lane;
-  __syncthreads();
-  if (tid < NM) {
-    uint32_t o = 0;
-    for (int w = 0; w < kWarps; ++w) o |= S.qor[w][tid];
-    S.wq[tid] = tid < r ? bit_width(o) : 0;
-  }
-  e1 = __fadd_rn(e1, __fadd_rn(e1v.x, e1v.y));
-  e2 = __fadd_rn(e2, __fadd_rn(e2v.x, e2v.y));
-  const float ev[2] = {e1, e2};
-  if (check) cta_reduce(S, ev, 2);
-  else __syncthreads();
-  return true;
-}
-
-// ---------------------------------------------------------------- k_enc's row pass
+// ---------------------------------------------------------------- row pass
 // Rows of a chunk in block order: row i of the chunk is block row lbase + i
 // (x fastest; a chunk is whole planes, or lines of one plane).
 struct ChunkRows {
@@ -1263,9 +1024,10 @@ __device__ __forceinline__ ChunkRows chunk_rows(const TileArgs& a, const Geom& g
 }
 
 // Projection, quantization and decode at rank r with FP32 estimates of E(r-1)
-// and E(r) (S.Ered[0], [1]) and, POINT, the corrections: q and k8 into the
-// block's slot, the nonzero-correction bitmap into S.bitsm; blocks of at most
-// 32 kBitsSmem points with 1 to NP time steps.  One row a thread.
+// and E(r) (S.Ered[0], [1]) and, POINT, the corrections: q, k8 (a byte an
+// element; -128 where k32 holds the value or an escape) and the bitmap of
+// nonzero corrections, S.bitsm or for blocks it cannot hold `bits`; blocks with
+// 1 to NP time steps.  One row a thread.
 // Every correction of a row is worked out, two a packed instruction, without a
 // branch: y = R / 2eb, k = rint(y) by adding 1.5 x 2^23 (k is then the low
 // byte of that sum, ready to store), xt = k 2eb + xhat.  A row is settled when
@@ -1287,22 +1049,24 @@ constexpr int kFastK = 59;
 template <int NP, bool POINT, int MC>
 __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
                                        const Geom& g, int r, const RowConst& rcst, const CorrConst& cc,
-                                       int32_t* __restrict__ qs, int8_t* __restrict__ k8, int32_t* __restrict__ k32) {
+                                       int32_t* __restrict__ qs, int8_t* __restrict__ k8, int32_t* __restrict__ k32,
+                                       uint32_t* bits) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = MC ? NP : g.n, M = MC ? MC : (int)g.M, rc = MC ? 256 : a.rc;
   const RowConst rq = rcst;
-  const CorrConst cq = cc;
+  const float eb_lo = cc.eb_lo_f;
   const int Lq = MC ? MC : (int)align_up(g.L, 4);
   const Chunks ch0 = chunks_of(a, g);
   // every chunk starts on a multiple of 32 rows, in every column
   const bool words = MC || ((M & 31) == 0 && (chunk_rows(a, g, ch0, 0).count & 31) == 0 &&
                             (ch0.ncy == 1 || (g.sx * g.sy & 31) == 0));
   if (tid == 0) { S.kmax = 0; S.ncorr = 0; S.nesc = 0; S.nesc_slot = 0; }
+  uint32_t* const bw = MC ? S.bitsm : bits;
   if (POINT && !words)
-    for (int i = tid; i < (n * M + 31) / 32; i += kTT) S.bitsm[i] = 0u;
+    for (int i = tid; i < (n * M + 31) / 32; i += kTT) bw[i] = 0u;
   __syncthreads();
   const float2 m1 = make_float2(-1.0f, -1.0f), mg = make_float2(kMagicF, kMagicF), nmg = make_float2(-kMagicF, -kMagicF);
-  const float2 inv2 = make_float2(cq.inv_step_f, cq.inv_step_f), step2 = make_float2(cq.step_f, cq.step_f);
+  const float2 inv2 = make_float2(cc.inv_step_f, cc.inv_step_f), step2 = make_float2(cc.step_f, cc.step_f);
   float2 e1 = make_float2(0.0f, 0.0f), e2 = make_float2(0.0f, 0.0f);
   uint32_t qor_lane = 0, kmx = 0;
   int nc = 0, ne = 0, ovf = 0, zmx = kMagicI, zmn = kMagicI;
@@ -1365,7 +1129,8 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
         float rq_f = __fsub_rn(z, kMagicF);
         int32_t q = __float_as_int(z) - kMagicI;
         if (!(fabsf(__fsub_rn(y, rq_f)) < 0.5f - __fmaf_rn(fabsf(y), 4.0e-7f, 1.0e-30f) && fabsf(y) < 4.0e6f)) {
-          q = quant_fp64(cf, rq.delta, &ovf);
+          q = quant_fp64(cf, rq.delta);
+          if (q == INT32_MIN) { q = 0; ovf = 1; }
           rq_f = __int2float_rn(q);
         }
         if (valid) qs[k * Lq + l] = q;
@@ -1410,8 +1175,8 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
         const float2 dd = __ffma2_rn(xt, m1, x2);
         zi[j] = __float_as_int(z.x);
         zi[j + 1] = __float_as_int(z.y);
-        settled = settled && fabsf(fr.x) < 0.49997f && fabsf(fr.y) < 0.49997f && fabsf(dd.x) <= cq.eb_lo_f &&
-                  fabsf(dd.y) <= cq.eb_lo_f;
+        settled = settled && fabsf(fr.x) < 0.49997f && fabsf(fr.y) < 0.49997f && fabsf(dd.x) <= eb_lo &&
+                  fabsf(dd.y) <= eb_lo;
       }
       int hi = zi[0], lo = zi[0];
 #pragma unroll
@@ -1433,7 +1198,7 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
             aj = j == jj ? acc[j] : aj;
             xj = j == jj ? x[j] : xj;
           }
-          const int32_t k = corr_decide(xj, aj, cq);
+          const int32_t k = corr_decide(xj, aj, S.ccc);
           const bool big = k < -127 || k > 127;            // includes escapes
           const int zb = kMagicI + (big ? -128 : k);
           if (big && valid) k32[jj * M + l] = k;
@@ -1471,12 +1236,12 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
       if (lane < n && (w != 0u || (words && (MC || i - lane < cr.count)))) {
         const uint32_t e0 = (uint32_t)(lane * M + (l - lane));
         if (words) {
-          S.bitsm[e0 >> 5] = w;
+          bw[e0 >> 5] = w;
         } else {
           const uint32_t sh = e0 & 31u;
-          atomicOr(&S.bitsm[e0 >> 5], w << sh);
+          atomicOr(&bw[e0 >> 5], w << sh);
           const uint32_t up = sh ? w >> (32u - sh) : 0u;
-          if (up) atomicOr(&S.bitsm[(e0 >> 5) + 1], up);
+          if (up) atomicOr(&bw[(e0 >> 5) + 1], up);
         }
       }
     }
@@ -1509,12 +1274,12 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
 template <bool POINT>
 __device__ __forceinline__ bool encode_rows(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
                                             const Geom& g, int r, const RowConst& rcst, const CorrConst& cc, int32_t* qs,
-                                            int8_t* k8, int32_t* k32) {
+                                            int8_t* k8, int32_t* k32, uint32_t* bits) {
   if (g.n == NM && g.M == 4096 && a.rc == 256 && g.sx == a.bxb && bitmap_rows(a, g))
-    return pass_rows<NM, POINT, 4096>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32);
-  if (g.n <= 4) return pass_rows<4, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32);
-  if (g.n <= 8) return pass_rows<8, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32);
-  return pass_rows<NM, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32);
+    return pass_rows<NM, POINT, 4096>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32, bits);
+  if (g.n <= 4) return pass_rows<4, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32, bits);
+  if (g.n <= 8) return pass_rows<8, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32, bits);
+  return pass_rows<NM, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32, bits);
 }
 
 // E(r) for every r in [0, rcap] (FP32 estimates into S.Ered).
@@ -1559,6 +1324,72 @@ __device__ __noinline__ bool pass_all_errors(const TileArgs& a, const Maps& tm, 
   });
   if (!ok) return false;
   cta_reduce(S, E, rcap + 1);
+  return true;
+}
+
+// E(m) for the ranks m of `mask` (at most kProbes of them, FP32 estimates into
+// S.Ered in increasing m): the probes of a bisection that ends at a predicted
+// rank.  The same arithmetic as pass_all_errors on the columns up to the
+// largest of them: at rank 3 of 16 half the columns and four residuals, where
+// all of them cost 16 of each.
+constexpr int kProbes = 6;
+__device__ __forceinline__ uint32_t bisection_probes(int target, int rcap) {
+  uint32_t m = 0;
+  for (int lo = 0, hi = rcap; lo < hi;) {
+    const int mid = (lo + hi) >> 1;
+    m |= 1u << mid;
+    if (mid >= target) hi = mid;
+    else lo = mid + 1;
+  }
+  return m;
+}
+template <int NF>
+__device__ __noinline__ bool pass_probe_errors(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
+                                               const Geom& g, uint32_t mask, const RowConst& rcst) {
+  const int tid = threadIdx.x, n = NF ? NF : g.n, rc = a.rc;
+  const int kmax = 31 - __clz(mask);
+  float E[kProbes];
+#pragma unroll
+  for (int q = 0; q < kProbes; ++q) E[q] = 0.0f;
+  const RowConst rq = rcst;
+  int ovf = 0;                                  // (none possible: the caller has checked)
+  const bool ok = stream_block(a, tm, S, cu, bi, g, kLayoutRow, [&](int c, const Chunks& ch, const float* tile) {
+    for (int rr = tid; rr < rc; rr += kTT) {
+      int xx;
+      if (row_index(a, g, ch, c, rr, &xx) < 0) continue;
+      const float* xr = tile + rr;
+      const float a0 = xr[0];
+      float x[NM], d[NM], acc[NM];
+#pragma unroll
+      for (int j = 0; j < NM; ++j) {
+        acc[j] = 0.0f;
+        x[j] = j < n ? xr[j * rc] : 0.0f;
+        d[j] = j < n ? __fsub_rn(x[j], a0) : 0.0f;
+      }
+      int slot = 0;
+#pragma unroll 1
+      for (int m = 0;; ++m) {
+        if ((mask >> m) & 1u) {
+          float2 t = make_float2(0.0f, 0.0f);
+#pragma unroll
+          for (int j = 0; j < NM; j += 2) {
+            const float2 dd = __ffma2_rn(make_float2(acc[j], acc[j + 1]), make_float2(-1.0f, -1.0f), make_float2(x[j], x[j + 1]));
+            t = __ffma2_rn(dd, dd, t);
+          }
+          const float e = __fadd_rn(t.x, t.y);
+#pragma unroll
+          for (int q = 0; q < kProbes; ++q) E[q] = q == slot ? __fadd_rn(E[q], e) : E[q];
+          ++slot;
+        }
+        if (m == kmax) break;
+        int32_t q;
+        const float chk = coeff_q<NF>(S, d, a0, n, m, rq, q, ovf);
+        row_decode_step(S, m, chk, acc);
+      }
+    }
+  });
+  if (!ok) return false;
+  cta_reduce(S, E, __popc(mask));
   return true;
 }
 
@@ -1627,9 +1458,10 @@ __device__ __noinline__ double exact_error(const TileArgs& a, TileSmem& S, const
 
 __device__ bool decide_pass(const TileArgs& a, TileSmem& S, const Geom& g, int r, double E32, double bnd, double el2,
                             const RowConst& rcst) {
-  const double lo = E32 / (1.0 + bnd), hi = E32 / (1.0 - bnd);
-  if (hi < el2 * (1.0 - 1e-12)) return true;
-  if (lo > el2 * (1.0 + 1e-12)) return false;
+  // (products, not quotients, and integer comparisons of non-negative values:
+  // every warp decides, and FP64 instructions hold a quarter of the SM each)
+  if (mag_below(E32, el2 * ((1.0 - 1e-12) * (1.0 - bnd)))) return true;
+  if (mag_above(E32, el2 * ((1.0 + 1e-12) * (1.0 + bnd)))) return false;
   if (threadIdx.x == 0) S.nexact += 1;
   return exact_error(a, S, g, r, rcst) <= el2;
 }
@@ -1826,8 +1658,8 @@ __device__ __forceinline__ void pack_q(uint32_t* qw, const int32_t* qs, const ui
   }
 }
 
-// Dense corrections: 32 elements of wk bits per task -> exactly wk words.
-// With the bitmap (bits != nullptr) k8 counts only where a bit is set.
+// Dense corrections: 32 elements of wk bits per task -> exactly wk words; k8
+// counts only where the bitmap has a bit (it has none for escapes).
 template <bool FIXED = false>
 __device__ __forceinline__ void pack_dense(uint32_t* cw, const int8_t* k8, const int32_t* k32, const uint32_t* bits,
                                            int wk, int64_t N) {
@@ -1836,7 +1668,7 @@ __device__ __forceinline__ void pack_dense(uint32_t* cw, const int8_t* k8, const
     const int64_t first = task * 32;
     const int cnt = (int)((N - first) < 32 ? (N - first) : 32);
     uint32_t* dst = cw + task * wk;
-    const uint32_t bw = bits ? bits[task] : 0xFFFFFFFFu;
+    const uint32_t bw = bits[task];
     if (FIXED && cnt == 32 && wk <= kMaxFixedW) {
       // no k32 values here (corrections below 64)
       const uint4* kv4 = reinterpret_cast<const uint4*>(k8 + first);
@@ -2121,20 +1953,11 @@ __device__ __noinline__ void write_record(const TileArgs& a, TileSmem& S, const 
   uint32_t* cw = reinterpret_cast<uint32_t*>(rec + lay.off_c);
   if (m.wk > 0) {
     if (lay.dense) {
-      // bitmap rows: k8 may hold stale bytes where the bitmap has no bit
-      pack_dense(cw, k8, k32, bitmap_rows(a, g) ? bits : nullptr, m.wk, N);
+      pack_dense(cw, k8, k32, bits, m.wk, N);
     } else {
       // entry list (element indices) into the q scratch
       uint32_t* list = reinterpret_cast<uint32_t*>(qs);
-      if (bitmap_rows(a, g)) {
-        bitmap_list(list, bits, N, m.ncorr, S.warp_cnt);
-      } else {
-        compact16(
-            S, k8, (int)N, [&](int8_t b, int e) { return b != 0 && (b != (int8_t)-128 || k32[e] != kEscape); },
-            [&](int e, int idx) {
-              if (idx < m.ncorr) list[idx] = (uint32_t)e;   // the count and the bytes agree by construction
-            });
-      }
+      bitmap_list(list, bits, N, m.ncorr, S.warp_cnt);
       pack_sparse(cw, list, k8, k32, m.ib, m.wk, m.ncorr);
     }
   }
@@ -2207,8 +2030,9 @@ struct FastBlock {
   int32_t pad[2];
 };
 // kFbRankFail: k_enc ran the exact test at the predicted rank and it failed
-// (or a coefficient overflowed), so k_tile goes straight to the search.
-enum : int32_t { kFbNonfinite = 1, kFbRR = 2, kFbOverflow = 4, kFbRankFail = 8 };
+// (or a coefficient overflowed), so k_tile goes straight to the search;
+// kFbRankLow: because the rank is above the prediction.
+enum : int32_t { kFbNonfinite = 1, kFbRR = 2, kFbOverflow = 4, kFbRankFail = 8, kFbRankLow = 16 };
 
 // Block counters of the phase kernels and the list of blocks k_enc leaves.
 struct FastCtl {
@@ -2643,18 +2467,16 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
   const Maps tm{&tmap, &tmapg};
   const Plan& P = a.P;
   int32_t* k32 = a.k32_scr + (int64_t)blockIdx.x * a.nptmax;
+  uint32_t* const bit_scr = a.bit_scr + (int64_t)blockIdx.x * (align_up(a.nptmax, 32) / 32);
   init_stream_smem(a, S);
   __syncthreads();
   PhaseClock pc;
   Cursor cu;
   cu.iss = 0; cu.con = 0; cu.pf_blk = -1; cu.pf_cnt = 0; cu.pf_layout = kLayoutRow;
   const bool pointwise = P.eb_type != DLS_EB_NRMSE;
-  auto eligible = [&](int64_t b, int* rp_out) -> bool {
-    const Geom gb = block_geom(P, P.b0 + b);
+  auto eligible = [&](int64_t b) -> bool {
     const FastBlock& fb = a.fb[b];
-    const int rp = fb.rpred;
-    *rp_out = rp;
-    return !(fb.flags & (kFbNonfinite | kFbRR | kFbOverflow)) && slot_scratch(rp, gb.n, gb.L, gb.N, pointwise).fits;
+    return !(fb.flags & (kFbNonfinite | kFbRR | kFbOverflow));
   };
   auto to_list = [&](int64_t b) {
     if (threadIdx.x == 0) {
@@ -2670,8 +2492,7 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
     if (bi >= a.bhi) break;
     if (threadIdx.x == 0) S.bnext = grab_range(a, &a.ctl->next_enc);
     const Geom g = block_geom(P, P.b0 + bi);
-    int rp = 0;
-    if (!eligible(bi, &rp)) {
+    if (!eligible(bi)) {
       if (!(a.fb[bi].flags & kFbNonfinite)) to_list(bi);
       __syncthreads();          // thread 0 has taken the next block
       continue;
@@ -2683,24 +2504,28 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
     const CorrConst cc = S.ccc;
     pc.start();
     load_basis(S, a.fb[bi]);
+    const int rp = S.r_pred;
     uint8_t* const slot = a.staging + align_up((g.pt_off - P.pt_base) * 4, 16) + 48 * bi;
     const SlotScratch sc = slot_scratch(rp, g.n, g.L, g.N, pointwise);
+    uint32_t* const bits = g.N <= (int64_t)kBitsSmem * 32 ? S.bitsm : bit_scr;
     if (threadIdx.x == 0) {
-      S.esc_list = reinterpret_cast<uint32_t*>(slot + sc.off_esc);
+      S.esc_list = sc.fits ? reinterpret_cast<uint32_t*>(slot + sc.off_esc) : nullptr;
       S.esc_cap = (int)sc.esc_cap;
     }
-    int32_t* const qs = reinterpret_cast<int32_t*>(slot + sc.off_q);
-    int8_t* const k8 = reinterpret_cast<int8_t*>(slot + sc.off_k8);
-    if (!(pointwise ? encode_rows<true>(a, tm, S, cu, bi, g, rp, rcst, cc, qs, k8, k32)
-                    : encode_rows<false>(a, tm, S, cu, bi, g, rp, rcst, cc, qs, k8, k32)))
+    // a rank that leaves the slot no room: into the CTA's scratch, and the record here
+    int32_t* const qs = sc.fits ? reinterpret_cast<int32_t*>(slot + sc.off_q) : a.q_scr + (int64_t)blockIdx.x * NM * a.lmax;
+    int8_t* const k8 = sc.fits ? reinterpret_cast<int8_t*>(slot + sc.off_k8) : a.k8_scr + (int64_t)blockIdx.x * a.nptmax;
+    if (!(pointwise ? encode_rows<true>(a, tm, S, cu, bi, g, rp, rcst, cc, qs, k8, k32, bits)
+                    : encode_rows<false>(a, tm, S, cu, bi, g, rp, rcst, cc, qs, k8, k32, bits)))
       break;
     pc.mark(S, kPhEncode);
-    bool accepted = false;
+    bool accepted = false, low = false;
     if (!S.ovf) {
       const Chunks chk = chunks_of(a, g);
       const double bnd = (double)(cdiv(a.rc, kTT) * chk.n * g.n + 40) * 6.6e-8;
       const double E_rm1 = S.Ered[0], E_r = S.Ered[1];
       const bool p_r = decide_pass(a, S, g, rp, E_r, bnd, el2, rcst);
+      low = !p_r;
       bool p_rm1 = false;
       if (rp > 0 && p_r) p_rm1 = decide_pass(a, S, g, rp - 1, E_rm1, bnd, el2, rcst);
       accepted = p_r && !p_rm1;
@@ -2710,24 +2535,24 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
     const bool rank_fail = !accepted;
     // a deferred record has no correction beyond kDeferMaxWk bits, its
     // escapes fit the slot's list and, when sparse, so does its entry list
-    if (accepted) {
+    if (accepted && sc.fits) {
       const int wk = bit_width((uint32_t)S.kmax), ib = bit_width((uint32_t)(g.N - 1));
       const bool dense = wk > 0 && (g.N * wk + 31) / 32 < ((int64_t)S.ncorr * (ib + wk) + 31) / 32;
       if (wk > kDeferMaxWk || (!dense && S.ncorr > sc.list_cap) || S.nesc > sc.esc_cap) accepted = false;
     }
     pc.mark(S, kPhDecide);
     if (!accepted) {
-      if (rank_fail && threadIdx.x == 0) a.fb[bi].flags |= kFbRankFail;
+      if (rank_fail && threadIdx.x == 0) a.fb[bi].flags |= kFbRankFail | (low ? kFbRankLow : 0);
       to_list(bi);
       __syncthreads();
       continue;
     }
     {
-      int rn = 0;
       const int64_t bn = S.bnext;
-      if (bn < a.bhi && eligible(bn, &rn)) prefetch(a, tm, S, cu, bn, block_geom(P, P.b0 + bn), kLayoutRow);
+      if (bn < a.bhi && eligible(bn)) prefetch(a, tm, S, cu, bn, block_geom(P, P.b0 + bn), kLayoutRow);
     }
-    defer_record(a, S, g, bi, rp, S.bitsm);
+    if (sc.fits) defer_record(a, S, g, bi, rp, S.bitsm);
+    else write_record(a, S, g, bi, false, rp, qs, k8, k32, bits);
     pc.mark(S, kPhPack);
     if (threadIdx.x == 0) S.ph[kCntAccepted] += 1;
   }
@@ -2755,7 +2580,7 @@ __global__ void __launch_bounds__(kTT, MINB) k_tile(const __grid_constant__ CUte
   int32_t* qs = a.q_scr + (int64_t)blockIdx.x * NM * a.lmax;
   int8_t* k8 = a.k8_scr + (int64_t)blockIdx.x * a.nptmax;
   int32_t* k32 = a.k32_scr + (int64_t)blockIdx.x * a.nptmax;
-  uint32_t* bits = a.bit_scr + (int64_t)blockIdx.x * (align_up(a.nptmax, 32) / 32);
+  uint32_t* const bit_scr = a.bit_scr + (int64_t)blockIdx.x * (align_up(a.nptmax, 32) / 32);
   const Plan& P = a.P;
   init_stream_smem(a, S);
   __syncthreads();
@@ -2812,34 +2637,22 @@ __global__ void __launch_bounds__(kTT, MINB) k_tile(const __grid_constant__ CUte
     if (did_rr) predicted_rank(a, S, g, bi, rcap, el2, vi.delta);
     pc.mark(S, kPhPredict);
 
-    // the encode pass at rank rr; SPARSE where the bitmap carries the corrections,
-    // kept in shared memory when the block has at most kBitsSmem * 32 points
-    const bool sparse = pointwise && bitmap_rows(a, g);
-    uint32_t* const bitp = g.N <= (int64_t)kBitsSmem * 32 ? S.bitsm : bits;
-    // SPARSE passes whose rank leaves room write q and k8 into the block's
-    // staging slot (deferred packing); the others use the CTA's scratch
+    // the row pass at rank rr, into the block's staging slot (deferred packing)
+    // when the rank leaves room, else into the CTA's scratch
+    uint32_t* const bits = g.N <= (int64_t)kBitsSmem * 32 ? S.bitsm : bit_scr;
     uint8_t* const slot = a.staging + align_up((g.pt_off - P.pt_base) * 4, 16) + 48 * bi;
     bool in_slot = false;
-    auto encode = [&](int rr, bool check, bool sp, bool cta_scratch) -> bool {
-      in_slot = false;
-      if (sp) {
-        int32_t* q = qs;
-        int8_t* k = k8;
-        uint32_t* esc = nullptr;
-        const SlotScratch sc = slot_scratch(rr, g.n, g.L, g.N);
-        if (!cta_scratch && sc.fits) {
-          q = reinterpret_cast<int32_t*>(slot + sc.off_q);
-          k = reinterpret_cast<int8_t*>(slot + sc.off_k8);
-          esc = reinterpret_cast<uint32_t*>(slot + sc.off_esc);
-          in_slot = true;
-        }
-        if (tid == 0) { S.esc_list = esc; S.esc_cap = (int)sc.esc_cap; }   // read after the pass's first barrier
-        return full ? pass_encode<NM, true>(a, tm, S, cu, bi, g, rr, check, rcst, cc, pointwise, q, k, k32, bitp)
-                    : pass_encode<0, true>(a, tm, S, cu, bi, g, rr, check, rcst, cc, pointwise, q, k, k32, bitp);
+    auto encode = [&](int rr, bool cta_scratch) -> bool {
+      const SlotScratch sc = slot_scratch(rr, g.n, g.L, g.N, pointwise);
+      in_slot = !cta_scratch && sc.fits;
+      int32_t* const q = in_slot ? reinterpret_cast<int32_t*>(slot + sc.off_q) : qs;
+      int8_t* const k = in_slot ? reinterpret_cast<int8_t*>(slot + sc.off_k8) : k8;
+      if (tid == 0) {                       // read after the pass's first barrier
+        S.esc_list = in_slot ? reinterpret_cast<uint32_t*>(slot + sc.off_esc) : nullptr;
+        S.esc_cap = (int)sc.esc_cap;
       }
-      if (tid == 0) S.esc_list = nullptr;
-      return full ? pass_encode<NM, false>(a, tm, S, cu, bi, g, rr, check, rcst, cc, pointwise, qs, k8, k32, bitp)
-                  : pass_encode<0, false>(a, tm, S, cu, bi, g, rr, check, rcst, cc, pointwise, qs, k8, k32, bitp);
+      return pointwise ? encode_rows<true>(a, tm, S, cu, bi, g, rr, rcst, cc, q, k, k32, bits)
+                       : encode_rows<false>(a, tm, S, cu, bi, g, rr, rcst, cc, q, k, k32, bits);
     };
     const Chunks chk = chunks_of(a, g);
     const int64_t rows_per_thread = cdiv(a.rc, kTT) * chk.n;
@@ -2848,7 +2661,7 @@ __global__ void __launch_bounds__(kTT, MINB) k_tile(const __grid_constant__ CUte
     int r = 0;
     if (a.learned != kRankSearch && !may_overflow && !(a.fb[bi].flags & kFbRankFail)) {
       const int rp = S.r_pred;
-      if (!encode(rp, true, sparse, false)) break;
+      if (!encode(rp, false)) break;
       pc.mark(S, kPhEncode);
       const double E_rm1 = S.Ered[0], E_r = S.Ered[1];
       if (!S.ovf) {
@@ -2868,34 +2681,67 @@ __global__ void __launch_bounds__(kTT, MINB) k_tile(const __grid_constant__ CUte
       __syncthreads();
       if (tid == 0) S.ovf = 0;
       __syncthreads();
-      int ovf = 0;
-      if (!(full ? pass_all_errors<NM>(a, tm, S, cu, bi, g, rcap, rcst, ovf)
-                 : pass_all_errors<0>(a, tm, S, cu, bi, g, rcap, rcst, ovf)))
-        break;
-      if (ovf) S.ovf = 1;
-      __syncthreads();
-      double Eall[NM + 1];
-      for (int i = 0; i <= rcap; ++i) Eall[i] = S.Ered[i];
-      if (S.ovf) {
-        raw = true;
-      } else {
+      // the bisection on the probes it would make towards a predicted rank;
+      // one that turns another way needs them all
+      bool found = false;
+      if (!may_overflow && rcap > 0) {
+        const int32_t fl = a.fb[bi].flags;
+        int target = S.r_pred;
+        if (fl & kFbRankFail) {
+          const int tail = a.feat ? (int)a.feat[bi * kMlpF + kMlpF - 1] : target;
+          target = tail != target ? tail : target + ((fl & kFbRankLow) ? 1 : -1);
+        }
+        target = target < 0 ? 0 : (target > rcap ? rcap : target);
+        const uint32_t mask = bisection_probes(target, rcap) | (pointwise ? 0u : 1u << target);
+        if (!(full ? pass_probe_errors<NM>(a, tm, S, cu, bi, g, mask, rcst)
+                   : pass_probe_errors<0>(a, tm, S, cu, bi, g, mask, rcst)))
+          break;
         int lo = 0, hi = rcap;
+        found = true;
+        auto at = [&](int m) { return S.Ered[__popc(mask & ((1u << m) - 1u))]; };
         while (lo < hi) {
           const int mid = (lo + hi) >> 1;
-          if (decide_pass(a, S, g, mid, Eall[mid], bnd, el2, rcst)) hi = mid;
+          if (!((mask >> mid) & 1u)) { found = false; break; }
+          if (decide_pass(a, S, g, mid, at(mid), bnd, el2, rcst)) hi = mid;
           else lo = mid + 1;
         }
+        if (found && !pointwise) {
+          if (!((mask >> lo) & 1u)) found = false;
+          else if (!decide_pass(a, S, g, lo, at(lo), bnd, el2, rcst)) raw = true;
+        }
         r = lo;
-        if (!pointwise && !decide_pass(a, S, g, r, Eall[r], bnd, el2, rcst)) raw = true;
-        if (!raw && !encode(r, false, sparse, false)) break;
+        __syncthreads();                        // S.Ered is read before another pass writes it
       }
+      if (!found) {
+        int ovf = 0;
+        if (!(full ? pass_all_errors<NM>(a, tm, S, cu, bi, g, rcap, rcst, ovf)
+                   : pass_all_errors<0>(a, tm, S, cu, bi, g, rcap, rcst, ovf)))
+          break;
+        if (ovf) S.ovf = 1;
+        __syncthreads();
+        double Eall[NM + 1];
+        for (int i = 0; i <= rcap; ++i) Eall[i] = S.Ered[i];
+        if (S.ovf) {
+          raw = true;
+        } else {
+          int lo = 0, hi = rcap;
+          while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (decide_pass(a, S, g, mid, Eall[mid], bnd, el2, rcst)) hi = mid;
+            else lo = mid + 1;
+          }
+          r = lo;
+          if (!pointwise && !decide_pass(a, S, g, r, Eall[r], bnd, el2, rcst)) raw = true;
+        }
+        __syncthreads();
+      }
+      if (!raw && !encode(r, false)) break;
       pc.mark(S, kPhSearch);
     }
     // a deferred record has no correction beyond kDeferMaxWk bits, its
     // escapes fit the slot's list and, when sparse, so does its entry list;
     // otherwise the block is encoded again into the CTA's scratch for the
-    // record writer here, with every element written when it has escapes
-    // (the writer lists escapes from k8 itself)
+    // record writer here
     // (the pass's counters are read into registers, and a barrier passed,
     // before another pass lets thread 0 reset them)
     if (!raw && in_slot) {
@@ -2903,14 +2749,10 @@ __global__ void __launch_bounds__(kTT, MINB) k_tile(const __grid_constant__ CUte
       const int kmax = S.kmax, ncorr = S.ncorr, nesc = S.nesc;
       const int wk = bit_width((uint32_t)kmax), ib = bit_width((uint32_t)(g.N - 1));
       const bool dense = wk > 0 && (g.N * wk + 31) / 32 < ((int64_t)ncorr * (ib + wk) + 31) / 32;
-      const SlotScratch sc = slot_scratch(r, g.n, g.L, g.N);
+      const SlotScratch sc = slot_scratch(r, g.n, g.L, g.N, pointwise);
       __syncthreads();
       if (wk > kDeferMaxWk || (!dense && ncorr > sc.list_cap) || nesc > sc.esc_cap)
-        if (!encode(r, false, nesc == 0, true)) break;
-    } else if (!raw && sparse) {
-      const int nesc = S.nesc;
-      __syncthreads();
-      if (nesc > 0 && !encode(r, false, false, true)) break;
+        if (!encode(r, true)) break;
     }
     const bool deferred = !raw && in_slot;
     // the next block's first chunks load while this record is packed
@@ -2918,8 +2760,8 @@ __global__ void __launch_bounds__(kTT, MINB) k_tile(const __grid_constant__ CUte
       const int64_t bn = S.bnext;
       if (bn < a.bhi) prefetch(a, tm, S, cu, bn, block_geom(P, P.b0 + bn), kLayoutRow);
     }
-    if (deferred) defer_record(a, S, g, bi, r, bitp);
-    else write_record(a, S, g, bi, raw, r, qs, k8, k32, bitp);
+    if (deferred) defer_record(a, S, g, bi, r, bits);
+    else write_record(a, S, g, bi, raw, r, qs, k8, k32, bits);
     pc.mark(S, kPhPack);
     if (tid == 0) S.ph[accepted ? kCntAccepted : kCntSearched] += 1;
   }

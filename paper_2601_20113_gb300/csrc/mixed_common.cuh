@@ -19,9 +19,10 @@ constexpr float kTwo24 = 16777216.0f;
 // exceeds its rounding error (a few ulps of |y|); otherwise the FP64 quotient
 // of the same c decides, so the result equals the FP64 definition.
 // The FP64 branch is rare and kept out of line, so the unrolled callers stay small.
-static __device__ __noinline__ int32_t quant_fp64(float c, double delta, int* ovf) {
+// (INT32_MIN for an overflow: an address would keep the caller's flag in memory.)
+static __device__ __noinline__ int32_t quant_fp64(float c, double delta) {
   const double Y = __ddiv_rn((double)c, delta);
-  if (!(fabs(Y) < 16777216.0)) { *ovf = 1; return 0; }
+  if (!(fabs(Y) < 16777216.0)) return INT32_MIN;
   return (int32_t)rint(Y);
 }
 __device__ __forceinline__ int32_t quant_exact(float c, double delta, float inv_delta, int& ovf) {
@@ -31,7 +32,9 @@ __device__ __forceinline__ int32_t quant_exact(float c, double delta, float inv_
   const float r = rintf(y);
   const float fr = fabsf(__fsub_rn(y, r));
   if (fr < 0.5f - m && ay < kTwo24 * 0.999999f) return (int32_t)r;
-  return quant_fp64(c, delta, &ovf);
+  const int32_t q = quant_fp64(c, delta);
+  if (q == INT32_MIN) ovf = 1;
+  return q == INT32_MIN ? 0 : q;
 }
 
 struct CorrConst {

@@ -56,7 +56,9 @@ SHAPES = [((32, 32, 16, 32), (16, 16, 16, 16)),        # the common block
           ((39, 27, 5, 21), (13, 9, 5, 7)),            # odd everything, order 7
           ((64, 40, 3, 16), (32, 32, 1, 16)),          # several chunks a plane
           ((40, 34, 4, 16), (20, 17, 4, 16)),          # ... that do not tile it
-          ((16, 8, 4, 33), (16, 8, 4, 11))]
+          ((16, 8, 4, 33), (16, 8, 4, 11)),
+          ((64, 48, 9, 20), (64, 48, 6, 16)),          # more points than the bitmap in shared memory holds
+          ((30, 22, 13, 4), (30, 22, 13, 3))]
 
 
 @pytest.mark.parametrize("dims,block", SHAPES)
