@@ -3,13 +3,14 @@
 // block of the usual shapes.  (Blocks with M_b < T_b go to k_mixed.cu.)
 //
 // Per block (Algorithm 1 step 3 of arXiv 2601.20113, pointwise-bound reading),
-// one CTA of 4 warps, several CTAs per SM, persistent over an atomic counter:
+// one CTA of 4 warps (the eigensolve: one warp), several CTAs per SM,
+// persistent over an atomic counter:
 //   Gram pass    the block streams through a two-stage shared-memory ring
 //                (TMA tensor tiles, or cp.async where the field's x extent is
 //                not 16-byte aligned); FP32 Gram G = A^T A (Sec. 2.7.1) and
 //                the block statistics
-//   eigensolve   register Jacobi in FP32 (one warp), one FP64 Ogita-Aishima
-//                refinement, and a Rayleigh-Ritz pass for tight bounds
+//   eigensolve   Jacobi in FP32 (one warp), an orthonormalisation by
+//                error-free transforms, and a Rayleigh-Ritz pass for tight bounds
 //   rank         predicted rank checked exactly, else the bisection of
 //                Algorithm 1 on E(r)
 //   encode pass  projection, quantization, decode, E(r-1), E(r), pointwise
@@ -36,6 +37,7 @@ constexpr int kHalf = kNP / 2;            // pairs per thread group (68)
 constexpr int kBitsSmem = 8 * NM * NM;    // bitmap words kept in shared memory (2048)
 constexpr int kGT = kTT / 2;              // threads per Gram group
 constexpr unsigned FULL = 0xffffffffu;
+constexpr int kEigLd = NM + 1;            // k_eig's row length: rows and columns spread over the banks
 // Bound of every wait on an mbarrier, in SM clock cycles (about a second):
 // a poll can return at once, so a bound in polls would be far shorter.
 constexpr long long kWaitCycles = 1ll << 31;
@@ -89,23 +91,13 @@ struct RowConst {
 struct __align__(1024) TileSmem {
   unsigned long long full[kStages];
   float G32[NM * NM];
-  float Vj[NM * NM];
   float red[kWarps][kNP + 8];
   __align__(16) float VstT[NM * NM];     // VstT[k * NM + j] = Vst[j][k]
   float vsum[NM];
-  // FP64 eigen scratch; from the encode pass through the record it holds the
-  // nonzero-correction bitmap of blocks of up to kBitsSmem * 32 points
-  union {
-    struct {
-      double G64[NM * NM], X64[NM * NM], R64[NM * NM], T64[NM * NM];
-    };
-    uint32_t bitsm[8 * NM * NM];
-  };
+  uint32_t bitsm[kBitsSmem];              // nonzero-correction bitmap of blocks of up to kBitsSmem * 32 points
   double lam_t[NM], lam[NM];
   float ered[kWarps][NM + 2];
   double Ered[NM + 2];
-  float featv[kMlpF];
-  float mh1[kMlpH];
   float st_min[kWarps], st_max[kWarps], st_tg[kWarps], st_xg[kWarps], st_rowmax[kWarps];
   int wq[NM];
   uint32_t qor[kWarps][NM];
@@ -120,7 +112,6 @@ struct __align__(1024) TileSmem {
   int sh32[32];
   int64_t colbase[NM + 1];
   unsigned long long ph[kPhases];   // cycle counters of this CTA (thread 0)
-  JacPairs jp;
   unsigned long long mma_bar;     // tcgen05.commit target
   uint32_t mma_phase;             // commits waited for so far (thread 0)
   int mma_pending;                // a wait for products timed out
@@ -182,6 +173,20 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src, bool valid
 }
 __device__ __forceinline__ void cp_async_arrive(unsigned long long* b) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+
+// The kernels' shared struct at the start of dynamic shared memory.  Functions
+// kept out of line take it from here, not from their caller: behind a
+// reference argument the compiler no longer knows the address space, and every
+// access becomes a generic one (16 384 blocks: k_enc 2.45 -> 2.38 ms).
+__device__ __forceinline__ TileSmem& tile_smem(unsigned char* smem_raw) {
+  // TMA destinations: align the tile ring to 1024 bytes explicitly
+  const uint32_t sbase = smem_u32(smem_raw);
+  return *reinterpret_cast<TileSmem*>(smem_raw + (((sbase + 1023u) & ~1023u) - sbase));
+}
+__device__ __forceinline__ TileSmem& tile_here() {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  return tile_smem(smem_raw);
 }
 
 // ---------------------------------------------------------------- tcgen05
@@ -398,14 +403,9 @@ __device__ bool stream_block(const TileArgs& a, const Maps& tm, TileSmem& S, Cur
   cu.pf_blk = -1;
   for (int c = 0; c < ch.n; ++c) {
     const bool in = __all_sync(FULL, wait_chunk(S, cu.con));
-    if (SYNC) {
-      if (__syncthreads_or(!in)) return false;
-      body(c, ch, &S.ring[cu.con % kStages][0]);
-      __syncthreads();
-    } else {
-      if (in) body(c, ch, &S.ring[cu.con % kStages][0]);
-      if (__syncthreads_or(!in)) return false;
-    }
+    if (SYNC && __syncthreads_or(!in)) return false;
+    if (in) body(c, ch, &S.ring[cu.con % kStages][0]);
+    if (__syncthreads_or(!in)) return false;
     ++cu.con;
     if (c + kStages < ch.n) issue_chunk(a, tm, S, bi, g, ch, c + kStages, cu.iss, layout);
   }
@@ -514,8 +514,9 @@ __device__ __forceinline__ void gram_entry(int grp, int q, int& i, int& j) {
 }
 
 template <bool PROJECT, int NF>
-__device__ __noinline__ bool pass_gram(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
+__device__ __noinline__ bool pass_gram(const TileArgs& a, const Maps& tm, TileSmem&, Cursor& cu, int64_t bi,
                           const Geom& g) {
+  TileSmem& S = tile_here();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int grp = tid / kGT, gt = tid % kGT;
   const int n = NF ? NF : g.n;
@@ -614,7 +615,6 @@ __device__ __noinline__ bool pass_gram(const TileArgs& a, const Maps& tm, TileSm
     gram_entry(p / kHalf, pp, i, j);
     if (i < n && j < n) {
       S.G32[i * NM + j] = v; S.G32[j * NM + i] = v;
-      S.G64[i * NM + j] = (double)v; S.G64[j * NM + i] = (double)v;
     }
   }
   __syncthreads();
@@ -646,8 +646,9 @@ __device__ __noinline__ bool pass_gram(const TileArgs& a, const Maps& tm, TileSm
 enum TcMode : int { kTcNone = 0, kTcTf32x3 = 1, kTcTf32 = 2, kTcBf16x3 = 3, kTcBf16 = 4 };
 __device__ __forceinline__ float tf32_trunc(float v) { return __uint_as_float(__float_as_uint(v) & 0xFFFFE000u); }
 
-__device__ __noinline__ bool pass_gram_tc(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
+__device__ __noinline__ bool pass_gram_tc(const TileArgs& a, const Maps& tm, TileSmem&, Cursor& cu, int64_t bi,
                                           const Geom& g, float* lo) {
+  TileSmem& S = tile_here();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = g.n;
   const int mode = a.tc_gram;
@@ -801,18 +802,10 @@ __device__ __noinline__ bool pass_gram_tc(const TileArgs& a, const Maps& tm, Til
     }
     __syncthreads();
   }
-  // symmetric from the upper triangle; FP64 copy; statistics
+  // symmetric from the upper triangle; statistics
   for (int e = tid; e < NM * NM; e += kTT) {
     const int i = e / NM, j = e % NM;
-    if (i < n && j < n) {
-      const float v = i <= j ? S.G32[i * NM + j] : S.G32[j * NM + i];
-      S.G64[e] = (double)v;
-    }
-  }
-  __syncthreads();
-  for (int e = tid; e < NM * NM; e += kTT) {
-    const int i = e / NM, j = e % NM;
-    if (i < n && j < n) S.G32[e] = (float)S.G64[e];
+    if (i > j && i < n) S.G32[e] = S.G32[j * NM + i];
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -828,115 +821,6 @@ __device__ __noinline__ bool pass_gram_tc(const TileArgs& a, const Maps& tm, Til
   __syncthreads();
   derived_stats(a, S, g, n);
   return true;
-}
-
-// ---------------------------------------------------------------- orthonormalisation
-// First-order orthonormalisation of the eigenvector matrix X (columns = modes;
-// all threads), into X64 for the ordering: X <- X + X R / 2, R = I - X^T X.
-// The FP32 Jacobi's rotations are orthogonal to a few ulps each, so its
-// eigenvectors are orthonormal to about 1e-5; the step takes that to its
-// square.  R is formed without rounding error that matters: each product
-// a b is split exactly into fl(a b) + fma(a, b, -fl(a b)) and the sums are
-// kept as unevaluated pairs (Knuth's two-sum), so R is exact to about 1e-14
-// with FP32 arithmetic alone (GB300's FP64 pipe is 1/64 of its FP32 rate);
-// the correction X R / 2, of size |R|, and the final rounding need only FP32.
-// With `rotate`, X = Vst W first (the Rayleigh-Ritz rotation of the first
-// basis, in FP32: its rounding is orthonormalised away with the rest).
-__device__ __noinline__ void orth_basis(TileSmem& S, int n, bool rotate) {
-  const int tid = threadIdx.x;
-  if (rotate) {
-    float* X = &S.red[0][0];                    // scratch (>= NM * NM floats)
-    static_assert(sizeof(S.red) >= NM * NM * sizeof(float), "scratch");
-    for (int e = tid; e < NM * NM; e += kTT) {
-      const int i = e / NM, j = e % NM;
-      float v = 0.0f;
-      if (i < n && j < n)
-        for (int k = 0; k < n; ++k) v = __fmaf_rn(S.VstT[k * NM + i], S.Vj[k * NM + j], v);
-      X[e] = v;
-    }
-    __syncthreads();
-    for (int e = tid; e < NM * NM; e += kTT) S.Vj[e] = X[e];
-    __syncthreads();
-  }
-  float* R = S.G32;                             // the Gram is not needed any more
-  for (int e = tid; e < NM * NM; e += kTT) {
-    const int i = e / NM, j = e % NM;
-    if (i < n && j < n && i <= j) {
-      float sh = 0.0f, sl = 0.0f;
-      for (int k = 0; k < n; ++k) {
-        const float x = S.Vj[k * NM + i], y = S.Vj[k * NM + j];
-        const float ph = __fmul_rn(x, y);
-        const float pl = __fmaf_rn(x, y, -ph);  // x y = ph + pl exactly
-        const float t = __fadd_rn(sh, ph);
-        const float bv = __fsub_rn(t, sh);
-        const float er = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bv)), __fsub_rn(ph, bv));   // sh + ph = t + er
-        sh = t;
-        sl = __fadd_rn(sl, __fadd_rn(er, pl));
-      }
-      // delta_ij - (sh + sl); 1 - sh is exact for sh in [1/2, 2]
-      const float r = i == j ? __fsub_rn(__fsub_rn(1.0f, sh), sl) : -__fadd_rn(sh, sl);
-      R[i * NM + j] = r;
-      R[j * NM + i] = r;
-    }
-  }
-  __syncthreads();
-  float xn[NM * NM / kTT];
-  int cnt = 0;
-  for (int e = tid; e < NM * NM; e += kTT, ++cnt) {
-    const int i = e / NM, j = e % NM;
-    xn[cnt] = 0.0f;
-    if (i < n && j < n) {
-      float c = 0.0f;
-      for (int k = 0; k < n; ++k) c = __fmaf_rn(S.Vj[i * NM + k], R[k * NM + j], c);
-      xn[cnt] = __fmaf_rn(0.5f, c, S.Vj[e]);
-    }
-  }
-  __syncthreads();
-  cnt = 0;
-  for (int e = tid; e < NM * NM; e += kTT, ++cnt) {
-    const int i = e / NM, j = e % NM;
-    if (i < n && j < n) S.X64[e] = (double)xn[cnt];
-  }
-  __syncthreads();
-}
-
-// Sort (stable, descending, lambda < 0 -> 0), sign-normalise, round to f32 (warp 0).
-__device__ void order_basis(TileSmem& S, int n, int lane) {
-  if (lane < n) {
-    const int k = lane;
-    double dk = S.lam_t[k];
-    dk = dk < 0.0 ? 0.0 : dk;
-    int pos = 0;
-    for (int j = 0; j < n; ++j) {
-      double dj = S.lam_t[j];
-      dj = dj < 0.0 ? 0.0 : dj;
-      if (dj > dk || (dj == dk && j < k)) ++pos;
-    }
-    int imax = 0;
-    double amax = -1.0;
-    for (int r = 0; r < n; ++r) {
-      const double av = fabs(S.X64[r * NM + k]);
-      if (av > amax) { amax = av; imax = r; }
-    }
-    const bool neg = S.X64[imax * NM + k] < 0.0;
-    S.lam[pos] = dk;
-    double cs = 0.0;
-    for (int r = 0; r < NM; ++r) {
-      float vf = 0.0f;
-      if (r < n) {
-        const double v = S.X64[r * NM + k];
-        vf = __double2float_rn(neg ? -v : v);
-        cs += (double)vf;
-      }
-      S.VstT[pos * NM + r] = vf;
-    }
-    S.vsum[pos] = (float)cs;
-  }
-  if (lane >= n && lane < NM) {
-    for (int r = 0; r < NM; ++r) S.VstT[lane * NM + r] = 0.0f;
-    S.vsum[lane] = 0.0f;
-  }
-  __syncwarp();
 }
 
 // ---------------------------------------------------------------- row arithmetic
@@ -1047,10 +931,11 @@ constexpr float kMagicF = 12582912.0f;              // 1.5 x 2^23
 constexpr int kMagicI = 0x4B400000;                 // its bits
 constexpr int kFastK = 59;
 template <int NP, bool POINT, int MC>
-__device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
+__device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSmem&, Cursor& cu, int64_t bi,
                                        const Geom& g, int r, const RowConst& rcst, const CorrConst& cc,
                                        int32_t* __restrict__ qs, int8_t* __restrict__ k8, int32_t* __restrict__ k32,
                                        uint32_t* bits) {
+  TileSmem& S = tile_here();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = MC ? NP : g.n, M = MC ? MC : (int)g.M, rc = MC ? 256 : a.rc;
   const RowConst rq = rcst;
@@ -1284,8 +1169,9 @@ __device__ __forceinline__ bool encode_rows(const TileArgs& a, const Maps& tm, T
 
 // E(r) for every r in [0, rcap] (FP32 estimates into S.Ered).
 template <int NF>
-__device__ __noinline__ bool pass_all_errors(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
+__device__ __noinline__ bool pass_all_errors(const TileArgs& a, const Maps& tm, TileSmem&, Cursor& cu, int64_t bi,
                                 const Geom& g, int rcap, const RowConst& rcst, int& ovf) {
+  TileSmem& S = tile_here();
   const int tid = threadIdx.x, n = NF ? NF : g.n;
   float E[NM + 1];
 #pragma unroll
@@ -1344,8 +1230,9 @@ __device__ __forceinline__ uint32_t bisection_probes(int target, int rcap) {
   return m;
 }
 template <int NF>
-__device__ __noinline__ bool pass_probe_errors(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
+__device__ __noinline__ bool pass_probe_errors(const TileArgs& a, const Maps& tm, TileSmem&, Cursor& cu, int64_t bi,
                                                const Geom& g, uint32_t mask, const RowConst& rcst) {
+  TileSmem& S = tile_here();
   const int tid = threadIdx.x, n = NF ? NF : g.n, rc = a.rc;
   const int kmax = 31 - __clz(mask);
   float E[kProbes];
@@ -1400,7 +1287,8 @@ __device__ __noinline__ bool pass_probe_errors(const TileArgs& a, const Maps& tm
 // rows once and accumulates every column's chunk sum; the chunk sums of a
 // group wait in the staging ring (idle between passes) and thread j adds
 // column j's in chunk order.
-__device__ __noinline__ double exact_error(const TileArgs& a, TileSmem& S, const Geom& g, int r, const RowConst& rcst) {
+__device__ __noinline__ double exact_error(const TileArgs& a, TileSmem&, const Geom& g, int r, const RowConst& rcst) {
+  TileSmem& S = tile_here();
   const int tid = threadIdx.x, n = g.n;
   const int64_t nch = cdiv(g.L, 32);
   double* part = reinterpret_cast<double*>(&S.ring[0][0]);      // kTT chunks x NM columns
@@ -1470,8 +1358,12 @@ __device__ bool decide_pass(const TileArgs& a, TileSmem& S, const Geom& g, int r
 // Warp 0: eigenvalue-tail rank estimate E(r) ~ sum_{i>=r} lambda_i + r L delta^2/12
 // and the 32 block features, one per lane (FP32; they only steer a prediction
 // that is then checked exactly).
-__device__ __noinline__ int predict_rank(const TileArgs& a, TileSmem& S, const Geom& g, int64_t bi, int rcap, double el2,
-                            double delta, int lane) {
+struct EigStats {
+  const double* lam;
+  const float *st_min, *st_max, *st_tg, *st_xg;
+};
+__device__ __forceinline__ int predict_rank(const TileArgs& a, const EigStats& S, float* featv, const Geom& g, int64_t bi,
+                                            int rcap, double el2, double delta, int lane) {
   const int n = g.n;
   double t = lane < n ? S.lam[lane] : 0.0;
 #pragma unroll
@@ -1507,7 +1399,7 @@ __device__ __noinline__ int predict_rank(const TileArgs& a, TileSmem& S, const G
   if (lane == 29) f = (float)((double)g.L * n / 65536.0);
   if (lane == 30) f = (float)n / 16.0f;
   if (lane == 31) f = (float)rp;
-  S.featv[lane] = f;
+  featv[lane] = f;
   if (a.feat) a.feat[bi * kMlpF + lane] = f;
   __syncwarp();
   return rp;
@@ -1936,8 +1828,9 @@ __device__ void record_prefix(TileSmem& S, const Geom& g, uint8_t* rec, int64_t 
 }
 
 // The whole record of block bi in its staging slot (k_compact moves it).
-__device__ __noinline__ void write_record(const TileArgs& a, TileSmem& S, const Geom& g, int64_t bi, bool raw, int r,
+__device__ __noinline__ void write_record(const TileArgs& a, TileSmem&, const Geom& g, int64_t bi, bool raw, int r,
                              int32_t* qs, const int8_t* k8, const int32_t* k32, const uint32_t* bits) {
+  TileSmem& S = tile_here();
   const int64_t L = g.L, N = g.N, M = g.M;
   uint8_t* rec = a.staging + align_up((g.pt_off - a.P.pt_base) * 4, 16) + 48 * bi;
   record_meta(a, S, g, bi, raw, r, false);
@@ -1979,8 +1872,9 @@ __device__ __noinline__ void write_record(const TileArgs& a, TileSmem& S, const 
 // A deferred record: metadata, then the prefix into the slot and the bitmap
 // after the q columns; k_pack_tile does the rest once the offsets are known.
 // Falls back to a raw record when the layout says so.
-__device__ __noinline__ void defer_record(const TileArgs& a, TileSmem& S, const Geom& g, int64_t bi, int r,
+__device__ __noinline__ void defer_record(const TileArgs& a, TileSmem&, const Geom& g, int64_t bi, int r,
                                           const uint32_t* bits) {
+  TileSmem& S = tile_here();
   uint8_t* slot = a.staging + align_up((g.pt_off - a.P.pt_base) * 4, 16) + 48 * bi;
   record_meta(a, S, g, bi, false, r, true);
   if (S.m.flags & kFlagRaw) {
@@ -1998,27 +1892,19 @@ __device__ __noinline__ void defer_record(const TileArgs& a, TileSmem& S, const 
 }
 
 // ---------------------------------------------------------------- the kernels
-// The eigensolver out of line: inline, it would share the kernel's registers
-// with the block state the body keeps live across it.
-__device__ __noinline__ void jacobi_tile(TileSmem& S, int n, float jfloor) {
-  if (n == NM) jacobi_cta<kTT, NM / 2>(S.G32, S.Vj, S.lam_t, n, jfloor, S.jp);
-  else jacobi_cta<kTT>(S.G32, S.Vj, S.lam_t, n, jfloor, S.jp);
-}
-
 // The compression of the tile route runs as phase kernels over all its
 // blocks:
 //   k_gram  the Gram pass and the block statistics (streams every block once);
-//   k_eig   the eigensolve, FP64 refinement, ordering and the rank prediction
-//           (no staging ring: many CTAs per SM hide its barriers and its
-//           FP64 latency);
-//   k_enc   the encode pass at the predicted rank, the exact acceptance test
-//           and the deferred record, for the blocks where all of that applies
-//           (learned or tail rank, pointwise bound, full blocks);
+//   k_eig   the eigensolve, orthonormalisation, ordering and the rank
+//           prediction, a warp a block;
+//   k_rrgram, k_eig<RR>  the Rayleigh-Ritz pass of the blocks that need it;
+//   k_enc   the row pass at the predicted rank, the exact acceptance test and
+//           the record, deferred where its slot has room (learned or tail rank);
 //   k_tile  every other block, from a list k_enc fills (or all blocks with
-//           the bisection): the Rayleigh-Ritz pass, the search, records that
-//           cannot be deferred.  It loads the state k_gram and k_eig left, so
-//           each block's basis, and so its stored bytes, do not depend on the
-//           kernel that writes its record.
+//           the bisection): the search, records that cannot be deferred.  It
+//           loads the state k_gram and k_eig left, so each block's basis, and
+//           so its stored bytes, do not depend on the kernel that writes its
+//           record.
 struct FastBlock {
   float G[NM * NM];                  // FP32 Gram, entries i, j < n
   float VstT[NM * NM];               // stored modes, VstT[k * NM + j] = Vst[j][k]
@@ -2110,60 +1996,15 @@ __device__ __forceinline__ float jacobi_floor(const TileArgs& a, const VarInfo& 
   return (float)(a.jfloor * (a.P.eb_type == DLS_EB_NRMSE ? el2 / g.n : vi.eb * vi.eb * (double)g.L));
 }
 
-// FP32 Jacobi, orthonormalisation of its eigenvectors, ordering, trace.
-// (An FP64 Ogita-Aishima refinement step took a third of the per-block time
-// and only improved eigenvector accuracy, whose effect on the energy a mode
-// captures is second order; the orthonormality of the stored modes is what
-// the method needs, and the re-orthonormalisation alone gives it.)
-__device__ void eigen_block(TileSmem& S, int n, float jfloor, PhaseClock& pc) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // the eigensolve starts from the identity: its result depends on this
-  // block's Gram alone, whichever blocks the CTA took before
-  jacobi_tile(S, n, jfloor);
-  pc.mark(S, kPhJacobi);
-  orth_basis(S, n, false);
-  if (warp == 0) {
-    order_basis(S, n, lane);
-    __syncwarp();
-    if (lane == 0) {
-      double tr = 0.0;
-      for (int i = 0; i < n; ++i) tr += S.lam[i];
-      S.lam_tr = tr;
-    }
-  }
-  __syncthreads();
-  pc.mark(S, kPhRefine);
+// |c_k| <= ||row|| (1 + 1e-4) for every column: no coefficient can reach 2^24
+// steps unless rowmax, the largest squared row norm, says so.
+__device__ __forceinline__ bool overflow_at(float rowmax, const VarInfo& vi) {
+  return !((double)sqrtf(rowmax) * 1.0001 < (16777216.0 * 0.999) * vi.delta);
 }
-
-// Tight bounds need the modes an FP32 Gram cannot resolve (eigenvalues near
-// 2^-24 trace G): a Rayleigh-Ritz step on the projected data fixes them, when
-// that resolution reaches half the per-mode budget eb^2 L.
-__device__ __forceinline__ bool rr_wanted(const TileSmem& S, const Plan& P, const VarInfo& vi, const Geom& g,
-                                          double el2) {
-  const double budget = (vi.eb * vi.eb) * (double)g.L;
-  const double noise = (P.eb_type == DLS_EB_NRMSE ? el2 / g.n : budget);
-  return g.n > 1 && 4.0 * 5.9604644775390625e-8 * S.lam_tr > 0.5 * noise;
-}
-
-// |c_k| <= ||row|| (1 + 1e-4) for every column: no coefficient can reach 2^24 steps.
 __device__ __forceinline__ bool overflow_possible(const TileSmem& S, const VarInfo& vi) {
   float rowmax = 0.0f;
   for (int w = 0; w < kWarps; ++w) rowmax = fmaxf(rowmax, S.st_rowmax[w]);
-  return !((double)sqrtf(rowmax) * 1.0001 / vi.delta < 16777216.0 * 0.999);
-}
-
-// The predicted rank (warp 0 computes, every thread returns it).
-__device__ int predicted_rank(const TileArgs& a, TileSmem& S, const Geom& g, int64_t bi, int rcap, double el2,
-                              double delta) {
-  const int lane = threadIdx.x & 31;
-  if (threadIdx.x < 32) {
-    const int rp = predict_rank(a, S, g, bi, rcap, el2, delta, lane);
-    int rm = rp;
-    if (a.learned == kRankMlp && a.model) rm = mlp_rank_warp(a.model, S.featv, S.mh1, lane, rcap);
-    if (lane == 0) S.r_pred = rm;
-  }
-  __syncthreads();
-  return S.r_pred;
+  return overflow_at(rowmax, vi);
 }
 
 // k_gram -> state: the Gram and the statistics of the block.
@@ -2178,38 +2019,6 @@ __device__ void store_gram(const TileSmem& S, FastBlock& f) {
     f.st_rowmax[tid] = S.st_rowmax[tid];
   }
   if (tid == 0) f.flags = S.nonfinite ? kFbNonfinite : 0;
-}
-// state -> k_eig: the Gram (and its FP64 copy) and the statistics.
-__device__ void load_gram(TileSmem& S, const FastBlock& f, int n) {
-  const int tid = threadIdx.x;
-  for (int e = tid; e < NM * NM; e += kTT) {
-    const float v = f.G[e];
-    S.G32[e] = v;
-    if (e / NM < n && e % NM < n) S.G64[e] = (double)v;
-  }
-  if (tid < kWarps) {
-    S.st_min[tid] = f.st_min[tid];
-    S.st_max[tid] = f.st_max[tid];
-    S.st_tg[tid] = f.st_tg[tid];
-    S.st_xg[tid] = f.st_xg[tid];
-    S.st_rowmax[tid] = f.st_rowmax[tid];
-  }
-  if (tid == 0) S.nonfinite = (f.flags & kFbNonfinite) ? 1 : 0;
-  __syncthreads();
-}
-// k_eig -> state: the ordered basis, eigenvalues, flags and predicted rank.
-__device__ void store_basis(const TileSmem& S, FastBlock& f, int32_t flags, int rpred) {
-  const int tid = threadIdx.x;
-  for (int e = tid; e < NM * NM; e += kTT) f.VstT[e] = S.VstT[e];
-  if (tid < NM) {
-    f.vsum[tid] = S.vsum[tid];
-    f.lam[tid] = S.lam[tid];
-  }
-  if (tid == 0) {
-    f.lam_tr = S.lam_tr;
-    f.flags = flags;
-    f.rpred = rpred;
-  }
 }
 // state -> k_enc / k_tile: everything the passes after the eigensolve read.
 __device__ void load_basis(TileSmem& S, const FastBlock& f) {
@@ -2282,12 +2091,6 @@ __device__ void alloc_tmem(TileSmem& S) {
   }
 }
 
-__device__ __forceinline__ TileSmem& tile_smem(unsigned char* smem_raw) {
-  // TMA destinations: align the tile ring to 1024 bytes explicitly
-  const uint32_t sbase = smem_u32(smem_raw);
-  return *reinterpret_cast<TileSmem*>(smem_raw + (((sbase + 1023u) & ~1023u) - sbase));
-}
-
 // ---------------------------------------------------------------- k_gram
 // The Gram pass of every block of the launch's range: FP32 Gram (or the
 // 3xTF32 tensor-core Gram) and statistics into the block's state.
@@ -2352,63 +2155,360 @@ __device__ __forceinline__ int64_t grab_rr(const TileArgs& a, unsigned long long
 // blocks whose coefficients might overflow for k_tile.
 // RR: the second solve of the Rayleigh-Ritz pass, on the flagged blocks, from
 // the Gram of their rows projected on the first basis (k_rrgram): the rotated
-// basis V = Vst W in FP64, orthonormalised, ordered, and the rank predicted.
-template <bool RR>
-// Twelve CTAs per SM (40 registers, 18 KB of shared memory each): the CTA
-// Jacobi waits at a barrier after every round, and more resident CTAs hide it
-// (16384 blocks of order 16: 0.95 ms at 5 CTAs per SM, 0.79 at 8, 0.69 at 12).
-__global__ void __launch_bounds__(kTT, 12) k_eig(const __grid_constant__ TileArgs a) {
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  TileSmem& S = tile_smem(smem_raw);       // only the part before the staging ring
-  const Plan& P = a.P;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  unsigned long long* ctr = RR ? &a.ctl->next_rre : &a.ctl->next_eig;
-  auto next = [&]() { return RR ? grab_rr(a, ctr) : grab_range(a, ctr); };
-  if (tid < kPhases) S.ph[tid] = 0;
-  if (tid == 0) {
-    S.nexact = 0;
-    S.bnext = next();
+// basis V = Vst W, orthonormalised, ordered, and the rank predicted.
+// A warp a block: the steps of a Jacobi round, and the serial ordering and
+// prediction, follow each other at a warp's own pace, and a block takes a
+// third of the instructions that four warps in step took (each of them ran
+// every round's loop for one or two of its 192 items).  Every entry is formed
+// by the same operations as jacobi_cta's and orth_basis's, so the bases are
+// theirs bit for bit.  Bound by the latency of a round (rotation, loads,
+// products, stores in turn): 16 384 blocks 0.68 -> 0.33 ms, 128 blocks 69 -> 50
+// us.
+struct EigWarp {
+  float A[NM * kEigLd], V[NM * kEigLd];    // A: the Gram, then R, then the stored modes (rows of NM)
+  JacPairs jp;
+  double lam[NM];
+  float lamf[NM], vsum[NM];
+  float st[5][kWarps];                     // st_min, st_max, st_tg, st_xg, st_rowmax
+  float featv[kMlpF], mh1[kMlpH];
+};
+
+// Whether a pair rotates: jacobi_cta's threshold max(1e-7 sqrt(a_pp a_qq),
+// 4 u max(a_pp, a_qq), floor).  4 u is 2.4e-7, so its first term never decides
+// unless the product overflows to infinity, which lets nothing rotate.
+__device__ __forceinline__ bool eig_above(float app, float aqq, float apq, float floor_abs) {
+  const float gpp = fabsf(app), gqq = fabsf(aqq);
+  const float thr = fmaxf(4.0f * 5.9604645e-8f * fmaxf(gpp, gqq), floor_abs);
+  return fabsf(apq) > thr && apq != 0.0f && !(__fmul_rn(gpp, gqq) == INFINITY);
+}
+// Its rotation (c, s, t), by jacobi_cta's functions.
+__device__ __forceinline__ void eig_rotation(float app, float aqq, float apq, float& c, float& s, float& t) {
+  const float theta = __fdividef(__fsub_rn(aqq, app), __fmul_rn(2.0f, apq));
+  if (fabsf(theta) > 1e18f) t = __fdividef(0.5f, theta);
+  else t = __fdividef(theta >= 0.0f ? 1.0f : -1.0f, __fadd_rn(fabsf(theta), __fsqrt_rn(__fmaf_rn(theta, theta, 1.0f))));
+  c = rsqrtf(__fmaf_rn(t, t, 1.0f));
+  s = __fmul_rn(t, c);
+}
+
+// jacobi_cta by one warp, on rows of kEigLd.  HF = 8 (order 16): a lane keeps
+// the column pair lane % 8 of a round and the row pairs lane / 8 and lane / 8 +
+// 4 of A, rows lane / 8 + 4 t of V, so that a round is one batch of
+// independent loads, products and stores.
+template <int HF>
+__device__ __forceinline__ void jacobi_warp32(EigWarp& W, int n, float floor_abs, int lane) {
+  const int m = HF ? 2 * HF : n + (n & 1), h = HF ? HF : m / 2;
+  float* A = W.A;
+  float* V = W.V;
+  for (int e = lane; e < NM * NM; e += 32) {
+    const int i = e / NM, j = e % NM;
+    V[i * kEigLd + j] = i == j ? 1.0f : 0.0f;
+    if (i >= n || j >= n) A[i * kEigLd + j] = 0.0f;
   }
-  __syncthreads();
-  PhaseClock pc;
+  // circle_pair's (a, b) of this lane: both move one place along the circle a
+  // round (a = m - 1 stays for lane 0)
+  int pa = lane == 0 ? m - 1 : lane, pb = lane == 0 ? 0 : m - 1 - lane;
+  __syncwarp();
+  for (int sweep = 0; sweep < 30 && n > 1; ++sweep) {
+    bool any = false;
+    for (int round = 0; round < m - 1; ++round) {
+      bool act = false;
+      const int p = min(pa, pb), q = max(pa, pb);
+      pa = lane == 0 ? pa : (pa + 1 == m - 1 ? 0 : pa + 1);
+      pb = pb + 1 == m - 1 ? 0 : pb + 1;
+      if (lane < h) {
+        const float app = A[p * kEigLd + p], aqq = A[q * kEigLd + q], apq = A[p * kEigLd + q];
+        float c = 1.0f, s = 0.0f, t = 0.0f;
+        act = eig_above(app, aqq, apq, floor_abs);
+        if (act) eig_rotation(app, aqq, apq, c, s, t);
+        W.jp.pq[lane] = p | q << 8 | (act ? 1 << 16 : 0);
+        W.jp.cs[lane] = make_float2(c, s);
+        W.jp.dg[lane] = make_float4(t, app, aqq, apq);
+      }
+      if (!__any_sync(FULL, act)) continue;
+      any = true;
+      __syncwarp();
+      // the 2 x 2 block (row pair k, column pair l) of A: J_k^T A_kl J_l
+      auto block = [&](int k, int l, const float2& csk, const float2& csl, float& a, float& b, float& c, float& d) {
+        const float ck = csk.x, sk = csk.y, cl = csl.x, sl = csl.y;
+        const float r1 = __fmaf_rn(ck, a, -__fmul_rn(sk, c)), r2 = __fmaf_rn(ck, b, -__fmul_rn(sk, d));
+        const float r3 = __fmaf_rn(sk, a, __fmul_rn(ck, c)), r4 = __fmaf_rn(sk, b, __fmul_rn(ck, d));
+        a = __fmaf_rn(cl, r1, -__fmul_rn(sl, r2));
+        b = __fmaf_rn(sl, r1, __fmul_rn(cl, r2));
+        c = __fmaf_rn(cl, r3, -__fmul_rn(sl, r4));
+        d = __fmaf_rn(sl, r3, __fmul_rn(cl, r4));
+        if (k == l) {
+          const float4 dg = W.jp.dg[k];      // (t, a_pp, a_qq, a_pq)
+          a = __fmaf_rn(-dg.x, dg.w, dg.y);
+          b = 0.0f;
+          c = 0.0f;
+          d = __fmaf_rn(dg.x, dg.w, dg.z);
+        }
+      };
+      if (HF == 8) {
+        const int l = lane & 7, k0 = lane >> 3;
+        const int jl = W.jp.pq[l], j0 = W.jp.pq[k0], j1 = W.jp.pq[k0 + 4];
+        const float2 csl = W.jp.cs[l], cs0 = W.jp.cs[k0], cs1 = W.jp.cs[k0 + 4];
+        const int pp = jl & 255, qq = (jl >> 8) & 255;
+        float* p0 = A + (j0 & 255) * kEigLd;
+        float* q0 = A + ((j0 >> 8) & 255) * kEigLd;
+        float* p1 = A + (j1 & 255) * kEigLd;
+        float* q1 = A + ((j1 >> 8) & 255) * kEigLd;
+        float a0 = p0[pp], b0 = p0[qq], c0 = q0[pp], d0 = q0[qq];
+        float a1 = p1[pp], b1 = p1[qq], c1 = q1[pp], d1 = q1[qq];
+        float x[4], y[4];
+        float* v = V + k0 * kEigLd;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          x[t] = v[4 * t * kEigLd + pp];
+          y[t] = v[4 * t * kEigLd + qq];
+        }
+        block(k0, l, cs0, csl, a0, b0, c0, d0);
+        block(k0 + 4, l, cs1, csl, a1, b1, c1, d1);
+        if ((j0 | jl) >> 16) { p0[pp] = a0; p0[qq] = b0; q0[pp] = c0; q0[qq] = d0; }
+        if ((j1 | jl) >> 16) { p1[pp] = a1; p1[qq] = b1; q1[pp] = c1; q1[qq] = d1; }
+        if (jl >> 16) {
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            v[4 * t * kEigLd + pp] = __fmaf_rn(csl.x, x[t], -__fmul_rn(csl.y, y[t]));
+            v[4 * t * kEigLd + qq] = __fmaf_rn(csl.y, x[t], __fmul_rn(csl.x, y[t]));
+          }
+        }
+      } else {
+        for (int it = lane; it < h * h; it += 32) {
+          const int k = it / h, l = it - k * h;
+          const int jk = W.jp.pq[k], jl = W.jp.pq[l];
+          if (!((jk | jl) >> 16)) continue;
+          const int p = (jk & 255) * kEigLd, q = ((jk >> 8) & 255) * kEigLd, pp = jl & 255, qq = (jl >> 8) & 255;
+          float a = A[p + pp], b = A[p + qq], c = A[q + pp], d = A[q + qq];
+          block(k, l, W.jp.cs[k], W.jp.cs[l], a, b, c, d);
+          A[p + pp] = a;
+          A[p + qq] = b;
+          A[q + pp] = c;
+          A[q + qq] = d;
+        }
+        for (int it = lane; it < n * h; it += 32) {
+          const int i = it / h, l = it - i * h;
+          const int jl = W.jp.pq[l];
+          if (!(jl >> 16)) continue;
+          const int p = jl & 255, q = (jl >> 8) & 255;
+          const float2 csl = W.jp.cs[l];
+          const float x = V[i * kEigLd + p], y = V[i * kEigLd + q];
+          V[i * kEigLd + p] = __fmaf_rn(csl.x, x, -__fmul_rn(csl.y, y));
+          V[i * kEigLd + q] = __fmaf_rn(csl.y, x, __fmul_rn(csl.x, y));
+        }
+      }
+      __syncwarp();
+    }
+    if (!any) break;
+    // after a sweep with rotations: stop if no pair is above its threshold now
+    bool up = false;
+#pragma unroll 4
+    for (int t = lane; t < n * n; t += 32) {
+      const int i = HF ? t / (2 * HF) : t / n, j = t - i * n;
+      if (i < j) up |= eig_above(A[i * kEigLd + i], A[j * kEigLd + j], A[i * kEigLd + j], floor_abs);
+    }
+    if (!__any_sync(FULL, up)) break;
+  }
+  if (lane < n) W.lamf[lane] = A[lane * kEigLd + lane];
+  __syncwarp();
+}
+
+// orth_basis's step by one warp: V <- V + V R / 2, R = I - V^T V by error-free
+// transforms; with `first` (global, rows of modes) V = Vst V before.
+template <int NF>
+__device__ __forceinline__ void orth_warp(EigWarp& W, int n_, const float* first, int lane) {
+  const int n = NF ? NF : n_;
+  float* A = W.A;
+  float* V = W.V;
+  float xn[NM * NM / 32];
+  if (first) {
+    for (int e = lane; e < NM * NM; e += 32) A[(e / NM) * kEigLd + e % NM] = first[e];
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < NM * NM / 32; ++t) {
+      const int e = lane + 32 * t, i = e / NM, j = e % NM;
+      float v = 0.0f;
+      if (i < n && j < n)
+        for (int k = 0; k < n; ++k) v = __fmaf_rn(A[k * kEigLd + i], V[k * kEigLd + j], v);
+      xn[t] = v;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < NM * NM / 32; ++t) {
+      const int e = lane + 32 * t;
+      V[(e / NM) * kEigLd + e % NM] = xn[t];
+    }
+    __syncwarp();
+  }
+  for (int e = lane; e < NM * (NM + 1) / 2; e += 32) {
+    // the upper triangle, row by row (136 entries: 4.25 rounds of the warp)
+    int i = 0, j = e;
+    while (j >= NM - i) { j -= NM - i; ++i; }
+    j += i;
+    if (i < n && j < n) {
+      float sh = 0.0f, sl = 0.0f;
+      for (int k = 0; k < n; ++k) {
+        const float x = V[k * kEigLd + i], y = V[k * kEigLd + j];
+        const float ph = __fmul_rn(x, y);
+        const float pl = __fmaf_rn(x, y, -ph);  // x y = ph + pl exactly
+        const float t = __fadd_rn(sh, ph);
+        const float bv = __fsub_rn(t, sh);
+        const float er = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bv)), __fsub_rn(ph, bv));   // sh + ph = t + er
+        sh = t;
+        sl = __fadd_rn(sl, __fadd_rn(er, pl));
+      }
+      const float r = i == j ? __fsub_rn(__fsub_rn(1.0f, sh), sl) : -__fadd_rn(sh, sl);
+      A[i * kEigLd + j] = r;
+      A[j * kEigLd + i] = r;
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int t = 0; t < NM * NM / 32; ++t) {
+    const int e = lane + 32 * t, i = e / NM, j = e % NM;
+    xn[t] = 0.0f;
+    if (i < n && j < n) {
+      float c = 0.0f;
+      for (int k = 0; k < n; ++k) c = __fmaf_rn(V[i * kEigLd + k], A[k * kEigLd + j], c);
+      xn[t] = __fmaf_rn(0.5f, c, V[i * kEigLd + j]);
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int t = 0; t < NM * NM / 32; ++t) {
+    const int e = lane + 32 * t;
+    V[(e / NM) * kEigLd + e % NM] = xn[t];
+  }
+  __syncwarp();
+}
+
+// order_basis by one warp (the values are floats, and compare as floats), the
+// stored modes into A as rows of NM.
+__device__ __forceinline__ void order_warp(EigWarp& W, int n, int lane) {
+  float* out = W.A;
+  if (lane < n) {
+    const int k = lane;
+    const float dk = W.lamf[k] < 0.0f ? 0.0f : W.lamf[k];
+    int pos = 0;
+    for (int j = 0; j < n; ++j) {
+      const float dj = W.lamf[j] < 0.0f ? 0.0f : W.lamf[j];
+      if (dj > dk || (dj == dk && j < k)) ++pos;
+    }
+    int imax = 0;
+    float amax = -1.0f;
+    for (int r = 0; r < n; ++r) {
+      const float av = fabsf(W.V[r * kEigLd + k]);
+      if (av > amax) { amax = av; imax = r; }
+    }
+    const bool neg = W.V[imax * kEigLd + k] < 0.0f;
+    W.lam[pos] = (double)dk;
+    double cs = 0.0;
+    for (int r = 0; r < NM; ++r) {
+      const float v = r < n ? W.V[r * kEigLd + k] : 0.0f;
+      const float vf = neg ? -v : v;
+      if (r < n) cs += widen(vf);
+      out[pos * NM + r] = r < n ? vf : 0.0f;
+    }
+    W.vsum[pos] = (float)cs;
+  }
+  if (lane >= n && lane < NM) {
+    for (int r = 0; r < NM; ++r) out[lane * NM + r] = 0.0f;
+    W.vsum[lane] = 0.0f;
+  }
+  __syncwarp();
+}
+
+template <bool RR>
+__global__ void __launch_bounds__(kTT, 10) k_eig(const __grid_constant__ TileArgs a) {
+  __shared__ __align__(16) EigWarp warps[kWarps];
+  const Plan& P = a.P;
+  const int lane = threadIdx.x & 31;
+  EigWarp& W = warps[threadIdx.x >> 5];
+  unsigned long long* ctr = RR ? &a.ctl->next_rre : &a.ctl->next_eig;
+  long long cyc[3] = {0, 0, 0}, t0 = 0;      // lane 0: Jacobi, refinement (RR: both), prediction
+  auto mark = [&](int i) {
+    const long long now = clock64();
+    cyc[i] += now - t0;
+    t0 = now;
+  };
   for (;;) {
-    const int64_t bi = S.bnext;
-    __syncthreads();
+    int64_t bi = 0;
+    if (lane == 0) bi = RR ? grab_rr(a, ctr) : grab_range(a, ctr);
+    bi = __shfl_sync(FULL, bi, 0);
     if (bi >= a.bhi) break;
-    if (tid == 0) S.bnext = next();
     const Geom g = block_geom(P, P.b0 + bi);
     const VarInfo vi = a.vars[g.v];
     const int n = g.n;
     const int rcap = P.rank_cap < n ? P.rank_cap : n;
     const double el2 = local_tol2(P, vi, g);
     FastBlock& f = a.fb[bi];
-    pc.start();
+    t0 = clock64();
     const int32_t flags0 = f.flags;
-    load_gram(S, f, n);
-    if (S.nonfinite) continue;                  // k_gram has set the status
+    if (flags0 & kFbNonfinite) continue;         // k_gram has set the status
+    __syncwarp();
+    for (int e = lane; e < NM * NM; e += 32) W.A[(e / NM) * kEigLd + e % NM] = f.G[e];
+    if (lane < kWarps) {
+      W.st[0][lane] = f.st_min[lane];
+      W.st[1][lane] = f.st_max[lane];
+      W.st[2][lane] = f.st_tg[lane];
+      W.st[3][lane] = f.st_xg[lane];
+      W.st[4][lane] = f.st_rowmax[lane];
+    }
+    __syncwarp();
     const float jfloor = jacobi_floor(a, vi, g, el2);
+    if (n == NM) jacobi_warp32<NM / 2>(W, n, jfloor, lane);
+    else jacobi_warp32<0>(W, n, jfloor, lane);
+    mark(0);
+    if (n == NM) orth_warp<NM>(W, n, RR ? f.VstT : nullptr, lane);
+    else orth_warp<0>(W, n, RR ? f.VstT : nullptr, lane);
+    order_warp(W, n, lane);
+    double tr = f.lam_tr;
+    if (!RR) {
+      tr = 0.0;
+      for (int i = 0; i < n; ++i) tr += W.lam[i];
+    }
+    mark(1);
     int32_t flags = 0;
     if (RR) {
-      load_basis(S, f);                         // the first basis
-      jacobi_tile(S, n, jfloor);
-      // V = Vst W, orthonormalised; eigenvalues from the Rayleigh-Ritz diagonal
-      orth_basis(S, n, true);
-      if (warp == 0) order_basis(S, n, lane);
-      __syncthreads();
-      pc.mark(S, kPhRR);
       flags = flags0 & ~kFbRR;
     } else {
-      eigen_block(S, n, jfloor, pc);
-      if (rr_wanted(S, P, vi, g, el2)) flags |= kFbRR;
-      if (overflow_possible(S, vi)) flags |= kFbOverflow;
+      // modes an FP32 Gram cannot resolve (rr_wanted), coefficients that might overflow
+      const double noise = P.eb_type == DLS_EB_NRMSE ? el2 / n : (vi.eb * vi.eb) * (double)g.L;
+      if (n > 1 && 4.0 * 5.9604644775390625e-8 * tr > 0.5 * noise) flags |= kFbRR;
+      float rowmax = 0.0f;
+      for (int w = 0; w < kWarps; ++w) rowmax = fmaxf(rowmax, W.st[4][w]);
+      if (overflow_at(rowmax, vi)) flags |= kFbOverflow;
     }
     int rp = 0;
-    if (!(flags & kFbRR)) rp = predicted_rank(a, S, g, bi, rcap, el2, vi.delta);
-    pc.mark(S, kPhPredict);
-    store_basis(S, f, flags, rp);
-    __syncthreads();
+    if (!(flags & kFbRR)) {
+      const EigStats st{W.lam, W.st[0], W.st[1], W.st[2], W.st[3]};
+      rp = predict_rank(a, st, W.featv, g, bi, rcap, el2, vi.delta, lane);
+      if (a.learned == kRankMlp && a.model) rp = mlp_rank_warp(a.model, W.featv, W.mh1, lane, rcap);
+    }
+    mark(2);
+    for (int e = lane; e < NM * NM; e += 32) f.VstT[e] = W.A[e];
+    if (lane < NM) {
+      f.vsum[lane] = W.vsum[lane];
+      f.lam[lane] = W.lam[lane];
+    }
+    if (lane == 0) {
+      f.lam_tr = tr;
+      f.flags = flags;
+      f.rpred = rp;
+    }
+    __syncwarp();
   }
-  flush_phases(a, S);
+  // CTA-cycles: a CTA runs kWarps blocks at a time
+  if (lane == 0 && a.phase) {
+    unsigned long long* ph = &a.phase[(int64_t)(blockIdx.x % a.ctas) * kPhases];
+    if (RR) {
+      atomicAdd(&ph[kPhRR], (unsigned long long)(cyc[0] + cyc[1]) / kWarps);
+    } else {
+      atomicAdd(&ph[kPhJacobi], (unsigned long long)cyc[0] / kWarps);
+      atomicAdd(&ph[kPhRefine], (unsigned long long)cyc[1] / kWarps);
+    }
+    atomicAdd(&ph[kPhPredict], (unsigned long long)cyc[2] / kWarps);
+  }
 }
 
 // ---------------------------------------------------------------- k_rrgram
@@ -2576,7 +2676,7 @@ __global__ void __launch_bounds__(kTT, MINB) k_tile(const __grid_constant__ CUte
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   TileSmem& S = tile_smem(smem_raw);
   const Maps tm{&tmap, &tmapg};
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   int32_t* qs = a.q_scr + (int64_t)blockIdx.x * NM * a.lmax;
   int8_t* k8 = a.k8_scr + (int64_t)blockIdx.x * a.nptmax;
   int32_t* k32 = a.k32_scr + (int64_t)blockIdx.x * a.nptmax;
@@ -2614,29 +2714,10 @@ __global__ void __launch_bounds__(kTT, MINB) k_tile(const __grid_constant__ CUte
 
     pc.start();
     const bool full = n == NM;   // Gram order 16: the passes without per-column predicates
-    const float jfloor = jacobi_floor(a, vi, g, el2);
     load_basis(S, a.fb[bi]);
     if (S.nonfinite) continue;                  // k_gram has set the status
     prefetch(a, tm, S, cu, bi, g, kLayoutRow);
-    // the Rayleigh-Ritz pass, if k_rrgram and k_eig<true> have not done it
-    bool did_rr = false;
-    if (a.fb[bi].flags & kFbRR) {
-      did_rr = true;
-      if (!(full ? pass_gram<true, NM>(a, tm, S, cu, bi, g) : pass_gram<true, 0>(a, tm, S, cu, bi, g))) break;
-      prefetch(a, tm, S, cu, bi, g, kLayoutRow);
-      jacobi_tile(S, n, jfloor);
-      // V = Vst W, orthonormalised; eigenvalues from the Rayleigh-Ritz diagonal
-      orth_basis(S, n, true);
-      if (warp == 0) order_basis(S, n, lane);
-      __syncthreads();
-    }
-    pc.mark(S, kPhRR);
-
     const bool may_overflow = overflow_possible(S, vi);
-    // the prediction k_eig made, unless the Rayleigh-Ritz pass changed the basis
-    if (did_rr) predicted_rank(a, S, g, bi, rcap, el2, vi.delta);
-    pc.mark(S, kPhPredict);
-
     // the row pass at rank rr, into the block's staging slot (deferred packing)
     // when the rank leaves room, else into the CTA's scratch
     uint32_t* const bits = g.N <= (int64_t)kBitsSmem * 32 ? S.bitsm : bit_scr;
@@ -2937,9 +3018,6 @@ size_t tile_smem_bytes(bool tc) {
   return 1024 + (size_t)align_up((int64_t)sizeof(TileSmem), 1024) + (tc ? (size_t)kStageFloats * 4 : 0);
 }
 
-// Dynamic shared memory of k_eig: the shared struct up to the staging ring.
-size_t eig_smem_bytes() { return 1024 + (size_t)offsetof(TileSmem, ring); }
-
 // The device's per-SM limits, read once a device (cudaGetDeviceProperties
 // fills in far more and took tens of microseconds at every launch).
 struct SmLimits {
@@ -3119,6 +3197,12 @@ int launch_tile_compress(const Plan& p, const void* d_in, const MixedWork& w, in
     if (c > nblk) c = nblk;
     return (int)(c > 0 ? c : 1);
   };
+  // k_eig: a warp a block, spread over the SMs first (a CTA an SM takes up to
+  // kWarps blocks only when there are more blocks than SMs)
+  auto eig_grid = [&](int per_sm) -> int {
+    const int64_t c = (int64_t)sms * per_sm;
+    return (int)(nblk < c ? nblk : c);
+  };
   const bool tc = a.tc_gram != 0;
   // counters and list of this launch
   if (cudaMemsetAsync(a.ctl, 0, sizeof(FastCtl), s) != cudaSuccess) return DLS_ERR_CUDA;
@@ -3136,23 +3220,21 @@ int launch_tile_compress(const Plan& p, const void* d_in, const MixedWork& w, in
   }
   // 2. eigensolve and prediction (no staging ring: more CTAs per SM)
   {
-    const size_t sm = eig_smem_bytes();
-    const int per = ctas_per_sm_of(k_eig<false>, sm, false);
+    const int per = ctas_per_sm_of(k_eig<false>, 0, false);
     cudaGetLastError();
     if (per < 1) return DLS_ERR_CUDA;
-    k_eig<false><<<grid_of(per, 0), kTT, sm, s>>>(a);
+    k_eig<false><<<eig_grid(per), kTT, 0, s>>>(a);
     if (!mark(1)) return DLS_ERR_CUDA;
   }
   // 2b. the Rayleigh-Ritz pass of the flagged blocks: projected Gram, second solve
   {
     const size_t tsm0 = tile_smem_bytes(false);
     const int per = ctas_per_sm_of(k_rrgram<4>, tsm0, false);
-    const size_t sm = eig_smem_bytes();
-    const int pere = ctas_per_sm_of(k_eig<true>, sm, false);
+    const int pere = ctas_per_sm_of(k_eig<true>, 0, false);
     cudaGetLastError();
     if (per < 1 || pere < 1) return DLS_ERR_CUDA;
     k_rrgram<4><<<grid_of(per, w.ctas), kTT, tsm0, s>>>(tmap, tmapg, a);
-    k_eig<true><<<grid_of(pere, 0), kTT, sm, s>>>(a);
+    k_eig<true><<<eig_grid(pere), kTT, 0, s>>>(a);
     if (!mark(2)) return DLS_ERR_CUDA;
   }
   // 3. encode pass and deferred record at the predicted rank
