@@ -390,14 +390,14 @@ __global__ void __launch_bounds__(256) k_gb_norm(GbPlan g, const float* __restri
 #pragma unroll
     for (int k = 0; k < kAhead; ++k) {
       bad |= not_finite(b[k]);
-      const double x = widen(b[k]);
+      const double x = widen_stream(b[k]);
       s = __fma_rn(x, x, s);
     }
   }
   for (; i < i1; i += 256) {
     const float b = __ldg(in + i);
     bad |= not_finite(b);
-    const double x = widen(b);
+    const double x = widen_stream(b);
     s = __fma_rn(x, x, s);
   }
   __shared__ double sh[256];

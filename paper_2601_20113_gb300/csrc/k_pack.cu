@@ -282,14 +282,14 @@ __global__ void __launch_bounds__(256) k_stats(Plan P, const T* __restrict__ in,
 #pragma unroll
     for (int k = 0; k < kAhead; ++k) {
       ra.add(b[k]);
-      const double xv = widen(b[k]);
+      const double xv = widen_stream(b[k]);
       s = __fma_rn(xv, xv, s);
     }
   }
   for (; i < i1; i += 256) {
     const T b = __ldg(x + i);
     ra.add(b);
-    const double xv = widen(b);
+    const double xv = widen_stream(b);
     s = __fma_rn(xv, xv, s);
   }
   __shared__ double ss[256];

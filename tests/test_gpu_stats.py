@@ -72,3 +72,17 @@ def test_non_finite_values_are_refused(bad, bound, dtype):
     with pytest.raises(dls.DlsError) as e:
         dls.compress(f, (2, 2, 1, 2), 1e-2, bound)
     assert e.value.status == -3
+
+
+@pytest.mark.parametrize("scale", [1e-38, 1e-40, 1e-44])
+def test_subnormal_values_are_summed_exactly(scale):
+    """Squares of subnormals, alone and beside the smallest normal values: sums of few terms, exact in any order."""
+    shape = (1, 2, 1, 16, 300)
+    f = torch.zeros(shape, dtype=torch.float32, device="cuda")
+    flat = f.view(-1)
+    vals = torch.tensor([scale, -3 * scale, 1.1754943508222875e-38, 0.0, -0.0], dtype=torch.float32)
+    flat[::2000] = vals.cuda()
+    p = dls.make_params(shape, torch.float32, (2, 2, 1, 2), 1.0, dls.EB_NRMSE)
+    x = vals.numpy().astype(np.float64)
+    got = dls.field_stats(p, f)[0]
+    assert got[2] == pytest.approx(float(np.sum(x * x)), rel=5 * 2.0 ** -52)
