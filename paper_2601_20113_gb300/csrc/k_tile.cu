@@ -233,9 +233,10 @@ struct Chunks {
   int ncy, ncz, n;
 };
 __device__ __forceinline__ Chunks chunks_of(const TileArgs& a, const Geom& g) {
+  // (32-bit quotients; mostly the chunk holds the block's whole y extent)
   Chunks c;
-  c.ncy = (int)cdiv(g.sy, a.yc);
-  c.ncz = (int)cdiv(g.sz, a.zc);
+  c.ncy = g.sy <= a.yc ? 1 : (int)((uint32_t)(g.sy + a.yc - 1) / (uint32_t)a.yc);
+  c.ncz = a.zc == 1 ? g.sz : (int)((uint32_t)(g.sz + a.zc - 1) / (uint32_t)a.zc);
   c.n = c.ncy * c.ncz;
   return c;
 }
@@ -939,6 +940,12 @@ __device__ __forceinline__ ChunkRows chunk_rows(const TileArgs& a, const Geom& g
 constexpr float kMagicF = 12582912.0f;              // 1.5 x 2^23
 constexpr int kMagicI = 0x4B400000;                 // its bits
 constexpr int kFastK = 59;
+// max(m, |a|, |b|), a NaN if one is (so that no comparison settles a row with one)
+__device__ __forceinline__ float max_abs_nan(float m, float a, float b) {
+  float r;
+  asm("{\n.reg .f32 x, y;\nabs.f32 x, %2;\nabs.f32 y, %3;\nmax.NaN.f32 %0, x, y;\nmax.NaN.f32 %0, %0, %1;\n}" : "=f"(r) : "f"(m), "f"(a), "f"(b));
+  return r;
+}
 template <int NP, bool POINT, int MC>
 __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSmem&, Cursor& cu, int64_t bi,
                                        const Geom& g, int r, const RowConst& rcst, const CorrConst& cc,
@@ -963,7 +970,8 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
   const float2 inv2 = make_float2(cc.inv_step_f, cc.inv_step_f), step2 = make_float2(cc.step_f, cc.step_f);
   float2 e1 = make_float2(0.0f, 0.0f), e2 = make_float2(0.0f, 0.0f);
   uint32_t qor_lane = 0, kmx = 0;
-  int nc = 0, ne = 0, ovf = 0, zmx = kMagicI, zmn = kMagicI;
+  int nc = 0, ne = 0, ovf = 0;
+  float zmx = 0.0f, zmn = 0.0f;
   const uint32_t msx = MC ? 0u : (g.sx > 1 ? 0xFFFFFFFFu / (uint32_t)g.sx + 1u : 0u);
   const bool ok = stream_block(a, tm, S, cu, bi, g, kLayoutRow, [&](int c, const Chunks& ch, const float* tile) {
     ChunkRows cr;
@@ -1055,7 +1063,7 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
       }
       // corrections
       int zi[NP];
-      bool settled = true;
+      float hi = 0.0f, lo = 0.0f, fmx = 0.0f, dmx = 0.0f;       // ranges (three-operand minima and maxima)
 #pragma unroll
       for (int j = 0; j < NP; j += 2) {
         const float2 x2 = make_float2(x[j], x[j + 1]), h2 = make_float2(acc[j], acc[j + 1]);
@@ -1069,19 +1077,15 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
         const float2 dd = __ffma2_rn(xt, m1, x2);
         zi[j] = __float_as_int(z.x);
         zi[j + 1] = __float_as_int(z.y);
-        settled = settled && fabsf(fr.x) < 0.49997f && fabsf(fr.y) < 0.49997f && fabsf(dd.x) <= eb_lo &&
-                  fabsf(dd.y) <= eb_lo;
-      }
-      int hi = zi[0], lo = zi[0];
-#pragma unroll
-      for (int j = 1; j < NP; ++j) {
-        hi = max(hi, zi[j]);
-        lo = min(lo, zi[j]);
+        hi = fmaxf(fmaxf(hi, k.x), k.y);
+        lo = fminf(fminf(lo, k.x), k.y);
+        fmx = max_abs_nan(fmx, fr.x, fr.y);
+        dmx = max_abs_nan(dmx, dd.x, dd.y);
       }
       uint32_t escm = 0;
-      if (settled && hi <= kMagicI + kFastK && lo >= kMagicI - kFastK) {
-        zmx = max(zmx, hi);
-        zmn = min(zmn, lo);
+      if (fmx < 0.49997f && dmx <= eb_lo && hi <= (float)kFastK && lo >= -(float)kFastK) {
+        zmx = fmaxf(zmx, hi);
+        zmn = fminf(zmn, lo);
       } else {
         // one by one, by the definition where FP32 leaves it open
 #pragma unroll 1
@@ -1141,7 +1145,7 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
     }
   });
   if (!ok) return false;
-  kmx |= max(zigzag(zmx - kMagicI), zigzag(zmn - kMagicI));
+  kmx |= max(zigzag((int32_t)zmx), zigzag((int32_t)zmn));
   nc = __reduce_add_sync(FULL, nc);
   ne = __reduce_add_sync(FULL, ne);
   kmx = __reduce_or_sync(FULL, kmx);
@@ -2631,7 +2635,7 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
     bool accepted = false, low = false;
     if (!S.ovf) {
       const Chunks chk = chunks_of(a, g);
-      const double bnd = (double)(cdiv(a.rc, kTT) * chk.n * g.n + 40) * 6.6e-8;
+      const double bnd = (double)(((a.rc + kTT - 1) / kTT) * chk.n * g.n + 40) * 6.6e-8;
       const double E_rm1 = S.Ered[0], E_r = S.Ered[1];
       const bool p_r = decide_pass(a, S, g, rp, E_r, bnd, el2, rcst);
       low = !p_r;
@@ -2745,8 +2749,7 @@ __global__ void __launch_bounds__(kTT, MINB) k_tile(const __grid_constant__ CUte
                        : encode_rows<false>(a, tm, S, cu, bi, g, rr, rcst, cc, q, k, k32, bits);
     };
     const Chunks chk = chunks_of(a, g);
-    const int64_t rows_per_thread = cdiv(a.rc, kTT) * chk.n;
-    const double bnd = (double)(rows_per_thread * n + 40) * 6.6e-8;
+    const double bnd = (double)(((a.rc + kTT - 1) / kTT) * chk.n * n + 40) * 6.6e-8;
     bool accepted = false;
     int r = 0;
     if (a.learned != kRankSearch && !may_overflow && !(a.fb[bi].flags & kFbRankFail)) {
