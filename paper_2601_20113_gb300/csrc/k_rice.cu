@@ -67,25 +67,32 @@ __device__ bool corr_src(const Geom& g, const uint8_t* rec, int es, CorrSrc& s) 
   return true;
 }
 
-
-// A warp's view of one chunk in shared memory: mask[L] holds the nonzeros of
-// elements c0 + 32 L .. c0 + 32 L + 31 (lane L's part), z[33 L + i] the
-// zigzag value of element c0 + 32 L + i where its bit is set (escapes are
-// zeros in both source forms).
+// A warp's buffer for one chunk: the zigzag values of its nonzeros (escapes
+// are zeros in both source forms), lane L's 32 elements at z[33 L ..] or, up
+// to eight bits ("narrow"), as bytes at 36 L, which leaves kStageWords words
+// for the coded chunk; and the lanes' nonzero masks of an entry list.
+constexpr int kByteWords = 288;            // 32 lanes of 36 bytes
+constexpr int kStageWords = 33 * 32 - kByteWords;
 struct WarpChunk {
   uint32_t mask[32];
   uint32_t z[32 * 33];
+  __device__ uint8_t* bytes() { return reinterpret_cast<uint8_t*>(z); }
+  __device__ uint32_t* stage() { return z + kByteWords; }
 };
 
 // Lane L's 32 dense fields of width WK (compile time): WK words from p, of
-// which the first cnt fields are the chunk's.
-template <int WK>
-__device__ __forceinline__ uint32_t dense_fields(const uint32_t* p, int cnt, uint32_t* z) {
+// which the first cnt fields are the chunk's.  Stores the values (STORE), or
+// collects the bits of value - 1; returns the nonzeros' mask.
+template <int WK, bool STORE>
+__device__ __forceinline__ uint32_t dense_fields(const uint32_t* p, int cnt, uint8_t* z, uint32_t& vor) {
   uint32_t w[WK];
-  const int nw = (cnt * WK + 31) >> 5;
 #pragma unroll
-  for (int k = 0; k < WK; ++k) w[k] = k < nw ? p[k] : 0u;
-  uint32_t m = 0;
+  for (int k = 0; k < WK; ++k) {
+    const int nb = cnt * WK - 32 * k;      // the chunk's bits from word k on
+    w[k] = nb > 0 ? p[k] : 0u;
+    if (nb > 0 && nb < 32) w[k] &= (1u << nb) - 1u;
+  }
+  uint32_t m = 0, four = 0;
 #pragma unroll
   for (int i = 0; i < 32; ++i) {
     constexpr uint32_t fm = (1u << WK) - 1u;
@@ -93,48 +100,50 @@ __device__ __forceinline__ uint32_t dense_fields(const uint32_t* p, int cnt, uin
     uint32_t f = w[k] >> sh;
     if (sh + WK > 32) f |= w[k + 1] << (32 - sh);
     f &= fm;
-    if (i < cnt && f != 0u) {
+    if (f != 0u) {
       m |= 1u << i;
-      z[i] = f;
+      if (!STORE) vor |= f - 1u;
+    }
+    if (STORE) {
+      four = i & 3 ? four | f << (8 * (i & 3)) : f;
+      if ((i & 3) == 3) reinterpret_cast<uint32_t*>(z)[i >> 2] = four;
     }
   }
   return m;
 }
 
-// Fills the warp's view of chunk [c0, c1) (all lanes of the warp); an
-// entry-list source's entries of the chunk are [lo, hi).
-__device__ void load_chunk(const CorrSrc& s, int64_t c0, int64_t c1, int64_t lo, int64_t hi, int lane,
-                           WarpChunk& V) {
-  if (s.dense && s.wk <= 8) {
-    const int64_t e0 = c0 + 32 * (int64_t)lane;
-    const int cnt = e0 >= c1 ? 0 : (int)((c1 - e0) < 32 ? (c1 - e0) : 32);
+// The nonzeros' mask of lane `lane`'s 32 elements of chunk [c0, c1) (all lanes
+// of the warp); an entry-list source's entries of the chunk are [lo, hi).
+// STORE: with their values in V; otherwise vor |= value - 1 of the warp's.
+template <bool STORE>
+__device__ uint32_t load_chunk(const CorrSrc& s, int64_t c0, int64_t c1, int64_t lo, int64_t hi, int lane,
+                               WarpChunk& V, uint32_t& vor) {
+  const int64_t e0 = c0 + 32 * (int64_t)lane;
+  const int cnt = e0 >= c1 ? 0 : (int)((c1 - e0) < 32 ? (c1 - e0) : 32);
+  const bool narrow = s.wk <= 8;
+  uint32_t m = 0;
+  if (s.dense && narrow) {
     const uint32_t* p = s.cw + (e0 >> 5) * s.wk;
-    uint32_t* z = V.z + 33 * lane;
-    uint32_t m = 0;
+    uint8_t* z = V.bytes() + 36 * lane;
     switch (s.wk) {
-      case 1: m = dense_fields<1>(p, cnt, z); break;
-      case 2: m = dense_fields<2>(p, cnt, z); break;
-      case 3: m = dense_fields<3>(p, cnt, z); break;
-      case 4: m = dense_fields<4>(p, cnt, z); break;
-      case 5: m = dense_fields<5>(p, cnt, z); break;
-      case 6: m = dense_fields<6>(p, cnt, z); break;
-      case 7: m = dense_fields<7>(p, cnt, z); break;
-      default: m = dense_fields<8>(p, cnt, z); break;
+      case 1: m = dense_fields<1, STORE>(p, cnt, z, vor); break;
+      case 2: m = dense_fields<2, STORE>(p, cnt, z, vor); break;
+      case 3: m = dense_fields<3, STORE>(p, cnt, z, vor); break;
+      case 4: m = dense_fields<4, STORE>(p, cnt, z, vor); break;
+      case 5: m = dense_fields<5, STORE>(p, cnt, z, vor); break;
+      case 6: m = dense_fields<6, STORE>(p, cnt, z, vor); break;
+      case 7: m = dense_fields<7, STORE>(p, cnt, z, vor); break;
+      default: m = dense_fields<8, STORE>(p, cnt, z, vor); break;
     }
-    V.mask[lane] = m;
-    __syncwarp();
-    return;
+    return m;                              // (a lane reads its own values)
   }
   if (s.dense) {
     // lane L's 32 fields start at bit (c0 + 32 L) wk: a word boundary
-    const int64_t e0 = c0 + 32 * (int64_t)lane;
-    const int cnt = e0 >= c1 ? 0 : (int)((c1 - e0) < 32 ? (c1 - e0) : 32);
     const int wk = s.wk;
     const uint64_t fm = wk >= 32 ? 0xFFFFFFFFull : ((1ull << wk) - 1ull);
     const uint32_t* p = s.cw + (e0 >> 5) * wk;
     uint64_t buf = 0;
     int nb = 0;
-    uint32_t m = 0;
     for (int i = 0; i < cnt; ++i) {
       if (nb < wk) {
         buf |= (uint64_t)(*p++) << nb;
@@ -145,12 +154,11 @@ __device__ void load_chunk(const CorrSrc& s, int64_t c0, int64_t c1, int64_t lo,
       nb -= wk;
       if (z != 0u) {
         m |= 1u << i;
-        V.z[33 * lane + i] = z;
+        if (STORE) V.z[33 * lane + i] = z;
+        else vor |= z - 1u;
       }
     }
-    V.mask[lane] = m;
-    __syncwarp();
-    return;
+    return m;
   }
   V.mask[lane] = 0u;
   __syncwarp();
@@ -159,10 +167,14 @@ __device__ void load_chunk(const CorrSrc& s, int64_t c0, int64_t c1, int64_t lo,
     const uint64_t pos = (uint64_t)j * W;
     const int d = (int)((int64_t)rd_bits(s.cw, pos, s.ib) - c0);
     if (d < 0 || d >= kRiceChunk) continue;     // entries are the chunk's (the packers sort them)
+    const uint32_t z = rd_bits(s.cw, pos + s.ib, s.wk);
     atomicOr(&V.mask[d >> 5], 1u << (d & 31));
-    V.z[33 * (d >> 5) + (d & 31)] = rd_bits(s.cw, pos + s.ib, s.wk);
+    if (!STORE) vor |= z - 1u;
+    else if (narrow) V.bytes()[36 * (d >> 5) + (d & 31)] = (uint8_t)z;
+    else V.z[33 * (d >> 5) + (d & 31)] = z;
   }
   __syncwarp();
+  return V.mask[lane];
 }
 
 // Entry-list sources: every chunk's first entry into chunks[c].first (all
@@ -192,55 +204,51 @@ __device__ __forceinline__ void chunk_entries(const CorrSrc& s, const RiceChunk*
   if (*lo > *hi) *lo = *hi;
 }
 
-// A lane's part of chunk [c0, c1): its first and last nonzero (-1 when none)
-// and, through a warp max-scan, the last nonzero before it and the chunk's
-// last nonzero (c0 - 1 when none).
+// Positions within the chunk, through a warp max-scan: the last nonzero before
+// the lane's part and the chunk's last one (-1 when none).
 struct LaneView {
-  int64_t e0;
   uint32_t m;
-  int32_t first, last, prev, chunk_last;
+  int prev, chunk_last;
 };
 
-__device__ __forceinline__ LaneView lane_view(const WarpChunk& V, int64_t c0, int lane) {
+__device__ __forceinline__ LaneView lane_view(uint32_t m, int lane) {
   LaneView v;
-  v.e0 = c0 + 32 * (int64_t)lane;
-  v.m = V.mask[lane];
-  v.first = v.m ? (int32_t)(v.e0 + __ffs(v.m) - 1) : -1;
-  v.last = v.m ? (int32_t)(v.e0 + 31 - __clz(v.m)) : -1;
-  int32_t incl = v.last >= 0 ? v.last : (int32_t)(c0 - 1);
+  v.m = m;
+  int incl = m ? 32 * lane + 31 - __clz(m) : -1;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl = t > incl ? t : incl;
   }
-  const int32_t ex = __shfl_up_sync(0xffffffffu, incl, 1);
-  v.prev = lane == 0 ? (int32_t)(c0 - 1) : ex;
+  const int ex = __shfl_up_sync(0xffffffffu, incl, 1);
+  v.prev = lane == 0 ? -1 : ex;
   v.chunk_last = __shfl_sync(0xffffffffu, incl, 31);
   return v;
 }
 
-// f(run, e, z) for the lane's nonzeros in element order, run = the zeros
+// f(run, i) for the lane's nonzeros i in element order, run = the zeros
 // before each (from the previous nonzero, or the lane view's prev).
 template <class F>
-__device__ __forceinline__ void lane_codes(const WarpChunk& V, const LaneView& v, int lane, F f) {
-  int64_t prev = v.prev;
+__device__ __forceinline__ void lane_codes(const LaneView& v, int lane, F f) {
+  int prev = v.prev - 32 * lane;
   for (uint32_t mm = v.m; mm; mm &= mm - 1) {
     const int i = __ffs(mm) - 1;
-    const int64_t e = v.e0 + i;
-    f((uint64_t)(e - prev - 1), e, V.z[33 * lane + i]);
-    prev = e;
+    f((uint32_t)(i - prev - 1), i);
+    prev = i;
   }
 }
 
 // Code bits of a lane's part with parameters (kr, wv): its nonzeros' codes
-// and, in the last lane, the chunk's closing code.
-__device__ __forceinline__ uint32_t lane_bits(const WarpChunk& V, const LaneView& v, int64_t c1, int lane, int kr,
-                                              int wv) {
-  uint32_t bits = 0;
-  lane_codes(V, v, lane, [&](uint64_t run, int64_t, uint32_t) {
-    bits += ((uint32_t)run >> kr) + 1u + (uint32_t)kr + (uint32_t)wv;
-  });
-  if (lane == 31) bits += ((uint32_t)(c1 - 1 - v.chunk_last) >> kr) + 1u + (uint32_t)kr;
+// and, in the last lane, the closing code of a chunk of len elements.
+__device__ __forceinline__ uint32_t lane_bits(const LaneView& v, int len, int lane, int kr, int wv) {
+  const uint32_t nz = (uint32_t)__popc(v.m);
+  uint32_t bits = nz * (uint32_t)(1 + kr + wv);
+  if (kr == 0) {
+    if (v.m) bits += (uint32_t)(32 * lane + 31 - __clz(v.m) - v.prev) - nz;     // the zeros up to the last nonzero
+  } else {
+    lane_codes(v, lane, [&](uint32_t run, int) { bits += run >> kr; });
+  }
+  if (lane == 31) bits += ((uint32_t)(len - 1 - v.chunk_last) >> kr) + 1u + (uint32_t)kr;
   return bits;
 }
 
@@ -255,20 +263,19 @@ __device__ __forceinline__ uint32_t warp_excl_sum(uint32_t x, int lane, uint32_t
   return incl - x;
 }
 
-// Writer of one chunk's bits from bit `pos` on: whole words inside the chunk
-// are stored, the first and the last (which the neighbouring chunks may
-// share) are OR-ed into words zeroed beforehand.
+// Writer of a lane's bits from bit `pos` on: whole words inside its part are
+// stored, the first and the last (which the neighbours may share) are OR-ed
+// into words zeroed beforehand.
 // Words at or past `limit` are not written (the sizes disagreed: `over` is set).
 struct BitEmit {
   uint32_t* w;
-  uint64_t word, limit;
+  uint32_t word, limit;
   uint64_t acc;
   int fill;
   bool first, over;
-  __device__ BitEmit(uint32_t* words, uint64_t pos, uint64_t nwords)
+  __device__ BitEmit(uint32_t* words, uint32_t pos, uint32_t nwords)
       : w(words), word(pos >> 5), limit(nwords), acc(0), fill((int)(pos & 31)), first(true), over(false) {}
   __device__ __forceinline__ void put(uint32_t v, int width) {   // v < 2^width, width <= 32
-    if (width == 0) return;
     acc |= (uint64_t)v << fill;
     fill += width;
     if (fill >= 32) {
@@ -281,14 +288,19 @@ struct BitEmit {
       fill -= 32;
     }
   }
-  __device__ void ones(uint64_t u) {
+  // the Rice code of `run`, then v in wv bits: one put where they fit a word
+  __device__ __forceinline__ void code(uint32_t run, int kr, uint32_t v, int wv) {
+    uint32_t u = run >> kr;
+    const uint32_t low = run & ((1u << kr) - 1u);
+    const int rest = 1 + kr + wv;
+    if ((int)u + rest < 32) {
+      put(((1u << u) - 1u) | ((low | (v << kr)) << (u + 1)), (int)u + rest);
+      return;
+    }
     for (; u >= 32; u -= 32) put(0xFFFFFFFFu, 32);
-    if (u) put((1u << u) - 1u, (int)u);
-  }
-  __device__ void code(uint64_t run, int kr) {
-    ones(run >> kr);
-    put(0u, 1);
-    put((uint32_t)(run & ((1ull << kr) - 1ull)), kr);
+    put((1u << u) - 1u, (int)u);
+    put(low << 1, 1 + kr);
+    put(v, wv);
   }
   __device__ void finish() {
     if (fill > 0 && acc != 0) {
@@ -297,6 +309,9 @@ struct BitEmit {
     }
   }
 };
+
+// Four bits into the low bits of four bytes.
+__device__ __forceinline__ uint32_t spread4(uint32_t x) { return (x * 0x00204081u) & 0x01010101u; }
 
 __device__ __forceinline__ const uint8_t* src_record(const Plan& P, const uint8_t* s0, int64_t bi, int64_t* bytes) {
   const uint64_t* offs = reinterpret_cast<const uint64_t*>(s0 + P.offsets_pos);
@@ -329,14 +344,7 @@ __global__ void __launch_bounds__(kRiceThreads) k_rice_plan(Plan P, const uint8_
   if (tid == 0) vor_sh = 0u;
   __syncthreads();
   const int64_t N = g.N, nch = cdiv(N, kRiceChunk);
-  uint32_t c[kRunBits];
-#pragma unroll
-  for (int i = 0; i < kRunBits; ++i) c[i] = 0u;
-  uint32_t nz = 0u, vor = 0u;
-  auto count = [&](uint32_t run) {
-#pragma unroll
-    for (int i = 0; i < kRunBits; ++i) c[i] += (run >> i) & 1u;
-  };
+  uint32_t vor = 0u;
   WarpChunk& V = views[warp];
   RiceChunk* rc = chunks + bi * rice_chunks_per_block(P);
   if (!src.dense) {
@@ -350,30 +358,39 @@ __global__ void __launch_bounds__(kRiceThreads) k_rice_plan(Plan P, const uint8_
     const int64_t c0 = ch * kRiceChunk, c1 = (c0 + kRiceChunk) < N ? c0 + kRiceChunk : N;
     int64_t lo, hi;
     chunk_entries(src, rc, ch, nch, &lo, &hi);
-    load_chunk(src, c0, c1, lo, hi, lane, V);
-    const LaneView v = lane_view(V, c0, lane);
+    const LaneView v = lane_view(load_chunk<false>(src, c0, c1, lo, hi, lane, V, vor), lane);
+    // runs with bit i set: four byte counters to a word (at most 33 runs a
+    // lane), then 16 bits in the warp's sums (at most 1025).  (4096 records,
+    // 1 GiB: the kernel 302 us with a counter a bit and the values through
+    // shared memory, 200 so; issue binds it.)
+    uint32_t b[3] = {0u, 0u, 0u};
+    auto count = [&](uint32_t run) {
+      b[0] += spread4(run & 15u);
+      if (run >= 16u) {
+        b[1] += spread4((run >> 4) & 15u);
+        b[2] += spread4(run >> 8);
+      }
+    };
+    lane_codes(v, lane, [&](uint32_t run, int) { count(run); });
+    if (lane == 31) count((uint32_t)((int)(c1 - c0) - 1 - v.chunk_last));
+    uint32_t hw[6] = {0u, 0u, 0u, 0u, 0u, 0u};       // c[0] | c[1] << 16, ...
+    const bool wide = __any_sync(0xffffffffu, (b[1] | b[2]) != 0u);
 #pragma unroll
-    for (int i = 0; i < kRunBits; ++i) c[i] = 0u;
-    nz = 0u;
-    lane_codes(V, v, lane, [&](uint64_t run, int64_t, uint32_t z) {
-      count((uint32_t)run);
-      ++nz;
-      vor |= z - 1u;
-    });
-    if (lane == 31) count((uint32_t)(c1 - 1 - v.chunk_last));
-    // the chunk's counts (runs <= 1025, so 16 bits each)
-    RiceChunk rec_c;
-#pragma unroll
-    for (int i = 0; i <= kRunBits; ++i) {
-      const uint32_t x = __reduce_add_sync(0xffffffffu, i < kRunBits ? c[i] : nz);
-      if (i < kRunBits) rec_c.c[i] = (uint16_t)x;
-      else rec_c.nnz = (uint16_t)x;
-      wsum[i] += x;
+    for (int q = 0; q < 3; ++q) {
+      if (q > 0 && !wide) break;
+      const uint32_t ev = __reduce_add_sync(0xffffffffu, b[q] & 0x00FF00FFu);
+      const uint32_t od = __reduce_add_sync(0xffffffffu, (b[q] >> 8) & 0x00FF00FFu);
+      hw[2 * q] = __byte_perm(ev, od, 0x5410);
+      hw[2 * q + 1] = __byte_perm(ev, od, 0x7632);
     }
+    static_assert(kRunBits == 11, "the twelfth half word is the nonzeros' count");
+    hw[5] = (hw[5] & 0xFFFFu) | (__reduce_add_sync(0xffffffffu, (uint32_t)__popc(v.m)) << 16);
+#pragma unroll
+    for (int i = 0; i <= kRunBits; ++i) wsum[i] += (hw[i >> 1] >> (16 * (i & 1))) & 0xFFFFu;
     if (lane == 0) {
 #pragma unroll
-      for (int i = 0; i < kRunBits; ++i) rc[ch].c[i] = rec_c.c[i];
-      rc[ch].nnz = rec_c.nnz;
+      for (int i = 0; i < kRunBits; ++i) rc[ch].c[i] = (uint16_t)(hw[i >> 1] >> (16 * (i & 1)));
+      rc[ch].nnz = (uint16_t)(hw[5] >> 16);
     }
     __syncwarp();
   }
@@ -442,15 +459,24 @@ __global__ void __launch_bounds__(kRiceThreads) k_rice_write(Plan P, const uint8
   const int64_t N = g.N, nch = cdiv(N, kRiceChunk);
   const int kr = ri.kr, wv = ri.wv;
   const RecLayout nl = rice_layout(src.lay, N, ri.words, src.nesc, es);
-  for (int64_t i = tid; i < nl.size / 16; i += kRiceThreads) reinterpret_cast<uint4*>(dst)[i] = make_uint4(0, 0, 0, 0);
-  __syncthreads();
   // the prefix up to the corrections (8-byte multiple), then the escapes
-  for (int64_t i = tid; i < nl.off_c / 8; i += kRiceThreads)
-    reinterpret_cast<uint2*>(dst)[i] = reinterpret_cast<const uint2*>(rec)[i];
+  const int64_t pre = nl.off_c / 16;
+#pragma unroll 4
+  for (int64_t i = tid; i < pre; i += kRiceThreads)
+    reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(rec)[i];
+  if (tid == 0 && 16 * pre < nl.off_c)
+    *reinterpret_cast<uint2*>(dst + 16 * pre) = *reinterpret_cast<const uint2*>(rec + 16 * pre);
   for (int64_t i = tid; i < src.nesc; i += kRiceThreads)
     reinterpret_cast<uint32_t*>(dst + nl.off_ei)[i] = reinterpret_cast<const uint32_t*>(rec + src.lay.off_ei)[i];
   for (int64_t i = tid; i < src.nesc * es / 4; i += kRiceThreads)
     reinterpret_cast<uint32_t*>(dst + nl.off_ev)[i] = reinterpret_cast<const uint32_t*>(rec + src.lay.off_ev)[i];
+  // the padding after each section
+  if (tid < 3) {
+    const int64_t from = tid == 0 ? nl.off_c + nl.corr_words * 4 : tid == 1 ? nl.off_ei + 4 * (int64_t)src.nesc
+                                                                          : nl.off_ev + (int64_t)src.nesc * es;
+    const int64_t to = tid == 0 ? nl.off_ei : tid == 1 ? nl.off_ev : nl.size;
+    for (int64_t b = from; b < to; b += 4) *reinterpret_cast<uint32_t*>(dst + b) = 0u;
+  }
   uint32_t* cw = reinterpret_cast<uint32_t*>(dst + nl.off_c);
   uint32_t* tab = cw + 2;
   uint32_t* words = cw + 2 + nch;
@@ -472,7 +498,14 @@ __global__ void __launch_bounds__(kRiceThreads) k_rice_write(Plan P, const uint8
     const int x = i < nch ? (int)tab[i] : 0;
     int tot;
     const int ex = block_excl_scan(x, sh_warp, &tot);
-    if (i < nch) tab[i] = carry + (uint32_t)ex;
+    if (i < nch) {
+      // the words that a chunk shares with its neighbours: the chunks' first
+      // and last ones, OR-ed together below
+      const uint32_t at = carry + (uint32_t)ex, end = at + (uint32_t)x;
+      tab[i] = at;
+      if ((at >> 5) < ri.words) words[at >> 5] = 0u;
+      if (end > at && ((end - 1) >> 5) < ri.words) words[(end - 1) >> 5] = 0u;
+    }
     carry += (uint32_t)tot;
   }
   if (tid == 0) {
@@ -482,23 +515,51 @@ __global__ void __launch_bounds__(kRiceThreads) k_rice_write(Plan P, const uint8
     cw[1] = (uint32_t)kr | ((uint32_t)wv << 8);
   }
   __syncthreads();
-  // the codes: each lane from its own first bit
+  // The codes, each lane from its own first bit: into the warp's buffer and
+  // from there in whole words, or (values past a byte) straight to their place.  (4096 records of 64 x 4096 points, 1 GiB: the kernel took
+  // 568 us when it zeroed the record first and every lane OR-ed its ends into
+  // global memory a code's part at a time, 381 so.)
   for (int64_t ch = warp; ch < nch; ch += kRiceThreads / 32) {
-    const int64_t c0 = ch * kRiceChunk, c1 = (c0 + kRiceChunk) < N ? c0 + kRiceChunk : N;
+    const int64_t c0 = ch * kRiceChunk;
+    const int len = (int)((c0 + kRiceChunk) < N ? kRiceChunk : N - c0);
     int64_t lo, hi;
     chunk_entries(src, rc, ch, nch, &lo, &hi);
-    load_chunk(src, c0, c1, lo, hi, lane, V);
-    const LaneView v = lane_view(V, c0, lane);
+    uint32_t unused = 0;
+    const LaneView v = lane_view(load_chunk<true>(src, c0, c0 + len, lo, hi, lane, V, unused), lane);
     uint32_t tot;
-    const uint32_t off = warp_excl_sum(lane_bits(V, v, c1, lane, kr, wv), lane, &tot);
-    BitEmit em(words, (uint64_t)tab[ch] + off, ri.words);
-    lane_codes(V, v, lane, [&](uint64_t run, int64_t, uint32_t z) {
-      em.code(run, kr);
-      em.put(z - 1u, wv);
-    });
-    if (lane == 31) em.code((uint64_t)(c1 - 1 - v.chunk_last), kr);
-    em.finish();
-    if (em.over) atomicOr(&st_w->corrupt, 1u);
+    const uint32_t off = warp_excl_sum(lane_bits(v, len, lane, kr, wv), lane, &tot);
+    const uint32_t at = tab[ch], w0 = at >> 5, nw = ((at & 31u) + tot + 31u) >> 5;
+    auto emit = [&](BitEmit& em, auto value) {
+      lane_codes(v, lane, [&](uint32_t run, int i) { em.code(run, kr, value(i) - 1u, wv); });
+      if (lane == 31) em.code((uint32_t)(len - 1 - v.chunk_last), kr, 0u, 0);
+      em.finish();
+      return em.over;
+    };
+    bool over = false;
+    if (src.wk <= 8) {
+      // (at most 8 bits a value, 11 a run's remainder and 1024 in the unary
+      // parts: the buffer holds them)
+      uint32_t* sw = V.stage();
+      const uint8_t* zb = V.bytes() + 36 * lane;
+      const uint32_t cap = nw < (uint32_t)kStageWords ? nw : (uint32_t)kStageWords;
+      for (uint32_t k = lane; k < cap; k += 32) sw[k] = 0u;
+      __syncwarp();
+      BitEmit em(sw, (at & 31u) + off, cap);
+      over = emit(em, [&](int i) { return (uint32_t)zb[i]; });
+      __syncwarp();
+      for (uint32_t k = lane; k < cap; k += 32) {
+        if (w0 + k >= ri.words) over = true;
+        else if (k == 0 || k == nw - 1) atomicOr(&words[w0 + k], sw[k]);
+        else words[w0 + k] = sw[k];
+      }
+    } else {
+      for (uint32_t k = lane + 1; k + 1 < nw; k += 32)
+        if (w0 + k < ri.words) words[w0 + k] = 0u;
+      __syncwarp();
+      BitEmit em(words, at + off, ri.words);
+      over = emit(em, [&](int i) { return V.z[33 * lane + i]; });
+    }
+    if (over) atomicOr(&st_w->corrupt, 1u);
     __syncwarp();
   }
 }
