@@ -46,7 +46,8 @@ enum { DLS_F32 = 0, DLS_F64 = 1 };
  * no pointwise correction in that mode. */
 enum { DLS_EB_ABS = 0, DLS_EB_REL_RANGE = 1, DLS_EB_NRMSE = 2 };
 /* Arithmetic of the Gram and projection products.
- *   FP64:   double precision everywhere (the plain form).
+ *   FP64:   every stored value by its double-precision definition (the plain
+ *           form; where FP32 provably settles a decision, it is taken there).
  *   FP32:   FP32 products on the CUDA cores with FP32 accumulation; FP32
  *           Jacobi eigensolve, its eigenvectors orthonormalised in FP64 (to
  *           below the rounding of the stored modes); every stored decision
@@ -206,12 +207,11 @@ int dls_plan_info(const dls_plan* plan, int32_t* variant, float* tune_ms);
 /* The plan's occupancy form per shape class -- 1: the kernels built for fewer
  * CTAs per SM with more registers per thread (2 per SM for the staged kernels,
  * 1 for the space-side kernel), 2: built for more (4, 2) -- and the device time
- * that chose it.  Classes: [0] "whole", the blocks of the full block
- * shape that the encode kernel finishes at the predicted rank (Sec. 2.5 rank
- * step); [1] "rest", what the searching kernels take: edge blocks of smaller
- * shapes (Sec. 2.7.1 partition remainders), predictions the exact test
- * rejects, blocks whose Gram side is space, or every block when the plan
- * searches.  forms: 2 entries (form 1 or 2 of each class); class_ms: 4
+ * that chose it.  Classes: [0] "whole", the blocks that the encode kernel
+ * finishes at the predicted rank (Sec. 2.5 rank step), of the full block shape
+ * and of the edges' smaller ones (Sec. 2.7.1 partition remainders); [1] "rest",
+ * what the searching kernels take: predictions the exact test rejects, blocks
+ * whose Gram side is space, or every block when the plan searches.  forms: 2 entries (form 1 or 2 of each class); class_ms: 4
  * entries, class_ms[2 c + f - 1] = ms of class c's kernels in form f during
  * tuning (0 if the choices came from the cache).  The forms run the same code,
  * so the stream does not depend on them.  Either pointer may be null. */

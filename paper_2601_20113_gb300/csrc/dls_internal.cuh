@@ -311,10 +311,9 @@ int launch_mixed_compress(const Plan& p, const void* d_in, const MixedWork& w, i
                           int spatial_only, cudaStream_t s);
 // Occupancy forms of the per-block kernels, one per shape class of a
 // compression's blocks (1: the form built for 2 CTAs per SM, with more
-// registers per thread; 2: the form built for 4).  `whole`: the blocks of the
-// full block shape that k_enc encodes at the predicted rank.  `rest`: what
-// k_tile and k_mixed take -- edge blocks of smaller shapes, predictions k_enc
-// rejects, blocks whose Gram side is space, every block in the search mode;
+// registers per thread; 2: the form built for 4).  `whole`: the blocks, of any
+// shape, that k_enc encodes at the predicted rank.  `rest`: what k_tile and
+// k_mixed take -- predictions k_enc rejects, blocks whose Gram side is space, every block in the search mode;
 // 0 there means the 2-CTA form behind k_enc (a short list) and the 4-CTA form
 // when k_tile takes every block.  Both forms run the same code, so the choice
 // changes the time and never a byte of the stream.

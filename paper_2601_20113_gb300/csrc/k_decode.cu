@@ -5,8 +5,10 @@
 // acc = fma(chat[l][k], Vst[j][k], acc) in the field dtype, with
 // chat = dtype(q) * dtype(delta).  Then xtilde = fma(dtype(k), dtype(2eb), acc)
 // where the correction k is nonzero, and escaped points take their raw value.
-// One CTA per block; every structural field of a record is validated against
-// the geometry before use.
+// Every structural field of a record is validated against the geometry before
+// use.  k_decode_f32 takes the time-side blocks of float32 fields (persistent
+// CTAs, the next record copied while one is decoded), k_decode the others, a
+// CTA a block.
 #include "dls_internal.cuh"
 
 namespace dls {

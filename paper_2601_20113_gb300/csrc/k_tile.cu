@@ -2676,10 +2676,9 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
 
 // ---------------------------------------------------------------- k_tile
 // Every block k_enc does not finish, with the block state (basis, eigenvalues,
-// statistics) k_gram and k_eig left: the Rayleigh-Ritz pass where the FP32
-// Gram cannot resolve the modes near the budget, the rank test of a
-// prediction and the bisection of Algorithm 1 when it fails (or always, with
-// the search rank mode), and records that cannot be deferred.  With
+// statistics) k_gram and k_eig left: the bisection of Algorithm 1 where the
+// rank test of a prediction failed (or always, with the search rank mode), and
+// the blocks k_enc could not settle.  With
 // a.from_list the blocks come from k_enc's list, else from the launch range.
 // The arguments stay in parameter space (the passes take their address).
 template <int MINB>
