@@ -734,8 +734,8 @@ int64_t or_block_compress(const or_params* p, const void* field, int64_t b, cons
     uint8_t* tmp = (uint8_t*)malloc((size_t)(rawsz + 4096 + 64 * (int64_t)n * n));
     sz = or_pack_record(r, g.side, n, L, g.M, p->dtype, Vr, qr, kk, esc, A, tmp,
                         rawsz + 4096 + 64 * (int64_t)n * n, p->corr_codec);
-    if (sz >= rawsz) {
-      raw = 1;
+    if (sz >= rawsz || sz == OR_ERR_CAPACITY) {
+      raw = 1;                     /* (a record past tmp is past a raw one too) */
     } else if (sz > rec_cap) {
       sz = OR_ERR_CAPACITY;
     } else {
