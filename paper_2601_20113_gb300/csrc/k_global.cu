@@ -119,18 +119,24 @@ GbLayout gb_layout(const GbPlan& g) {
 }
 
 // ---------------------------------------------------------------- step 1: the basis
-// Row s of Q: the patch of the first snapshot at origins[s] (x fastest).
+// Row s of Q: the patch of the first snapshot at origins[s] (x fastest).  What
+// the call refuses (an origin outside the snapshot, a non-finite value) leaves
+// zeros, so that the Gram and the eigensolve run on finite values: the status
+// is read after the last kernel.
 __global__ void k_gb_sample(GbPlan g, const float* __restrict__ in, const int64_t* __restrict__ origins, double* Q,
                             GbStatus* st) {
   const int64_t s = blockIdx.x;
   const int64_t x0 = origins[3 * s], y0 = origins[3 * s + 1], z0 = origins[3 * s + 2];
   if (x0 < 0 || y0 < 0 || z0 < 0 || x0 + g.px > g.dims[0] || y0 + g.py > g.dims[1] || z0 + g.pz > g.dims[2]) {
     if (threadIdx.x == 0) atomicOr(&st->bad_origin, 1u);
+    for (int i = threadIdx.x; i < g.M; i += blockDim.x) Q[s * g.M + i] = 0.0;
     return;
   }
   for (int i = threadIdx.x; i < g.M; i += blockDim.x) {
     const int ix = i % g.px, iy = (i / g.px) % g.py, iz = i / (g.px * g.py);
-    Q[s * g.M + i] = (double)in[((z0 + iz) * g.dims[1] + (y0 + iy)) * g.dims[0] + (x0 + ix)];
+    const float v = in[((z0 + iz) * g.dims[1] + (y0 + iy)) * g.dims[0] + (x0 + ix)];
+    if (not_finite(v)) atomicOr(&st->nonfinite, 1u);
+    Q[s * g.M + i] = not_finite(v) ? 0.0 : (double)v;
   }
 }
 
@@ -349,9 +355,19 @@ __global__ void __cluster_dims__(kJacCtas, 1, 1) __launch_bounds__(kJacThreads, 
   __threadfence();
   cl.sync();
   if (rank != 0) return;
+  // places by a total order (the keys', zeros of either sign alike), so that
+  // every place is taken whatever the eigenvalues are
+  auto key_of = [&](int k) {
+    const double x = S.lam[k];
+    return dkey((__double_as_longlong(x) << 1) ? x : 0.0);
+  };
   for (int k = tid; k < M; k += kJacThreads) {
+    const unsigned long long key = key_of(k);
     int at = 0;
-    for (int j = 0; j < M; ++j) at += (S.lam[j] > S.lam[k] || (S.lam[j] == S.lam[k] && j < k)) ? 1 : 0;
+    for (int j = 0; j < M; ++j) {
+      const unsigned long long other = key_of(j);
+      at += (other > key || (other == key && j < k)) ? 1 : 0;
+    }
     S.order[at] = k;
   }
   __syncthreads();
