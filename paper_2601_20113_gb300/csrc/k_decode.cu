@@ -748,6 +748,9 @@ __global__ void __launch_bounds__(kDecThreads, 3) k_decode_f32(Plan P, const uin
     } else {
       decode_block_f32(P, comp, comp_bytes, out, st, bi, reinterpret_cast<uint32_t*>(dsm), kRecCapAll / 4);
     }
+    // the next record's copy writes, through the async proxy, what this block
+    // left by ordinary stores (the plane, a record staged by decode_block)
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (tid == 0) fetch();
     __syncthreads();
