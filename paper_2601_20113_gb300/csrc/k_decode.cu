@@ -19,6 +19,12 @@ constexpr int kDecThreads = 256;
 // (72 KB: three CTAs per SM, as the launch bounds ask of the registers).
 constexpr int kDecStageWords = 18432;
 
+// Whether a record's table entries lie in order inside the payload (`room` bytes
+// after payload_pos), the first a multiple of 16: entries near 2^64 must not wrap.
+__device__ __forceinline__ bool record_in(uint64_t o0, uint64_t o1, uint64_t room) {
+  return o1 <= room && o0 <= o1 && o1 - o0 >= 16 && (o0 & 15) == 0;
+}
+
 template <typename T> __device__ __forceinline__ T dq(int32_t q, T d);
 template <> __device__ __forceinline__ float dq<float>(int32_t q, float d) { return __fmul_rn(__int2float_rn(q), d); }
 template <> __device__ __forceinline__ double dq<double>(int32_t q, double d) { return __dmul_rn((double)q, d); }
@@ -82,7 +88,7 @@ __device__ __forceinline__ void decode_block(const Plan& P, const uint8_t* __res
   const int es = (int)sizeof(T);
   const uint64_t* offs = reinterpret_cast<const uint64_t*>(comp + P.offsets_pos);
   const uint64_t o0 = offs[bi], o1 = offs[bi + 1];
-  if (o1 < o0 + 16 || (uint64_t)P.payload_pos + o1 > comp_bytes || (o0 & 15) != 0) {
+  if (!record_in(o0, o1, comp_bytes - (uint64_t)P.payload_pos)) {
     if (tid == 0) atomicOr(&st->corrupt, 1u);
     return;
   }
@@ -644,8 +650,7 @@ __global__ void __launch_bounds__(kDecThreads, 3) k_decode_f32(Plan P, const uin
     bytes = 0;
     if (b >= P.nb) return;
     const uint64_t o0 = offs[b], o1 = offs[b + 1];
-    if (o1 < o0 + 16 || (uint64_t)P.payload_pos + o1 > comp_bytes || ((o0 | o1) & 15) != 0 || o1 - o0 > (uint64_t)kRecCapAll)
-      return;
+    if (!record_in(o0, o1, comp_bytes - (uint64_t)P.payload_pos) || (o1 & 15) != 0 || o1 - o0 > (uint64_t)kRecCapAll) return;
     const uint32_t nb = (uint32_t)(o1 - o0);
     bytes = (int)nb;
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&full)), "r"(nb) : "memory");
@@ -783,7 +788,7 @@ __device__ void verify_stream(const Plan& P, const uint8_t* __restrict__ comp, u
     unsigned long long n[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (bi < P.nb) {
       const uint64_t o0 = offs[bi], o1 = offs[bi + 1];
-      if (!(o1 < o0 + 16 || (uint64_t)P.payload_pos + o1 > comp_bytes || (o0 & 15) != 0)) {
+      if (record_in(o0, o1, comp_bytes - (uint64_t)P.payload_pos)) {
         const uint8_t* rec = comp + P.payload_pos + o0;
         const uint32_t* rec32 = reinterpret_cast<const uint32_t*>(rec);
         const int r = rec[0], flags = rec[1];

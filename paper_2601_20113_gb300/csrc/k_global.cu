@@ -949,7 +949,8 @@ __global__ void __launch_bounds__(256) k_gb_decode(GbPlan g, const uint8_t* __re
   const uint64_t* ot = reinterpret_cast<const uint64_t*>(comp + g.offsets_pos);
   const double* basis = reinterpret_cast<const double*>(comp + kGbHdr);   // [mode][component]
   const uint64_t o0 = ot[p], o1 = ot[p + 1];
-  if (o1 < o0 + 8 || (uint64_t)g.payload_pos + o1 > comp_bytes || (o0 & 7) != 0) {
+  // (entries near 2^64 must not wrap)
+  if (o1 > comp_bytes - (uint64_t)g.payload_pos || o0 > o1 || o1 - o0 < 8 || (o0 & 7) != 0) {
     if (lane == 0) atomicOr(&st->corrupt, 1u);
     return;
   }
