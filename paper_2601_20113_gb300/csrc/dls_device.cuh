@@ -15,12 +15,21 @@ __device__ __forceinline__ double widen(float x) {
   if ((u & 0x7F800000u) == 0u) return (double)x;       // zeros and subnormals
   return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
 }
-// The same for passes that stream their input: a subnormal is scaled by 2^32
+// (double)x exactly whatever x is, for values that nothing has screened (a
+// decoded value may have overflowed): widen with the exponent of infinities and
+// NaNs kept at its largest.
+__device__ __forceinline__ double widen_any(float x) {
+  const uint32_t u = __float_as_uint(x);
+  if ((u & 0x7F800000u) != 0x7F800000u) return widen(x);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x70000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen_any(double x) { return x; }
+// widen for passes that stream their input: a subnormal is scaled by 2^32
 // first (exactly) instead of converted, since the compiler runs the conversion
 // for every value and selects (the statistics pass on 43 M floats: 196 us with
 // it, 96 without; the norm pass on 34 M: 152 and 73).  In chains of dependent FMAs
-// the extra integer work costs more (the patch kernel: 1576 us with the form
-// above, 1757 with this one).
+// the extra integer work costs more (the patch kernel: 1576 us with widen,
+// 1757 with this one).
 __device__ __forceinline__ double widen_stream(float x) {
   const bool small = (__float_as_uint(x) & 0x7F800000u) == 0u;
   const uint32_t u = __float_as_uint(small ? __fmul_rn(x, 4294967296.0f) : x), m = u & 0x7FFFFFFFu;

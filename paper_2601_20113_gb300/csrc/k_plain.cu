@@ -330,7 +330,7 @@ __device__ __noinline__ double block_err(Smem<T, NM>& S, const Plan& P, const Ge
 #pragma unroll
         for (int k = 0; k < NM; ++k)
           if (k < r) acc = tfma<T>(ch[k], S.Vt[k * NM + j], acc);
-        S.buf[lr * LD + j] = dsub(widen(row[S.coff[j]]), widen(acc));
+        S.buf[lr * LD + j] = dsub(widen(row[S.coff[j]]), widen_any(acc));   // (an infinite acc makes E infinite)
       }
     }
     __syncthreads();
