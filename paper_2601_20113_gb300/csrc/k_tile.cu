@@ -943,7 +943,8 @@ constexpr int kFastK = 59;
 // max(m, |a|, |b|), a NaN if one is (so that no comparison settles a row with one)
 __device__ __forceinline__ float max_abs_nan(float m, float a, float b) {
   float r;
-  asm("{\n.reg .f32 x, y;\nabs.f32 x, %2;\nabs.f32 y, %3;\nmax.NaN.f32 %0, x, y;\nmax.NaN.f32 %0, %0, %1;\n}" : "=f"(r) : "f"(m), "f"(a), "f"(b));
+  // (into a scratch register: %0 may share %1's until %1 has been read)
+  asm("{\n.reg .f32 x, y;\nabs.f32 x, %2;\nabs.f32 y, %3;\nmax.NaN.f32 x, x, y;\nmax.NaN.f32 %0, x, %1;\n}" : "=f"(r) : "f"(m), "f"(a), "f"(b));
   return r;
 }
 template <int NP, bool POINT, int MC>
