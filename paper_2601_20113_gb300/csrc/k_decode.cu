@@ -875,8 +875,8 @@ __global__ void __launch_bounds__(256) k_verify_points(Plan P, const T* __restri
 // unevaluated float pairs (x^2 = p + fma(x, x, -p) exactly, d^2 = s^2 + 2 s e
 // to within e^2 <= 2^-48 s^2), two points an instruction (packed FP32), per
 // batch of 1024 points of a thread; each batch is added in FP64, and one whose
-// pairs overflowed is summed again in FP64.  Loads are float4 when the field
-// allows (4 | K, 16-byte pointers).  Bound by the issue slots (about 20
+// squares reach 2^117 (or with a NaN or an infinity) is summed again in FP64.
+// Loads are float4 when the field allows (4 | K, 16-byte pointers).  Bound by the issue slots (about 20
 // instructions a point; scalar FP32 with a branch a point took twice that):
 // two fields of 1 GiB 0.74 -> 0.49 ms, the records' pass included.
 struct FF2 {
@@ -967,7 +967,7 @@ __global__ void __launch_bounds__(256) k_verify_points_f32(Plan P, const float* 
   };
   auto flush = [&](const float* a0, const float* b0, int64_t i, int64_t n, int64_t stride, int width) {
     const float h = (fe.hi.x + fe.hi.y) + (fx.hi.x + fx.hi.y) + (fe.lo.x + fe.lo.y) + (fx.lo.x + fx.lo.y);
-    if (fabsf(h) < 3.0e38f) {
+    if (fabsf(h) < 0x1p117f) {             // every |x| and |s| below 2^59, every |y| below 2^60
       se += ((double)fe.hi.x + (double)fe.lo.x) + ((double)fe.hi.y + (double)fe.lo.y);
       sx += ((double)fx.hi.x + (double)fx.lo.x) + ((double)fx.hi.y + (double)fx.lo.y);
     } else {
