@@ -872,10 +872,11 @@ __global__ void __launch_bounds__(256) k_verify_points(Plan P, const T* __restri
 // |s| reaches the thread's running maximum (rounding is monotone, so the point
 // of the largest |x - y| is among them) or the bound less a relative 2^-20, or
 // is not finite: one test for four points.  The sums of squares run as
-// unevaluated float pairs (x^2 = p + fma(x, x, -p) exactly, d^2 = s^2 + 2 s e
-// to within e^2 <= 2^-48 s^2), two points an instruction (packed FP32), per
+// unevaluated float pairs (x^2 = p + fma(x, x, -p) exactly where neither is
+// subnormal, d^2 = s^2 + 2 s e to within e^2 <= 2^-48 s^2), two points an instruction (packed FP32), per
 // batch of 1024 points of a thread; each batch is added in FP64, and one whose
-// squares reach 2^117 (or with a NaN or an infinity) is summed again in FP64.
+// squares reach 2^117 (or with a NaN or an infinity), or stay below 2^-92
+// without being zeros, is summed again in FP64.
 // Loads are float4 when the field allows (4 | K, 16-byte pointers).  Bound by the issue slots (about 20
 // instructions a point; scalar FP32 with a branch a point took twice that):
 // two fields of 1 GiB 0.74 -> 0.49 ms, the records' pass included.
@@ -925,6 +926,26 @@ __device__ __noinline__ void verify_point(VerRare& V, float x, float y) {
   if (ad > V.mx32) V.mx32 = ad;
   if (edge && d > V.eb) ++V.over;
 }
+// A batch's pairs are exact to 2^-46 of a sum of at least kPairsLeast (below
+// 2^-126 a square or its residual is off by up to 2^-150, three a point, 1024
+// points) and, below kPairsMost, every |x| and |s| is below 2^59, every |y| below
+// 2^60.  (Maxima kept with the points for these tests took a fifth more time; a
+// batch's sums out of line altogether 2%.)
+constexpr float kPairsLeast = 0x1p-92f, kPairsMost = 0x1p117f;
+// Whether the sums of a batch below kPairsLeast are sums of zeros: `err`,
+// differences have been seen; `val`, the values' squares are as small (they are
+// read again).
+__device__ __noinline__ bool verify_zeros(const float* __restrict__ a, int64_t i, int64_t n, int64_t stride, int width, bool err,
+                                          bool val) {
+  if (err) return false;
+  uint32_t any = 0u;
+  if (val) {
+#pragma unroll 8
+    for (int64_t k = 0; k < n; ++k)
+      for (int c = 0; c < width; ++c) any |= __float_as_uint(a[(i + k * stride) * width + c]) << 1;
+  }
+  return any == 0u;
+}
 __device__ __noinline__ void verify_sums_fp64(const float* __restrict__ a, const float* __restrict__ b, int64_t i, int64_t n,
                                               int64_t stride, int width, double* se, double* sx) {
   for (int64_t k = 0; k < n; ++k, i += stride)
@@ -966,8 +987,10 @@ __global__ void __launch_bounds__(256) k_verify_points_f32(Plan P, const float* 
     return s;
   };
   auto flush = [&](const float* a0, const float* b0, int64_t i, int64_t n, int64_t stride, int width) {
-    const float h = (fe.hi.x + fe.hi.y) + (fx.hi.x + fx.hi.y) + (fe.lo.x + fe.lo.y) + (fx.lo.x + fx.lo.y);
-    if (fabsf(h) < 0x1p117f) {             // every |x| and |s| below 2^59, every |y| below 2^60
+    const float he = fe.hi.x + fe.hi.y, hx = fx.hi.x + fx.hi.y;
+    const float h = he + hx + (fe.lo.x + fe.lo.y) + (fx.lo.x + fx.lo.y);       // a NaN when any of them is
+    if ((fabsf(h) < kPairsMost && fminf(he, hx) >= kPairsLeast) ||
+        (fabsf(h) < kPairsMost && verify_zeros(a0, i, n, stride, width, he < kPairsLeast && V.mx32 > 0.0f, hx < kPairsLeast))) {
       se += ((double)fe.hi.x + (double)fe.lo.x) + ((double)fe.hi.y + (double)fe.lo.y);
       sx += ((double)fx.hi.x + (double)fx.lo.x) + ((double)fx.hi.y + (double)fx.lo.y);
     } else {
