@@ -462,24 +462,25 @@ __device__ __forceinline__ void dec_rows(const Plan& P, const Geom& g, const Dec
 #pragma unroll
           for (int v = 0; v < V; ++v) acc[v] = __fmaf_rn(ch[c][v], b[c], acc[v]);
       }
-      // a correction of zero adds zero
+      // fma(-k, -step, acc): a correction of zero adds a zero of negative sign,
+      // which leaves every acc as it is, zeros of either sign among them
       if (CM == 1) {
-        // (float)k as (2^23 + k + 8) - (2^23 + 8): exact, and off the conversion pipe
+        // (float)-k as (2^23 + 8) - (2^23 + k + 8): exact, and off the conversion pipe
         const int e = j * M + l;
         const uint32_t k4 = V == 4 ? (uint32_t)reinterpret_cast<const uint16_t*>(plane)[e >> 2]
                                    : (uint32_t)plane[e >> 1] >> ((e & 1) * 4);
 #pragma unroll
         for (int v = 0; v < V; ++v)
-          acc[v] = __fmaf_rn(__fsub_rn(__uint_as_float(((k4 >> (4 * v)) & 15u) | 0x4B000000u), 8388616.0f), step, acc[v]);
+          acc[v] = __fmaf_rn(__fsub_rn(8388616.0f, __uint_as_float(((k4 >> (4 * v)) & 15u) | 0x4B000000u)), -step, acc[v]);
       }
       if (CM == 2) {
-        // V wk <= 32 bits from one unaligned word
+        // V wk <= 32 bits from one unaligned word; (float)-k as above, |k| <= 128
         const uint32_t pos = (uint32_t)(j * M + l) * (uint32_t)wk;
         const uint32_t* p = cw + (pos >> 5);
         const uint32_t f = __funnelshift_r(p[0], p[1], pos & 31u);
 #pragma unroll
         for (int v = 0; v < V; ++v)
-          acc[v] = __fmaf_rn((float)unzigzag((f >> (v * wk)) & kmask), step, acc[v]);
+          acc[v] = __fmaf_rn(__fsub_rn(8388864.0f, __int_as_float(0x4B000100 + unzigzag((f >> (v * wk)) & kmask))), -step, acc[v]);
       }
       if (V == 4) *reinterpret_cast<float4*>(o) = make_float4(acc[0], acc[V > 1 ? 1 : 0], acc[V > 2 ? 2 : 0], acc[V > 3 ? 3 : 0]);
       else *o = acc[0];
