@@ -1931,8 +1931,11 @@ struct FastBlock {
 };
 // kFbRankFail: k_enc ran the exact test at the predicted rank and it failed
 // (or a coefficient overflowed), so k_tile goes straight to the search;
-// kFbRankLow: because the rank is above the prediction.
-enum : int32_t { kFbNonfinite = 1, kFbRR = 2, kFbOverflow = 4, kFbRankFail = 8, kFbRankLow = 16 };
+// kFbRankLow: because the rank is above the prediction.  kFbNoDefer: the rank
+// passed but the record cannot be deferred, so k_tile encodes into its scratch
+// at once (256 blocks of a ragged 62 x 61 x 63 x 61 field, a few corrections past
+// a byte in each: k_tile 198 -> 122 us).
+enum : int32_t { kFbNonfinite = 1, kFbRR = 2, kFbOverflow = 4, kFbRankFail = 8, kFbRankLow = 16, kFbNoDefer = 32 };
 
 // Block counters of the phase kernels and the list of blocks k_enc leaves.
 struct FastCtl {
@@ -2656,7 +2659,7 @@ __global__ void __launch_bounds__(kTT, MINB) k_enc(const __grid_constant__ CUten
     }
     pc.mark(S, kPhDecide);
     if (!accepted) {
-      if (rank_fail && threadIdx.x == 0) a.fb[bi].flags |= kFbRankFail | (low ? kFbRankLow : 0);
+      if (threadIdx.x == 0) a.fb[bi].flags |= rank_fail ? kFbRankFail | (low ? kFbRankLow : 0) : kFbNoDefer;
       to_list(bi);
       __syncthreads();
       continue;
@@ -2754,7 +2757,7 @@ __global__ void __launch_bounds__(kTT, MINB) k_tile(const __grid_constant__ CUte
     int r = 0;
     if (a.learned != kRankSearch && !may_overflow && !(a.fb[bi].flags & kFbRankFail)) {
       const int rp = S.r_pred;
-      if (!encode(rp, false)) break;
+      if (!encode(rp, (a.fb[bi].flags & kFbNoDefer) != 0)) break;
       pc.mark(S, kPhEncode);
       const double E_rm1 = S.Ered[0], E_r = S.Ered[1];
       if (!S.ovf) {
