@@ -930,8 +930,11 @@ __device__ __forceinline__ ChunkRows chunk_rows(const TileArgs& a, const Geom& g
 // through corr_decide.  A ballot a column is one word of the bitmap, and each
 // warp writes whole 32-byte sectors of k8.
 // MC = 4096: the 16 x 16 x 16 x 16 block (chunks of 256 rows, every row and
-// offset known); 0: any shape, by row arithmetic and, where a column's rows do
-// not start on a word of the bitmap, by OR-ing shifted words.
+// offset known); 1: NP time steps and chunks of whole lines (bitmap_rows), every
+// row a block row in turn, its count known at run time; 0: any shape, by row
+// arithmetic and, where a column's rows do not start on a word of the bitmap, by
+// OR-ing shifted words.  (64 blocks of 32 x 32 x 16 x 16: k_enc 346 us in the
+// last form, 248 in the second; 1024 of them 1.69 and 1.41 ms.)
 // Bound by its instructions and their latencies at 16 warps an SM: 700 warp
 // instructions a 32 rows at rank 3, 30.4 of 32 lanes active (1001 and 22.4 with
 // a per-lane loop over the corrections' candidates, a select chain each).
@@ -947,6 +950,7 @@ __device__ __forceinline__ float max_abs_nan(float m, float a, float b) {
   asm("{\n.reg .f32 x, y;\nabs.f32 x, %2;\nabs.f32 y, %3;\nmax.NaN.f32 x, x, y;\nmax.NaN.f32 %0, x, %1;\n}" : "=f"(r) : "f"(m), "f"(a), "f"(b));
   return r;
 }
+constexpr int kFullRows = 4096;
 template <int NP, bool POINT, int MC>
 __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSmem&, Cursor& cu, int64_t bi,
                                        const Geom& g, int r, const RowConst& rcst, const CorrConst& cc,
@@ -954,16 +958,17 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
                                        uint32_t* bits) {
   TileSmem& S = tile_here();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = MC ? NP : g.n, M = MC ? MC : (int)g.M, rc = MC ? 256 : a.rc;
+  constexpr bool kFull = MC == kFullRows, kLines = MC != 0;
+  const int n = kLines ? NP : g.n, M = kFull ? MC : (int)g.M, rc = kFull ? 256 : a.rc;
   const RowConst rq = rcst;
   const float eb_lo = cc.eb_lo_f;
-  const int Lq = MC ? MC : (int)align_up(g.L, 4);
+  const int Lq = kFull ? MC : (int)align_up(g.L, 4);
   const Chunks ch0 = chunks_of(a, g);
   // every chunk starts on a multiple of 32 rows, in every column
-  const bool words = MC || ((M & 31) == 0 && (chunk_rows(a, g, ch0, 0).count & 31) == 0 &&
+  const bool words = kLines || ((M & 31) == 0 && (chunk_rows(a, g, ch0, 0).count & 31) == 0 &&
                             (ch0.ncy == 1 || (g.sx * g.sy & 31) == 0));
   if (tid == 0) { S.kmax = 0; S.ncorr = 0; S.nesc = 0; S.nesc_slot = 0; }
-  uint32_t* const bw = MC ? S.bitsm : bits;
+  uint32_t* const bw = kFull ? S.bitsm : bits;
   if (POINT && !words)
     for (int i = tid; i < (n * M + 31) / 32; i += kTT) bw[i] = 0u;
   __syncthreads();
@@ -973,14 +978,14 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
   uint32_t qor_lane = 0, kmx = 0;
   int nc = 0, ne = 0, ovf = 0;
   float zmx = 0.0f, zmn = 0.0f;
-  const uint32_t msx = MC ? 0u : (g.sx > 1 ? 0xFFFFFFFFu / (uint32_t)g.sx + 1u : 0u);
+  const uint32_t msx = kLines ? 0u : (g.sx > 1 ? 0xFFFFFFFFu / (uint32_t)g.sx + 1u : 0u);
   const bool ok = stream_block(a, tm, S, cu, bi, g, kLayoutRow, [&](int c, const Chunks& ch, const float* tile) {
     ChunkRows cr;
     uint32_t mys = 0;
-    if (MC) {
-      cr.lbase = c * 256;
-      cr.count = 256;
-      cr.ys = 16;
+    if (kLines) {
+      cr.lbase = c * rc;
+      cr.count = rc;
+      cr.ys = 0;
     } else {
       cr = chunk_rows(a, g, ch, c);
       mys = cr.ys > 1 ? 0xFFFFFFFFu / (uint32_t)cr.ys + 1u : 0u;
@@ -988,9 +993,10 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
 #pragma unroll 1
     for (int rb = 0; rb < cr.count; rb += kTT) {        // same trip count in every lane
       const int i = rb + tid, l = cr.lbase + i;
-      const bool valid = MC ? true : i < cr.count;
+      if (kLines && !kFull && i - lane >= rc) continue;      // (a whole warp's: rc is a multiple of 32)
+      const bool valid = kLines ? true : i < cr.count;
       int rr = i;
-      if (!MC) {
+      if (!kLines) {
         // (x, y, z) in the chunk, and the row of its tile; invalid lanes take zeros and store nothing
         const int t = fdiv(i, msx), x = i - t * g.sx, zl = fdiv(t, mys), yl = t - zl * cr.ys;
         rr = valid ? (zl * a.yc + yl) * a.bxb + x : 0;
@@ -998,7 +1004,7 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
       float x[NP], d[NP], acc[NP];
 #pragma unroll
       for (int j = 0; j < NP; ++j) {
-        x[j] = (MC || (valid && j < n)) ? tile[j * rc + rr] : 0.0f;
+        x[j] = (kLines || (valid && j < n)) ? tile[j * rc + rr] : 0.0f;
         acc[j] = 0.0f;
       }
       const float a0 = x[0];
@@ -1111,7 +1117,7 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
       int8_t* kp = k8 + l;
 #pragma unroll
       for (int j = 0; j < NP; ++j) {
-        if (MC || j < n) {
+        if (kLines || j < n) {
           const unsigned bal = __ballot_sync(FULL, zi[j] != kMagicI);
           w = lane == j ? bal : w;
           if (valid) kp[j * M] = (int8_t)zi[j];
@@ -1132,7 +1138,7 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
         }
       }
       nc += __popc(w);
-      if (lane < n && (w != 0u || (words && (MC || i - lane < cr.count)))) {
+      if (lane < n && (w != 0u || (words && (kLines || i - lane < cr.count)))) {
         const uint32_t e0 = (uint32_t)(lane * M + (l - lane));
         if (words) {
           bw[e0 >> 5] = w;
@@ -1174,8 +1180,11 @@ template <bool POINT>
 __device__ __forceinline__ bool encode_rows(const TileArgs& a, const Maps& tm, TileSmem& S, Cursor& cu, int64_t bi,
                                             const Geom& g, int r, const RowConst& rcst, const CorrConst& cc, int32_t* qs,
                                             int8_t* k8, int32_t* k32, uint32_t* bits) {
-  if (g.n == NM && g.M == 4096 && a.rc == 256 && g.sx == a.bxb && bitmap_rows(a, g))
-    return pass_rows<NM, POINT, 4096>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32, bits);
+  if (g.n == NM && bitmap_rows(a, g)) {
+    if (g.M == kFullRows && a.rc == 256)
+      return pass_rows<NM, POINT, kFullRows>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32, bits);
+    return pass_rows<NM, POINT, 1>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32, bits);
+  }
   if (g.n <= 4) return pass_rows<4, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32, bits);
   if (g.n <= 8) return pass_rows<8, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32, bits);
   return pass_rows<NM, POINT, 0>(a, tm, S, cu, bi, g, r, rcst, cc, qs, k8, k32, bits);
