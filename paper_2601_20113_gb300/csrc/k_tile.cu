@@ -926,8 +926,10 @@ __device__ __forceinline__ ChunkRows chunk_rows(const TileArgs& a, const Geom& g
 // branch: y = R / 2eb, k = rint(y) by adding 1.5 x 2^23 (k is then the low
 // byte of that sum, ready to store), xt = k 2eb + xhat.  A row is settled when
 // every |y - k| is clear of 1/2, every |x - xt| of the bound, by more than
-// their roundings (|k| <= 59 bounds the first), else its elements go one by one
-// through corr_decide.  A ballot a column is one word of the bitmap, and each
+// their roundings (|k| <= 59 bounds the first), else its elements go through
+// corr_fast, and one by one through corr_slow where that leaves them open (256
+// blocks whose corrections mostly pass 59: k_enc 217 -> 152 us, with every
+// element of such a row one by one before).  A ballot a column is one word of the bitmap, and each
 // warp writes whole 32-byte sectors of k8.
 // MC = 4096: the 16 x 16 x 16 x 16 block (chunks of 256 rows, every row and
 // offset known); 1: NP time steps and chunks of whole lines (bitmap_rows), every
@@ -1094,21 +1096,35 @@ __device__ __noinline__ bool pass_rows(const TileArgs& a, const Maps& tm, TileSm
         zmx = fmaxf(zmx, hi);
         zmn = fminf(zmn, lo);
       } else {
-        // one by one, by the definition where FP32 leaves it open
+        // values past kFastK, or elements left open: each by itself, and by the
+        // definition where FP32 does not settle it
+        auto place = [&](int jj, int32_t k) -> int {
+          const bool big = k < -127 || k > 127;            // includes escapes
+          if (big && valid) k32[jj * M + l] = k;
+          if (k == kEscape) escm |= 1u << jj;
+          else kmx |= zigzag(k);
+          return kMagicI + (big ? -128 : k);
+        };
+        uint32_t open = 0;
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+          if (kLines || j < n) {
+            bool u;
+            const int32_t k = corr_fast(x[j], acc[j], S.ccc, &u);
+            if (u) open |= 1u << j;
+            else zi[j] = place(j, k);
+          }
+        }
 #pragma unroll 1
-        for (int jj = 0; jj < n; ++jj) {
+        for (; open; open &= open - 1) {
+          const int jj = __ffs(open) - 1;
           float aj = acc[0], xj = x[0];
 #pragma unroll
           for (int j = 1; j < NP; ++j) {
             aj = j == jj ? acc[j] : aj;
             xj = j == jj ? x[j] : xj;
           }
-          const int32_t k = corr_decide(xj, aj, S.ccc);
-          const bool big = k < -127 || k > 127;            // includes escapes
-          const int zb = kMagicI + (big ? -128 : k);
-          if (big && valid) k32[jj * M + l] = k;
-          if (k == kEscape) escm |= 1u << jj;
-          else kmx |= zigzag(k);
+          const int zb = place(jj, corr_slow(xj, aj, S.ccc));
 #pragma unroll
           for (int j = 0; j < NP; ++j) zi[j] = j == jj ? zb : zi[j];
         }
