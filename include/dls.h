@@ -283,7 +283,8 @@ int dls_compress_noalloc(const dls_params* p, const void* d_in, void* d_out, siz
  * d_out must hold nvars * nx*ny*nz*nt values of the stream's dtype; blocks
  * outside the stream's block range are left untouched.  Reads the header
  * with one synchronous copy and synchronizes `stream` at the end to report
- * DLS_ERR_CORRUPT. */
+ * DLS_ERR_CORRUPT, or DLS_ERR_TIMEOUT when a record's copy did not arrive within
+ * its bounded wait (blocks may then be missing from d_out). */
 int dls_decompress(const void* d_comp, size_t comp_bytes, void* d_out, size_t out_cap,
                    dls_stream_t stream);
 

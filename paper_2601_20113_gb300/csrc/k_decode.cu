@@ -6,9 +6,9 @@
 // chat = dtype(q) * dtype(delta).  Then xtilde = fma(dtype(k), dtype(2eb), acc)
 // where the correction k is nonzero, and escaped points take their raw value.
 // Every structural field of a record is validated against the geometry before
-// use.  k_decode_f32 takes the time-side blocks of float32 fields (persistent
-// CTAs, the next record copied while one is decoded), k_decode the others, a
-// CTA a block.
+// use.  k_decode_f32 takes float32 plans of time-side blocks of up to 16 time
+// steps and 65 536 points (persistent CTAs, a record brought in by one bulk
+// copy), k_decode the others, a CTA a block.
 #include "dls_internal.cuh"
 
 namespace dls {
@@ -409,10 +409,11 @@ __global__ void __launch_bounds__(kDecThreads, 3) k_decode(Plan P, const uint8_t
 
 // ---------------------------------------------------------------- float32, Gram order <= 16
 // Persistent decoder of float32 plans with Gram order <= 16 and blocks of at
-// most 65 536 points: CTAs take blocks from a counter and bring each record in
-// whole by one bulk copy.  Time-side blocks of rank <= 8 take the path below
-// when their corrections are dense (up to 8 bits) or listed or Rice coded (up
-// to 4 bits, |k| <= 8), any other block decode_block.
+// most 65 536 points whose whole blocks are time-side: CTAs take blocks from a
+// counter and bring each record in whole by one bulk copy, the next once the
+// block is done.  Time-side blocks of rank <= 8 take the path below when their
+// corrections are dense (up to 8 bits), listed (up to 4 bits, |k| <= 8) or Rice
+// coded (values up to 3 bits, |k| <= 4), any other block decode_block.
 //  - Listed and Rice-coded corrections go to a nibble a point in shared memory
 //    first (entries by all threads, a Rice chunk a thread), so that the rows
 //    add them as they write each output: no output is read back.
@@ -557,7 +558,7 @@ __device__ __forceinline__ void plane_put(uint32_t* plane, uint32_t e, int32_t k
 
 // One Rice chunk [e, c1) into the plane by one thread; false when the coded
 // words do not hold it.  A code is read from one 64-bit window at its first bit
-// (31 ones, a zero, kr <= 20 and wv <= 4 bits at most), so that the chain from
+// (31 ones, a zero, kr <= 20 and wv <= 3 bits at most), so that the chain from
 // one code to the next is a load, a count and a few shifts; longer runs of ones
 // take the loop.
 __device__ bool dec_rice_chunk(const uint32_t* __restrict__ rw, uint32_t words, uint32_t pos, int kr, int wv, int e,

@@ -2,9 +2,9 @@
 // variable, learned from random patches of the first snapshot, Sec. 2.3
 // Eq. 2-3; per patch of every snapshot the coefficients on it, Sec. 2.5
 // Eq. 5, the largest-magnitude prefix meeting the local tolerance of Sec. 2.4
-// Eq. 4 found by bisection, Eq. 6; reconstruction, Sec. 2.6).  FP64
-// throughout, so that every stored decision is the definition's; the device
-// steps are
+// Eq. 4 found by bisection, Eq. 6; reconstruction, Sec. 2.6).  Every stored
+// decision is the FP64 definition's (the patches take it in FP32 where that
+// provably settles it); the device steps are
 //   k_gb_sample   the sample matrix Q (S x M) from the first snapshot,
 //   k_gb_gram     G = Q^T Q, each entry a sequential sum over the samples,
 //   k_gb_jacobi   the eigenvectors of G by cyclic Jacobi in one cluster of

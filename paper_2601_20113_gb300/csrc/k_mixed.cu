@@ -975,9 +975,9 @@ __global__ void k_stage_quantize(const float* c, int64_t n, double delta, int32_
   }
 }
 
-// path 0: corr_exact (the row-loading kernel's decision); 1: the per-block
-// kernel's candidate filter, then corr_decide for candidates (its sparse
-// encode pass); 2: corr_decide for every element (its dense encode pass).
+// path 0: corr_exact (the row-loading kernel's decision); 2: corr_decide, the
+// decision of the row pass for a row that its packed test leaves open; 1: the
+// same behind the filter |fl(x - xhat)| >= eb, rounded down, which no kernel uses.
 __global__ void k_stage_correct(const float* x, const float* xh, int64_t n, double eb, int path, int32_t* k) {
   const CorrConst cc = make_corr_const(eb, 2.0 * eb, true);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {

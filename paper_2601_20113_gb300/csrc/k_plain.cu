@@ -3,7 +3,7 @@
 // Per block (Algorithm 1 step 3 of arXiv 2601.20113, with the readings of the
 // pointwise-bound form):
 //   Gram G = A^T A (cross-product SVD, Sec. 2.7.1)      FP64, sequential fma per entry
-//   Jacobi eigensolve, round-robin ordering (Sec. 2.3)   FP64, one warp, lane = row
+//   Jacobi eigensolve, round-robin ordering (Sec. 2.3)   FP64, the whole CTA, an entry a thread
 //   projection C = A Vst (Sec. 2.5, Eq. 5)               FP64 fma chain per coefficient
 //   quantization q = rint(C / delta)
 //   bisection for the smallest rank with E(r) <= eps_l^2 (Sec. 2.4 Eq. 4, Eq. 6)

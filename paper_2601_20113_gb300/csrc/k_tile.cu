@@ -86,8 +86,8 @@ struct RowConst {
   float inv_delta, delta_f;
 };
 
-// The staging ring is the last member, so that the kernels that stream no
-// block (k_eig) allocate only the part before it.
+// The state of the kernels that stream blocks, the staging ring last (the
+// eigensolve has a struct of its own, EigWarp).
 struct __align__(1024) TileSmem {
   unsigned long long full[kStages];
   float G32[NM * NM];
@@ -2202,8 +2202,8 @@ __device__ __forceinline__ int64_t grab_rr(const TileArgs& a, unsigned long long
 // prediction, follow each other at a warp's own pace, and a block takes a
 // third of the instructions that four warps in step took (each of them ran
 // every round's loop for one or two of its 192 items).  Every entry is formed
-// by the same operations as jacobi_cta's and orth_basis's, so the bases are
-// theirs bit for bit.  Bound by the latency of a round (rotation, loads,
+// by the same operations as in the CTA-wide solve it replaced, so the bases are
+// the same bit for bit.  Bound by the latency of a round (rotation, loads,
 // products, stores in turn): 16 384 blocks 0.68 -> 0.33 ms, 128 blocks 69 -> 50
 // us.
 struct EigWarp {
@@ -2355,8 +2355,8 @@ __device__ __forceinline__ void jacobi_warp32(EigWarp& W, int n, float floor_abs
   __syncwarp();
 }
 
-// orth_basis's step by one warp: V <- V + V R / 2, R = I - V^T V by error-free
-// transforms; with `first` (global, rows of modes) V = Vst V before.
+// Orthonormalisation by one warp, one step: V <- V + V R / 2, R = I - V^T V by
+// error-free transforms; with `first` (global, rows of modes) V = Vst V before.
 template <int NF>
 __device__ __forceinline__ void orth_warp(EigWarp& W, int n_, const float* first, int lane) {
   const int n = NF ? NF : n_;
@@ -2424,8 +2424,8 @@ __device__ __forceinline__ void orth_warp(EigWarp& W, int n_, const float* first
   __syncwarp();
 }
 
-// order_basis by one warp (the values are floats, and compare as floats), the
-// stored modes into A as rows of NM.
+// The modes in order by one warp (the values are floats, and compare as
+// floats), the stored modes into A as rows of NM.
 __device__ __forceinline__ void order_warp(EigWarp& W, int n, int lane) {
   float* out = W.A;
   if (lane < n) {
@@ -2514,7 +2514,7 @@ __global__ void __launch_bounds__(kTT, 10) k_eig(const __grid_constant__ TileArg
     if (RR) {
       flags = flags0 & ~kFbRR;
     } else {
-      // modes an FP32 Gram cannot resolve (rr_wanted), coefficients that might overflow
+      // modes an FP32 Gram cannot resolve, coefficients that might overflow
       const double noise = P.eb_type == DLS_EB_NRMSE ? el2 / n : (vi.eb * vi.eb) * (double)g.L;
       if (n > 1 && 4.0 * 5.9604644775390625e-8 * tr > 0.5 * noise) flags |= kFbRR;
       float rowmax = 0.0f;

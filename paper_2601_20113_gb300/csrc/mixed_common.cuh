@@ -99,16 +99,15 @@ __device__ __forceinline__ int32_t corr_fast(float x, float xh, const CorrConst&
   *unsure = !zero && !(clear && (in || out));
   return zero ? 0 : (out ? kEscape : (int32_t)r);
 }
-// The decision of one element the per-block kernel selected as a candidate
-// (|fl(x - xhat)| at or above eb, rounded down): the branch-free FP32 test,
-// and the FP64 definition where that test leaves the decision open.
+// One element's decision: the branch-free FP32 test, and the FP64 definition
+// where that test leaves the decision open.
 static __device__ __noinline__ int32_t corr_slow(float x, float xh, const CorrConst& cc);
 __device__ __forceinline__ int32_t corr_decide(float x, float xh, const CorrConst& cc) {
   bool u;
   const int32_t k = corr_fast(x, xh, cc, &u);
   return u ? corr_slow(x, xh, cc) : k;
 }
-// The candidate filter of the per-block kernel: elements with |fl(x - xhat)|
+// A filter in front of it (the stage test's path 1): elements with |fl(x - xhat)|
 // below eb (1 - 1e-6), rounded down, need no correction and no decision.
 __device__ __forceinline__ bool corr_candidate(float R, const CorrConst& cc) { return !(fabsf(R) < cc.eb_lo_f); }
 static __device__ __noinline__ int32_t corr_slow(float x, float xh, const CorrConst& cc) {
@@ -183,134 +182,6 @@ __device__ __forceinline__ int mlp_rank_warp(const MlpModel* M, const float* fea
   return r;
 }
 
-// ---------------------------------------------------------------- register Jacobi
-template <int NP>
-__device__ __forceinline__ float pick(const float (&a)[NP], int i) {
-  float v = a[0];
-#pragma unroll
-  for (int j = 1; j < NP; ++j) v = (i == j) ? a[j] : v;
-  return v;
-}
-
-// Parallel cyclic Jacobi of the symmetric matrix G (order n <= NP, row stride
-// ldg, shared) by one warp, in FP32.  Lanes [0, NP) hold the rows of A by
-// position, lanes [NP, 2 NP) the rows of the accumulated rotation V.  Each
-// round rotates the position pairs (2k, 2k+1) at once; then rows and columns
-// move one step along the round-robin circle (position 0 fixed), so NP - 1
-// rounds pair every two positions once.  The permutation of the columns is
-// fixed, so it is a renaming of registers.  Pairs with |a_pq| at or below the
-// threshold are skipped: tol_abs, or with `relative` max(1e-7 sqrt(a_pp a_qq),
-// 4 u max(a_pp, a_qq)) (reachable in FP32 on graded matrices), and never
-// below floor_abs.  Stops after a
-// sweep without rotation, or 30 sweeps.  Writes the eigenvectors as columns
-// of Vout (row stride ldv) and the eigenvalues to lam, both in the original
-// index order of the positions (any order: the caller sorts).
-template <int NP>
-__device__ void jacobi_reg(const float* G, int ldg, int n, bool relative, float tol_rel_trace, float* Vout, int ldv,
-                           double* lam, int lane, float floor_abs = 0.0f) {
-  constexpr unsigned FULL = 0xffffffffu;
-  constexpr int H = NP / 2;
-  const bool isA = lane < NP;
-  const bool isV = lane >= NP && lane < 2 * NP;
-  const int row = isA ? lane : (isV ? lane - NP : 0);
-  float a[NP];
-#pragma unroll
-  for (int j = 0; j < NP; ++j) {
-    float v = 0.0f;
-    if (isA) v = (row < n && j < n) ? G[row * ldg + j] : 0.0f;
-    else if (isV) v = (row == j) ? 1.0f : 0.0f;
-    a[j] = v;
-  }
-  int idx = row;
-  float tr = (isA && row < n) ? pick<NP>(a, row) : 0.0f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(FULL, tr, o);
-  const float tol = tol_rel_trace * tr;
-  const bool top = (row & 1) == 0;
-  // source lane of the row moved into this position after a round
-  int src = lane;
-  if (isA) {
-    if (row == 0) src = 0;
-    else if (row == 2) src = 1;
-    else if (!(row & 1)) src = row - 2;
-    else if (row == NP - 1) src = NP - 2;
-    else src = row + 2;
-  }
-  for (int sweep = 0; sweep < 30 && n > 1; ++sweep) {
-    unsigned any = 0;
-#pragma unroll 1
-    for (int round = 0; round < NP - 1; ++round) {
-      const float dself = pick<NP>(a, row);
-      const float off = pick<NP>(a, row ^ 1);
-      const float dpart = __shfl_xor_sync(FULL, dself, 1);
-      const float apq = __shfl_sync(FULL, off, lane & ~1);
-      const float app = top ? dself : dpart, aqq = top ? dpart : dself;
-      float c = 1.0f, s = 0.0f, t = 0.0f;
-      bool act = false;
-      if (isA) {
-        const float gpp = fabsf(app), gqq = fabsf(aqq);
-        float thr = relative ? fmaxf(1.0e-7f * sqrtf(gpp * gqq), 4.0f * 5.9604645e-8f * fmaxf(gpp, gqq)) : tol;
-        thr = fmaxf(thr, floor_abs);
-        if (fabsf(apq) > thr && apq != 0.0f) {
-          const float theta = (aqq - app) / (2.0f * apq);
-          if (fabsf(theta) > 1e18f) t = 0.5f / theta;
-          else t = (theta >= 0.0f ? 1.0f : -1.0f) / (fabsf(theta) + sqrtf(1.0f + theta * theta));
-          c = 1.0f / sqrtf(1.0f + t * t);
-          s = t * c;
-          act = true;
-        }
-      }
-      const unsigned actm = __ballot_sync(FULL, act);
-      any |= actm;
-      if (actm) {
-        // columns (A and V lanes): a[:, 2k], a[:, 2k+1] rotated by pair k
-#pragma unroll
-        for (int k = 0; k < H; ++k) {
-          const float ck = __shfl_sync(FULL, c, 2 * k), sk = __shfl_sync(FULL, s, 2 * k);
-          const float x = a[2 * k], y = a[2 * k + 1];
-          a[2 * k] = ck * x - sk * y;
-          a[2 * k + 1] = sk * x + ck * y;
-        }
-        // rows (A lanes): this row with its partner's
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-          const float b = __shfl_xor_sync(FULL, a[j], 1);
-          if (isA) a[j] = top ? (c * a[j] - s * b) : (s * b + c * a[j]);
-        }
-        // exact 2x2 result of the active pairs
-        if (act) {
-          const float nd = top ? app - t * apq : aqq + t * apq;
-#pragma unroll
-          for (int j = 0; j < NP; ++j) a[j] = (j == row) ? nd : ((j == (row ^ 1)) ? 0.0f : a[j]);
-        }
-      }
-      // one step along the circle: rows between lanes, columns between registers
-#pragma unroll
-      for (int j = 0; j < NP; ++j) a[j] = __shfl_sync(FULL, a[j], src);
-      idx = __shfl_sync(FULL, idx, src);
-      float na[NP];
-      na[0] = a[0];
-      na[2] = a[1];
-#pragma unroll
-      for (int k = 2; k < H; ++k) na[2 * k] = a[2 * k - 2];
-      na[NP - 1] = a[NP - 2];
-#pragma unroll
-      for (int k = 0; k + 1 < H; ++k) na[2 * k + 1] = a[2 * k + 3];
-#pragma unroll
-      for (int j = 0; j < NP; ++j) a[j] = na[j];
-    }
-    if (!any) break;
-  }
-  // eigenvalues (A lanes) and eigenvector columns (V lanes), by original index
-  if (isA && idx < n) lam[idx] = (double)pick<NP>(a, row);
-#pragma unroll
-  for (int P = 0; P < NP; ++P) {
-    const int ip = __shfl_sync(FULL, idx, P);
-    if (isV && row < n && ip < n) Vout[row * ldv + ip] = a[P];
-  }
-  __syncwarp();
-}
-
 // ---------------------------------------------------------------- CTA Jacobi
 // Scratch of the CTA Jacobi (shared).
 struct JacPairs {
@@ -335,9 +206,9 @@ __device__ __forceinline__ void circle_pair(int round, int i, int m, int& p, int
 // circle (m = n rounded up to even): rotation parameters by m/2 threads, then
 // in one step every 2x2 block of A (rows of pair k, columns of pair l) becomes
 // J_k^T A_kl J_l, with the exact 2x2 result on the rotated diagonal blocks, and
-// the columns of V rotate.  Thresholds as in
-// jacobi_reg (relative, with floor_abs).  Stops after a sweep without rotation
-// or 30 sweeps.  All threads call.
+// the columns of V rotate.  Pairs with |a_pq| at or below max(1e-7 sqrt(a_pp
+// a_qq), 4 u max(a_pp, a_qq), floor_abs) are skipped (reachable in FP32 on graded
+// matrices).  Stops after a sweep without rotation or 30 sweeps.  All threads call.
 template <int NT, int HF = 0>
 __device__ void jacobi_cta(float* A, float* V, double* lam, int n, float floor_abs, JacPairs& J) {
   const int tid = threadIdx.x;
