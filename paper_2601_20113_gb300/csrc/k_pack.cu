@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kPackThreads) k_pack(Plan P, const T* __restri
 
 // ---------------------------------------------------------------- bound resolution
 constexpr int kStatCtas = 512;
-constexpr int kRangeCtas = 152 * 8;      // k_range: all that are resident at 256 threads
+constexpr int kRangeCtasPerSm = 8;       // k_range: all that are resident at 256 threads
 
 // A thread's running minimum, maximum and non-finite flag.  float64 values are
 // compared as integers (order-preserving for finite values): FP64 comparisons
@@ -446,8 +446,12 @@ int launch_stats_resolve(const Plan& p, const void* d_in, const Work& w, double*
     } else {
       const int kv = p.dtype == DLS_F32 ? 4 : 2;
       const int vec = ((uintptr_t)d_in & 15) == 0 && p.K % kv == 0;
-      const int64_t want = cdiv(p.K, (vec ? kv * 4 : 8) * 256);
-      const dim3 grid((unsigned)(want < kRangeCtas ? want : kRangeCtas), p.nvars);
+      int dev = 0, sms = 0;
+      if (cudaGetDevice(&dev) != cudaSuccess ||
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return DLS_ERR_CUDA;
+      const int64_t want = cdiv(p.K, (vec ? kv * 4 : 8) * 256), most = (int64_t)sms * kRangeCtasPerSm;
+      const dim3 grid((unsigned)(want < most ? want : most), p.nvars);
       if (p.dtype == DLS_F32) k_range<float><<<grid, 256, 0, s>>>(p, (const float*)d_in, w, vec);
       else k_range<double><<<grid, 256, 0, s>>>(p, (const double*)d_in, w, vec);
     }
