@@ -417,9 +417,12 @@ int dls_stream_info_get(const void* d_comp, size_t comp_bytes, dls_stream_info* 
  * `arg` (an index into the call's block range).  Its bounded wait for that
  * chunk runs out after about a second of SM clock, the kernel drains the
  * copies it did issue and ends, and the call returns DLS_ERR_TIMEOUT.
- * DLS_FAULT_NONE (arg ignored) switches the hook off.  Not thread-safe with
- * respect to concurrent compressions; meant for tests only. */
-enum { DLS_FAULT_NONE = 0, DLS_FAULT_WITHHOLD_CHUNK = 1 };
+ * DLS_FAULT_WITHHOLD_RECORD: likewise in every later decompression of a float32
+ * plan of time-side blocks of up to 16 time steps and 65 536 points, the copy of
+ * the record of block `arg`.
+ * DLS_FAULT_NONE (arg ignored) switches both off.  Not thread-safe with
+ * respect to concurrent calls; meant for tests only. */
+enum { DLS_FAULT_NONE = 0, DLS_FAULT_WITHHOLD_CHUNK = 1, DLS_FAULT_WITHHOLD_RECORD = 2 };
 int dls_set_fault_hook(int32_t kind, int64_t arg);
 
 /* Static text for a DLS_* status ("unknown status" for other values). */

@@ -603,9 +603,10 @@ static void tune_store(const std::string& key, int variant, const float* ms) {
 
 namespace dls {
 namespace {
-std::atomic<int64_t> g_withheld{-1};
+std::atomic<int64_t> g_withheld{-1}, g_withheld_record{-1};
 }
 int64_t fault_withheld_block() { return g_withheld.load(); }
+int64_t fault_withheld_record() { return g_withheld_record.load(); }
 }  // namespace dls
 
 using namespace dls;
@@ -805,10 +806,11 @@ int dls_mlp_train(float* d_params, float* d_adam, const float* d_feat, const flo
 int dls_set_fault_hook(int32_t kind, int64_t arg) {
   if (kind == DLS_FAULT_NONE) {
     g_withheld.store(-1);
+    g_withheld_record.store(-1);
     return DLS_OK;
   }
-  if (kind != DLS_FAULT_WITHHOLD_CHUNK || arg < 0) return DLS_ERR_INVALID_ARG;
-  g_withheld.store(arg);
+  if ((kind != DLS_FAULT_WITHHOLD_CHUNK && kind != DLS_FAULT_WITHHOLD_RECORD) || arg < 0) return DLS_ERR_INVALID_ARG;
+  (kind == DLS_FAULT_WITHHOLD_CHUNK ? g_withheld : g_withheld_record).store(arg);
   return DLS_OK;
 }
 

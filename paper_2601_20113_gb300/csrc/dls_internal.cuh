@@ -302,6 +302,8 @@ int make_plan(const dls_params* p, Plan* out);
 // Test hook (dls_set_fault_hook): the block, in a call's block range, whose
 // first staged chunk the per-block kernel never copies; -1 for none.
 int64_t fault_withheld_block();
+// The same for the block whose record the float32 decoder never copies.
+int64_t fault_withheld_record();
 
 // Small stream-ordered device allocation (freed with cudaFreeAsync): dls_api.cu.
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);

@@ -677,7 +677,7 @@ __device__ void dec_parse(const Plan& P, const Geom& g, const uint8_t* rec, int 
 
 __global__ void __launch_bounds__(kDecThreads, 3) k_decode_f32(Plan P, const uint8_t* __restrict__ comp,
                                                                unsigned long long comp_bytes, float* __restrict__ out,
-                                                               Status* st, int vec) {
+                                                               Status* st, int vec, long long withhold) {
   extern __shared__ __align__(128) unsigned char dsm[];       // the record, then the plane
   constexpr int NT = kDecThreads;
   uint32_t* plane = reinterpret_cast<uint32_t*>(dsm + kRecCap + kRecPad);
@@ -701,6 +701,7 @@ __global__ void __launch_bounds__(kDecThreads, 3) k_decode_f32(Plan P, const uin
     const uint32_t nb = (uint32_t)(o1 - o0);
     bytes = (int)nb;
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&full)), "r"(nb) : "memory");
+    if (b == withhold) return;               // test hook: nothing arrives, the wait runs out
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                      smem_addr(dsm)),
                  "l"(comp + P.payload_pos + o0), "r"(nb), "r"(smem_addr(&full))
@@ -1137,7 +1138,8 @@ int launch_decode(const Plan& p, const void* d_comp, unsigned long long comp_byt
     // 16-byte stores need whole x lines and planes of 16-byte multiples
     const int vec = p.dims[0] % 4 == 0 && p.block[0] % 4 == 0 && ((uintptr_t)d_out & 15) == 0 ? 1 : 0;
     const int64_t most = (int64_t)sms * 3;
-    k_decode_f32<<<(unsigned)(p.nb < most ? p.nb : most), kDecThreads, smem, s>>>(p, c, comp_bytes, (float*)d_out, st, vec);
+    k_decode_f32<<<(unsigned)(p.nb < most ? p.nb : most), kDecThreads, smem, s>>>(p, c, comp_bytes, (float*)d_out, st, vec,
+                                                                                   fault_withheld_record());
     return cudaGetLastError() == cudaSuccess ? DLS_OK : DLS_ERR_CUDA;
   }
   const unsigned grid = (unsigned)p.nb;

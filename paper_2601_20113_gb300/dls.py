@@ -330,7 +330,7 @@ def stage_correct(x: torch.Tensor, xh: torch.Tensor, eb: float):
 
 
 CORR_PATH_EXACT, CORR_PATH_SPARSE, CORR_PATH_DENSE = 0, 1, 2
-FAULT_NONE, FAULT_WITHHOLD_CHUNK = 0, 1
+FAULT_NONE, FAULT_WITHHOLD_CHUNK, FAULT_WITHHOLD_RECORD = 0, 1, 2
 
 
 def stage_correct_path(x: torch.Tensor, xh: torch.Tensor, eb: float, path: int):
@@ -346,7 +346,8 @@ def stage_correct_path(x: torch.Tensor, xh: torch.Tensor, eb: float, path: int):
 
 def set_fault_hook(kind: int, arg: int = 0) -> int:
     """Test hook: FAULT_WITHHOLD_CHUNK withholds the first chunk copy of block
-    `arg` in later compressions (they return ERR_TIMEOUT); FAULT_NONE clears it."""
+    `arg` in later compressions, FAULT_WITHHOLD_RECORD the copy of its record in
+    later decompressions (they return ERR_TIMEOUT); FAULT_NONE clears both."""
     return lib().dls_set_fault_hook(int(kind), int(arg))
 
 
