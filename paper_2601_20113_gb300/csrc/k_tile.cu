@@ -937,11 +937,11 @@ __device__ __forceinline__ ChunkRows chunk_rows(const TileArgs& a, const Geom& g
 // arithmetic and, where a column's rows do not start on a word of the bitmap, by
 // OR-ing shifted words.  (64 blocks of 32 x 32 x 16 x 16: k_enc 346 us in the
 // last form, 248 in the second; 1024 of them 1.69 and 1.41 ms.)
-// Bound by its instructions and their latencies at 16 warps an SM: 700 warp
-// instructions a 32 rows at rank 3, 30.4 of 32 lanes active (1001 and 22.4 with
-// a per-lane loop over the corrections' candidates, a select chain each).
-// 128 blocks of 16^3 x 16: 100 -> 70 us; 16 384: 2.65 -> 2.51 ms; 4096 at rank
-// 7: 1.19 -> 0.96 ms.
+// Bound by its instructions and their latencies at 16 warps an SM: the kernel
+// issues 640 warp instructions a 32 rows at rank 3, 30.9 of 32 lanes active (1001
+// and 22.4 with a per-lane loop over the corrections' candidates, a select chain
+// each).  k_enc on 128 blocks of 16^3 x 16: 100 -> 62 us; 16 384: 2.65 -> 2.21 ms;
+// 4096 at rank 7: 1.19 -> 0.84 ms.
 constexpr float kMagicF = 12582912.0f;              // 1.5 x 2^23
 constexpr int kMagicI = 0x4B400000;                 // its bits
 constexpr int kFastK = 59;
