@@ -506,7 +506,7 @@ static int compress_host_pipelined(const Plan& P, const Layout& L, const void* h
     if (cudaStreamWaitEvent(s, ev[k], 0) != cudaSuccess ||
         cudaMemsetAsync(&w.status->pad[1], 0, sizeof(unsigned long long), s) != cudaSuccess)
       return done(DLS_ERR_CUDA);
-    if ((st = launch_tile_compress(P, d_in, mw, mode, kOccDefault, s, k * nbs, (k + 1) * nbs)) != DLS_OK) return done(st);
+    if ((st = launch_tile_compress(P, d_in, mw, mode, kOccDirect, s, k * nbs, (k + 1) * nbs)) != DLS_OK) return done(st);
   }
   uint8_t* out1 = P.corr_codec ? d_ws + L.rice_tmp : d_out;
   if ((st = launch_scan(P, w, bound, out1, s)) != DLS_OK) return done(st);
@@ -654,7 +654,7 @@ int dls_compress(const dls_params* p, const void* d_in, void* d_out, size_t out_
   cudaStream_t s = (cudaStream_t)stream;
   Work w = carve(L, d_workspace);
   if ((st = upload_basis(p, P, L, d_workspace, s)) != DLS_OK) return st;
-  if ((st = enqueue_compress(P, L, d_in, d_out, out_cap, d_workspace, kOccDefault, s)) != DLS_OK) return st;
+  if ((st = enqueue_compress(P, L, d_in, d_out, out_cap, d_workspace, kOccDirect, s)) != DLS_OK) return st;
   Status hs;
   CK(cudaMemcpyAsync(&hs, w.status, sizeof(Status), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));

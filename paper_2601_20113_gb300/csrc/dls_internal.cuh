@@ -314,16 +314,19 @@ int launch_mixed_compress(const Plan& p, const void* d_in, const MixedWork& w, i
 // Occupancy forms of the per-block kernels, one per shape class of a
 // compression's blocks (1: the form built for 2 CTAs per SM, with more
 // registers per thread; 2: the form built for 4).  `whole`: the blocks, of any
-// shape, that k_enc encodes at the predicted rank.  `rest`: what k_tile and
-// k_mixed take -- predictions k_enc rejects, blocks whose Gram side is space, every block in the search mode;
-// 0 there means the 2-CTA form behind k_enc (a short list) and the 4-CTA form
-// when k_tile takes every block.  Both forms run the same code, so the choice
-// changes the time and never a byte of the stream.
+// shape, that k_enc encodes at the predicted rank; 0 there means the 2-CTA form
+// for up to two blocks an SM whose records k_enc writes itself, and the 4-CTA form
+// for the others.  `rest`: what k_tile and k_mixed take --
+// predictions k_enc rejects, blocks whose Gram side is space, every block in the
+// search mode; 0 there means the 2-CTA form behind k_enc (a short list) and the
+// 4-CTA form when k_tile takes every block.  Both forms run the same code, so the
+// choice changes the time and never a byte of the stream.
 struct Occupancy {
   int whole;
   int rest;
 };
-constexpr Occupancy kOccDefault{2, 0};
+constexpr Occupancy kOccDefault{2, 0};   // a plan's, until it is tuned
+constexpr Occupancy kOccDirect{0, 0};    // a direct call's
 
 // Records ev on s: as an event node of the graph while s is being captured
 // (its time is then read after each replay), as a plain record otherwise (the

@@ -3280,11 +3280,18 @@ int launch_tile_compress(const Plan& p, const void* d_in, const MixedWork& w, in
   // 3. encode pass and deferred record at the predicted rank
   const size_t tsm = tile_smem_bytes(false);
   if (learned != kRankSearch) {
-    const int per = occ.whole == 1 ? ctas_per_sm_of(k_enc<2>, tsm, false) : ctas_per_sm_of(k_enc<4>, tsm, false);
+    // the 2-CTA form has no spills, which long passes over few large blocks show:
+    // 64 blocks of 32 x 32 x 16 x 16 511 -> 477 us a call, of 64 x 32 x 16 x 16 845 ->
+    // 770.  Few smaller blocks, whose records are deferred, are within 6% either
+    // way (256 of 16^3 x 16 273 -> 260, 128 of them with the NRMSE bound 260 -> 275)
+    // and stay with the other.
+    const bool few_large = nblk <= 2 * (int64_t)sms && w.nptmax > (int64_t)kBitsSmem * 32;
+    const int wf = occ.whole != 0 ? occ.whole : (few_large ? 1 : 2);
+    const int per = wf == 1 ? ctas_per_sm_of(k_enc<2>, tsm, false) : ctas_per_sm_of(k_enc<4>, tsm, false);
     cudaGetLastError();
     if (per < 1) return DLS_ERR_CUDA;
     const int grid = grid_of(per, w.ctas);
-    if (occ.whole == 1) k_enc<2><<<grid, kTT, tsm, s>>>(tmap, tmapg, a);
+    if (wf == 1) k_enc<2><<<grid, kTT, tsm, s>>>(tmap, tmapg, a);
     else k_enc<4><<<grid, kTT, tsm, s>>>(tmap, tmapg, a);
     a.from_list = 1;
   }
