@@ -923,8 +923,8 @@ __global__ void __launch_bounds__(256) k_verify_points(Plan P, const T* __restri
 // unevaluated float pairs (x^2 = p + fma(x, x, -p) exactly where neither is
 // subnormal, d^2 = s^2 + 2 s e to within e^2 <= 2^-48 s^2), two points an instruction (packed FP32), per
 // batch of 1024 points of a thread; each batch is added in FP64, and one whose
-// squares reach 2^117 (or with a NaN or an infinity), or stay below 2^-92
-// without being zeros, is summed again in FP64.
+// squares reach 2^117 (or with a NaN or an infinity) is summed again in FP64, as
+// are all of a thread's points where its sums stay below 2^-88 without being zeros.
 // Loads are float4 when the field allows (4 | K, 16-byte pointers).  Bound by the issue slots (about 20
 // instructions a point; scalar FP32 with a branch a point took twice that):
 // two fields of 1 GiB 0.74 -> 0.49 ms, the records' pass included.
@@ -974,26 +974,12 @@ __device__ __noinline__ void verify_point(VerRare& V, float x, float y) {
   if (ad > V.mx32) V.mx32 = ad;
   if (edge && d > V.eb) ++V.over;
 }
-// A batch's pairs are exact to 2^-46 of a sum of at least kPairsLeast (below
-// 2^-126 a square or its residual is off by up to 2^-150, three a point, 1024
-// points) and, below kPairsMost, every |x| and |s| is below 2^59, every |y| below
-// 2^60.  (Maxima kept with the points for these tests took a fifth more time; a
-// batch's sums out of line altogether 2%.)
-constexpr float kPairsLeast = 0x1p-92f, kPairsMost = 0x1p117f;
-// Whether the sums of a batch below kPairsLeast are sums of zeros: `err`,
-// differences have been seen; `val`, the values' squares are as small (they are
-// read again).
-__device__ __noinline__ bool verify_zeros(const float* __restrict__ a, int64_t i, int64_t n, int64_t stride, int width, bool err,
-                                          bool val) {
-  if (err) return false;
-  uint32_t any = 0u;
-  if (val) {
-#pragma unroll 8
-    for (int64_t k = 0; k < n; ++k)
-      for (int c = 0; c < width; ++c) any |= __float_as_uint(a[(i + k * stride) * width + c]) << 1;
-  }
-  return any == 0u;
-}
+// Below kPairsMost every |x| and |s| of a batch is below 2^59, every |y| below 2^60.
+constexpr float kPairsMost = 0x1p117f;
+// Below 2^-126 a square or its residual is off by up to 2^-150, three a point: the
+// pairs' sum over a thread's batches (sixteen of them for 5 G points) is exact to
+// 2^-46 of it from kPairsLeast on.
+constexpr double kPairsLeast = 0x1p-88;
 __device__ __noinline__ void verify_sums_fp64(const float* __restrict__ a, const float* __restrict__ b, int64_t i, int64_t n,
                                               int64_t stride, int width, double* se, double* sx) {
   for (int64_t k = 0; k < n; ++k, i += stride)
@@ -1003,8 +989,25 @@ __device__ __noinline__ void verify_sums_fp64(const float* __restrict__ a, const
       *sx = fma(x, x, *sx);
     }
 }
+// A thread's sums again in FP64 where one is below kPairsLeast, unless that is a
+// sum of zeros (`seen`: differences have been seen; the values are read again).
+// (Once a thread: the same test a batch took 1 to 2% of the kernel.)
+__device__ __noinline__ void verify_sums_small(const float* __restrict__ a, const float* __restrict__ b, int64_t i, int64_t n,
+                                               int64_t stride, int width, bool seen, double* se, double* sx) {
+  if (!(*se < kPairsLeast && seen)) {
+    uint32_t any = 0u;
+#pragma unroll 8
+    for (int64_t k = 0; k < n; ++k)
+      for (int c = 0; c < width; ++c) any |= __float_as_uint(a[(i + k * stride) * width + c]) << 1;
+    if (any == 0u) return;
+  }
+  *se = *sx = 0.0;
+  verify_sums_fp64(a, b, i, n, stride, width, se, sx);
+}
 
-__global__ void __launch_bounds__(256) k_verify_points_f32(Plan P, const float* __restrict__ a,
+// Four CTAs an SM: at 70 registers, three of them, 1 GiB took 644 us a call
+// instead of 537.
+__global__ void __launch_bounds__(256, 4) k_verify_points_f32(Plan P, const float* __restrict__ a,
                                                            const float* __restrict__ b, const uint8_t* comp,
                                                            unsigned long long comp_bytes, double* acc, int vec4) {
   const int v = blockIdx.y;
@@ -1035,10 +1038,8 @@ __global__ void __launch_bounds__(256) k_verify_points_f32(Plan P, const float* 
     return s;
   };
   auto flush = [&](const float* a0, const float* b0, int64_t i, int64_t n, int64_t stride, int width) {
-    const float he = fe.hi.x + fe.hi.y, hx = fx.hi.x + fx.hi.y;
-    const float h = he + hx + (fe.lo.x + fe.lo.y) + (fx.lo.x + fx.lo.y);       // a NaN when any of them is
-    if ((fabsf(h) < kPairsMost && fminf(he, hx) >= kPairsLeast) ||
-        (fabsf(h) < kPairsMost && verify_zeros(a0, i, n, stride, width, he < kPairsLeast && V.mx32 > 0.0f, hx < kPairsLeast))) {
+    const float h = (fe.hi.x + fe.hi.y) + (fx.hi.x + fx.hi.y) + (fe.lo.x + fe.lo.y) + (fx.lo.x + fx.lo.y);
+    if (fabsf(h) < kPairsMost) {
       se += ((double)fe.hi.x + (double)fe.lo.x) + ((double)fe.hi.y + (double)fe.lo.y);
       sx += ((double)fx.hi.x + (double)fx.lo.x) + ((double)fx.hi.y + (double)fx.lo.y);
     } else {
@@ -1102,6 +1103,11 @@ __global__ void __launch_bounds__(256) k_verify_points_f32(Plan P, const float* 
       const int64_t left = (P.K - i0 + stride - 1) / stride;
       flush(a + base, b + base, i0, n < left ? n : left, stride, 1);
     }
+  }
+  if ((se < kPairsLeast && V.mx32 > 0.0f) || sx < kPairsLeast) {
+    const int64_t i0 = blockIdx.x * 256ll + threadIdx.x, end = vec4 ? P.K / 4 : P.K;
+    if (i0 < end)
+      verify_sums_small(a + base, b + base, i0, (end - i0 + stride - 1) / stride, stride, vec4 ? 4 : 1, V.mx32 > 0.0f, &se, &sx);
   }
   double mx = V.mx;
   unsigned long long over = V.over;
